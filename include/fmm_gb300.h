@@ -58,12 +58,16 @@ extern "C" {
 #define FMM_ERR_UNSUPPORTED 10   /* combination not built (e.g. tensor-core M2L for this p) */
 
 /* ---- precision of the far-field contraction (and of everything else) ----- */
-#define FMM_PREC_FP32 0   /* FP32 everywhere (SIMT bilinear forms) */
+#define FMM_PREC_FP32 0   /* FP32 everywhere; bilinear forms of orders 3..6 on the tensor cores
+                             with every operand split into two halves of 11 significant
+                             bits (FP32's digits) and a compensated FP32 sum over the
+                             interaction list, of other orders in FP32 multiply-adds */
 #define FMM_PREC_FP64 1   /* FP64 everywhere; outputs are float64 */
-#define FMM_PREC_TF32X3 2 /* bilinear forms on tcgen05 tensor cores, 3-pass split TF32,
-                             FP32 accumulate; rest FP32 */
-#define FMM_PREC_TF32X1 3 /* tensor cores, one TF32 pass (10-bit mantissa operands),
-                             FP32 accumulate; rest FP32 */
+#define FMM_PREC_TF32X3 2 /* bilinear forms on tcgen05 tensor cores, 3-pass split with TF32's
+                             significand (two halves of 11 bits, scaled per cell so that
+                             the half type's range does not enter), FP32 accumulate; rest FP32 */
+#define FMM_PREC_TF32X1 3 /* tensor cores, one pass with TF32's significand (operands
+                             rounded to 11 bits, scaled per cell), FP32 accumulate; rest FP32 */
 #define FMM_PREC_BF16X3 4 /* tensor cores, 3-pass split BF16 (hi = bf16(x),
                              lo = bf16(x - hi)), FP32 accumulate; rest FP32 */
 

@@ -1,5 +1,6 @@
 // C ABI of the GB300 replacement-FMM library: plans, tables, workspace layout
 // and the order of the stages of one evaluation.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -47,11 +48,11 @@ struct fmm_plan_s {
     void *Kbar;   // [comp][343][p^3] row means of the unit-cell kernels
     void *Klat;   // [comp][p^3][p^3] lattice kernel minus its row mean (periodic form)
     void *Klbar;  // [comp][p^3] row means of the lattice kernel
-    void *Ktc_hi, *Ktc_lo;  // [comp][343][a][b] split of Kt, padded (tensor-core plans)
+    void *Ktc;              // [comp][343][a] rows of the split of Kt (tensor-core contraction)
     void *Kbar_tc;          // [comp][343][a] row means, padded to 32
-    alignas(64) unsigned char khi_map[4][128], klo_map[4][128];  // their TMA tensor maps
+    alignas(64) unsigned char k_map[4][128];  // TMA tensor map of each component's rows
     bool tc;                // bilinear forms of every level on tensor cores
-    int tc_mode;            // FMM_TC_*: split TF32 x3, TF32 x1, split BF16 x3
+    int tc_mode;            // FMM_TC_*
     int inject;             // FMM_INJECT_* for the next evaluation (test hook)
     bool shared;            // tables belong to another plan (batched systems)
     void *sf_tab;           // App. A.2 forms of every level (shift-free plans), FP64
@@ -75,9 +76,6 @@ struct fmm_plan_s {
 
 static std::atomic<long long> g_plan_counter{0};
 
-namespace fmm {
-int plan_device(const fmm_plan_s *P) { return P->device; }
-}  // namespace fmm
 
 // Tag of an evaluation in the workspace header: plan id and n.
 static long long eval_tag(const fmm_plan_s *P, int64_t n) { return (P->id << 32) | (long long)n; }
@@ -139,18 +137,6 @@ void far_image_grad(double rx, double ry, double rz, double g[3]) {
             }
 }
 
-// The function of the bilinear forms between unit cells at separation
-// (dx, dy, dz) = a - (o + b): comp 0 is 1/r (§2.1.7), comps 1..3 the x, y, z
-// components of r/|r|^3 (§4.1: the forces directly from the kernel).
-// power 2: 1/r^2 and the components of its force kernel 2 r/r^4 (§4.1 names
-// 1/r^2 as another function the replacement applies to).
-double kernel_value(int comp, int power, double dx, double dy, double dz) {
-    const double r2 = dx * dx + dy * dy + dz * dz, r = std::sqrt(r2);
-    const double d = comp == 1 ? dx : comp == 2 ? dy : dz;
-    if (power == 2) return comp == 0 ? 1.0 / r2 : 2.0 * d / (r2 * r2);
-    return comp == 0 ? 1.0 / r : d / (r2 * r);
-}
-
 double far_image_sum(double rx, double ry, double rz) {
     const double alpha = 2.0;
     const int RM = 7, HM = 7;
@@ -206,111 +192,28 @@ int upload(void **dst, const std::vector<real> &v) {
     return FMM_OK;
 }
 
-// bfloat16 = the upper 16 bits of an IEEE binary32; round to nearest, ties to
-// even, on the discarded 16 bits (finite inputs only)
-static uint16_t bf16_rne(float f) {
-    uint32_t u;
-    memcpy(&u, &f, 4);
-    u += 0x7FFFu + ((u >> 16) & 1u);
-    return (uint16_t)(u >> 16);
-}
-static float bf16_value(uint16_t h) {
-    uint32_t u = (uint32_t)h << 16;
-    float f;
-    memcpy(&f, &u, 4);
-    return f;
-}
-
 // Unit-cell kernels of eq. (bilinear), K_o[a,b] = 1/|a - (o + b)| for the 316
 // offsets 2 <= |o|_inf <= 3 (and, with FMM_FORCE_KERNEL, the three force
 // kernels), split into row mean and remainder (FP64, then rounded to the
-// plan's type).
+// plan's type), computed on the device; the lattice tables on the host.
 template <typename real>
 int upload_tables(fmm_plan_t P) {
-    const int p = P->p, p3 = p * p * p, nc = P->ncomp, pw = P->geom.power;
+    const int p = P->p, p3 = p * p * p, nc = P->ncomp;
     const double gs = P->opts.grid_scale;
-    const size_t nk = (size_t)343 * p3 * p3;
-    std::vector<real> KtT(nc * nk, (real)0), Kbar((size_t)nc * 343 * p3, (real)0);
-    std::vector<double> row(p3);
-    for (int c = 0; c < nc; c++)
-        for (int oz = -3; oz <= 3; oz++)
-            for (int oy = -3; oy <= 3; oy++)
-                for (int ox = -3; ox <= 3; ox++) {
-                    if (std::abs(ox) <= 1 && std::abs(oy) <= 1 && std::abs(oz) <= 1) continue;
-                    size_t oi = (size_t)c * 343 + (size_t)(((oz + 3) * 7 + (oy + 3)) * 7 + (ox + 3));
-                    for (int a = 0; a < p3; a++) {
-                        double ax = node(p, gs, a % p), ay = node(p, gs, (a / p) % p), az = node(p, gs, a / (p * p));
-                        double mean = 0.0;
-                        for (int b = 0; b < p3; b++) {
-                            row[b] = kernel_value(c, pw, ax - (ox + node(p, gs, b % p)),
-                                                  ay - (oy + node(p, gs, (b / p) % p)),
-                                                  az - (oz + node(p, gs, b / (p * p))));
-                            mean += row[b];
-                        }
-                        mean /= p3;
-                        Kbar[oi * p3 + a] = (real)mean;
-                        for (int b = 0; b < p3; b++) KtT[(oi * p3 + b) * p3 + a] = (real)(row[b] - mean);
-                    }
-                }
-    int rc = upload(&P->Kunit, KtT);
-    if (!rc) rc = upload(&P->Kbar, Kbar);
+    const size_t no = (size_t)343 * nc;
+    if (cudaMalloc(&P->Kunit, no * p3 * p3 * sizeof(real)) != cudaSuccess ||
+        cudaMalloc(&P->Kbar, no * p3 * sizeof(real)) != cudaSuccess)
+        return FMM_ERR_OOM;
+    const size_t rows = (size_t)343 * tc_padded(p3);
+    if (P->tc && (cudaMalloc(&P->Ktc, nc * rows * tc_row_bytes(p3)) != cudaSuccess ||
+                  cudaMalloc(&P->Kbar_tc, nc * rows * sizeof(float)) != cudaSuccess))
+        return FMM_ERR_OOM;
+    int rc = build_tables<real>(p, gs, P->geom.power, nc, P->tc_mode, (real *)P->Kunit, (real *)P->Kbar, P->Ktc,
+                                (float *)P->Kbar_tc);
+    for (int c = 0; P->tc && c < nc && !rc; c++)
+        rc = tc_encode_kernel_map(P->k_map[c], (const char *)P->Ktc + c * rows * tc_row_bytes(p3), p3, P->tc_mode);
     if (rc) return rc;
-    if (P->tc) {
-        // Kt_o[a][b] = K_o[a][b] - Kbar_o[a] (natural layout, rows zero-padded to
-        // p3s = p^3 rounded up to 32, columns to pk), split from the FP64 value:
-        // TF32: hi = Kt with its 13 low mantissa bits cleared (rounded to nearest
-        // for the 1-pass form), lo = Kt - hi;
-        // BF16: hi = bf16(Kt), lo = bf16(Kt - hi), rounded to nearest even
-        const int p3s = tc_padded(p3), pk = tc_padded_k(p3, P->tc_mode);
-        const bool bf16 = P->tc_mode == FMM_TC_BF16X3;
-        const size_t nt = (size_t)343 * p3s * pk;
-        std::vector<float> Khi(nc * nt, 0.0f), Klo(nc * nt, 0.0f), Kb((size_t)nc * 343 * p3s, 0.0f);
-        std::vector<uint16_t> Khi16(bf16 ? nc * nt : 0, 0), Klo16(bf16 ? nc * nt : 0, 0);
-        for (int oc = 0; oc < 343 * nc; oc++) {
-            const int c = oc / 343, oi = oc % 343;
-            int ox = oi % 7 - 3, oy = (oi / 7) % 7 - 3, oz = oi / 49 - 3;
-            if (std::abs(ox) <= 1 && std::abs(oy) <= 1 && std::abs(oz) <= 1) continue;
-            for (int a = 0; a < p3; a++) {
-                double ax = node(p, gs, a % p), ay = node(p, gs, (a / p) % p), az = node(p, gs, a / (p * p));
-                double mean = 0.0;
-                for (int b = 0; b < p3; b++) {
-                    row[b] = kernel_value(c, pw, ax - (ox + node(p, gs, b % p)), ay - (oy + node(p, gs, (b / p) % p)),
-                                          az - (oz + node(p, gs, b / (p * p))));
-                    mean += row[b];
-                }
-                mean /= p3;
-                Kb[(size_t)oc * p3s + a] = (float)mean;
-                for (int b = 0; b < p3; b++) {
-                    double k = row[b] - mean;
-                    size_t idx = ((size_t)oc * p3s + a) * pk + b;
-                    if (bf16) {
-                        uint16_t h = bf16_rne((float)k);
-                        Khi16[idx] = h;
-                        Klo16[idx] = bf16_rne((float)(k - (double)bf16_value(h)));
-                        continue;
-                    }
-                    float f = (float)k;
-                    uint32_t u;
-                    memcpy(&u, &f, 4);
-                    if (P->tc_mode == FMM_TC_TF32X1) u += 0x1000u;  // nearest (no lo pass)
-                    u &= 0xFFFFE000u;
-                    float hi;
-                    memcpy(&hi, &u, 4);
-                    Khi[idx] = hi;
-                    Klo[idx] = (float)(k - (double)hi);
-                }
-            }
-        }
-        rc = bf16 ? upload(&P->Ktc_hi, Khi16) : upload(&P->Ktc_hi, Khi);
-        if (!rc) rc = bf16 ? upload(&P->Ktc_lo, Klo16) : upload(&P->Ktc_lo, Klo);
-        if (!rc) rc = upload(&P->Kbar_tc, Kb);
-        const size_t cb = nt * (bf16 ? 2 : 4);  // bytes of one component's table
-        for (int c = 0; c < nc && !rc; c++) {
-            rc = tc_encode_kernel_map(P->khi_map[c], (const char *)P->Ktc_hi + c * cb, p3s, pk, P->tc_mode);
-            if (!rc) rc = tc_encode_kernel_map(P->klo_map[c], (const char *)P->Ktc_lo + c * cb, p3s, pk, P->tc_mode);
-        }
-        if (rc) return rc;
-    }
+    std::vector<double> row(p3);
     if (P->periodic) {
         // psi depends on a - b only: (2p-1)^3 distinct arguments; the force
         // components take -grad psi
@@ -416,25 +319,6 @@ WsLayout make_layout(const fmm_plan_t P, int64_t n) {
     }
     W.q_level[P->depth + 1] = qc;
     W.qlev = take((size_t)qc * rs);
-    size_t part = 0;
-    for (int l = 2; l <= P->depth; l++) {
-        int G = m2l_groups(l, p3);
-        if (G > 1) {
-            size_t need = (size_t)G * ((size_t)1 << (3 * l)) * p3;
-            if (need > part) part = need;
-        }
-    }
-    if (P->periodic) {
-        int G = m2l_groups(1, p3);
-        size_t need = (size_t)G * 8 * p3;
-        if (G > 1 && need > part) part = need;
-    }
-    W.m2l_part = take(part * rs);
-    const size_t p3s = (size_t)tc_padded(p3);
-    const size_t pht = (size_t)tc_level_first(P->depth + 1);  // cells of the operand layout
-    W.phihi = take(P->tc ? pht * p3s * rs : 0);
-    W.philo = take(P->tc ? pht * p3s * rs : 0);
-    W.occ = take(P->tc ? (size_t)occ_ints(P->depth, P->periodic ? 1 : 2) * 4 : 0);
     W.delta = take(cont && !P->fp64 ? (size_t)W.cap * 4 : 0);
     W.slist = take(cont && !P->fp64 ? (size_t)(n + 2) * 4 : 0);
     W.pord = take((size_t)(W.ncell + 16) * 4);
@@ -442,6 +326,26 @@ WsLayout make_layout(const fmm_plan_t P, int64_t n) {
     W.scan_blocks = (int)(mx / 2048 + 2);
     W.scan_tmp = take((size_t)(W.scan_blocks + 1) * 4);
     W.epart = take((size_t)((n + 255) / 256 + 1) * 16);  // (hi, lo) per block, real <= 8 B
+    // Last, the contraction's scratch: the SIMT form's partials, or the
+    // tensor-core form's operand copy, cell charges, partials and cell lists.  An
+    // FP32 plan takes either (total_simt: a caller's workspace of at least that
+    // size evaluates with the SIMT form)
+    const bool simt = !P->tc || P->opts.precision == FMM_PREC_FP32;
+    size_t part = 0;
+    for (int l = P->periodic ? 1 : 2; l <= P->depth && simt; l++) {
+        const int G = m2l_groups(l, p3);
+        if (G > 1) part = std::max(part, (size_t)G * ((size_t)1 << (3 * l)) * p3);
+    }
+    const size_t o0 = o;
+    W.m2l_part = take(part * rs);
+    W.total_simt = o;
+    o = o0;
+    W.op = take(P->tc ? (size_t)qc * tc_row_bytes(p3) : 0);
+    W.qsc = take(P->tc ? (size_t)qc * sizeof(float2) : 0);
+    W.tc_part = take(P->tc ? (size_t)tc_part_values(P->depth, p3) * 4 : 0);
+    W.occ = take(P->tc ? (size_t)occ_ints(P->depth, P->periodic ? 1 : 2) * 4 : 0);
+    if (!simt) W.total_simt = o;
+    o = std::max(o, W.total_simt);
     W.total = o;
     return W;
 }
@@ -473,8 +377,9 @@ Ptrs<real> make_ptrs(const WsLayout &W, void *ws) {
     P.loc = (real *)(b + W.loc);
     P.qlev = (real *)(b + W.qlev);
     P.m2l_part = (real *)(b + W.m2l_part);
-    P.phihi = (real *)(b + W.phihi);
-    P.philo = (real *)(b + W.philo);
+    P.op = b + W.op;
+    P.qsc = (float2 *)(b + W.qsc);
+    P.tc_part = (float *)(b + W.tc_part);
     P.occ = (int *)(b + W.occ);
     P.delta = (float *)(b + W.delta);
     P.slist = (int *)(b + W.slist);
@@ -518,7 +423,7 @@ int check_ws(const fmm_plan_t P, int64_t n, const void *ws, size_t bytes) {
     if (!ws) return FMM_ERR_WORKSPACE;
     if (((uintptr_t)ws) & 255) return FMM_ERR_WORKSPACE;
     WsLayout W = make_layout(P, n);
-    if (bytes < W.total) return FMM_ERR_WORKSPACE;
+    if (bytes < W.total_simt) return FMM_ERR_WORKSPACE;
     return FMM_OK;
 }
 
@@ -534,9 +439,10 @@ int finish(fmm_plan_t P, const WsHeader *hdr, cudaStream_t st, bool sync) {
 
 template <typename real>
 int eval_impl(fmm_plan_t P, int64_t n, const float *pos, const float *q, real *potential,
-              double *energy, real *forces, void *ws, const Streams &S, Tracer &tr) {
+              double *energy, real *forces, void *ws, size_t ws_bytes, const Streams &S, Tracer &tr) {
     cudaStream_t st = S.main;
     WsLayout W = make_layout(P, n);
+    const bool tc = P->tc && ws_bytes >= W.total;
     Ptrs<real> ptr = make_ptrs<real>(W, ws);
     const Coef<real> &C = *reinterpret_cast<const Coef<real> *>(P->fp64 ? (const void *)&P->cd
                                                                         : (const void *)&P->cf);
@@ -577,11 +483,10 @@ int eval_impl(fmm_plan_t P, int64_t n, const float *pos, const float *q, real *p
         T.Kbar[c] = (const real *)P->Kbar + (size_t)c * 343 * p3;
         T.Klt[c] = P->Klat ? (const real *)P->Klat + (size_t)c * p3 * p3 : nullptr;
         T.Klbar[c] = P->Klbar ? (const real *)P->Klbar + (size_t)c * p3 : nullptr;
-        T.tc_khi_map[c] = P->khi_map[c];
-        T.tc_klo_map[c] = P->klo_map[c];
+        T.tc_k_map[c] = P->k_map[c];
         T.tc_kbar[c] = P->Kbar_tc ? (const float *)P->Kbar_tc + (size_t)c * 343 * tc_padded(p3) : nullptr;
     }
-    T.tc_lmin = P->tc ? (P->periodic ? 1 : 2) : 0;  // every level on the tensor cores
+    T.tc_lmin = tc ? (P->periodic ? 1 : 2) : 0;  // every level on the tensor cores
     T.tc_mode = P->tc_mode;
     T.tc_inject = P->inject;
     P->inject = FMM_INJECT_NONE;  // one evaluation only
@@ -641,6 +546,15 @@ Tracer make_tracer(fmm_plan_t P, cudaStream_t st) {
 }
 
 }  // namespace
+
+namespace fmm {
+int plan_device(const fmm_plan_s *P) { return P->device; }
+int plan_min_workspace(const fmm_plan_s *P, int64_t n, size_t *bytes) {
+    if (n < 0 || n > P->max_n) return FMM_ERR_ARG;
+    *bytes = make_layout(const_cast<fmm_plan_t>(P), n).total_simt;
+    return FMM_OK;
+}
+}  // namespace fmm
 
 // ---------------------------------------------------------------------------
 // C ABI
@@ -728,10 +642,12 @@ int fmm_plan_create(fmm_plan_t *out, const double box[4], int depth, int p, int 
     memcpy(P->box, box, sizeof(double) * 4);
     P->max_n = max_n;
     P->fp64 = o.precision == FMM_PREC_FP64;
-    P->tc = tc_prec;
+    // plain FP32 plans of the orders the MMA tiles cover take the split form too
+    P->tc = tc_prec || (o.precision == FMM_PREC_FP32 && p >= 3 && p <= 6);
     P->tc_mode = o.precision == FMM_PREC_BF16X3   ? FMM_TC_BF16X3
-                 : o.precision == FMM_PREC_TF32X1 ? FMM_TC_TF32X1
-                                                  : FMM_TC_TF32X3;
+                 : o.precision == FMM_PREC_TF32X1 ? FMM_TC_F16X1
+                 : o.precision == FMM_PREC_FP32   ? FMM_TC_F16X3C
+                                                  : FMM_TC_F16X3;
     cudaGetDevice(&P->device);
     fill_coef<float>(p, o.grid_scale, P->cf);
     fill_coef<double>(p, o.grid_scale, P->cd);
@@ -805,8 +721,7 @@ void fmm_plan_destroy(fmm_plan_t P) {
     if (P->Kbar) cudaFree(P->Kbar);
     if (P->Klat) cudaFree(P->Klat);
     if (P->Klbar) cudaFree(P->Klbar);
-    if (P->Ktc_hi) cudaFree(P->Ktc_hi);
-    if (P->Ktc_lo) cudaFree(P->Ktc_lo);
+    if (P->Ktc) cudaFree(P->Ktc);
     if (P->Kbar_tc) cudaFree(P->Kbar_tc);
     if (P->sf_tab) cudaFree(P->sf_tab);
     if (P->sf_H) cudaFree(P->sf_H);
@@ -838,9 +753,11 @@ int fmm_eval(fmm_plan_t P, int64_t n, const float *pos, const float *q, void *po
                  P->s_far, P->e_far};
     if (P->serial) S.near = S.coarse = st, S.far = nullptr;  // isolated stage times
     if (P->fp64)
-        rc = eval_impl<double>(P, n, pos, q, (double *)potential, energy, (double *)forces, workspace, S, tr);
+        rc = eval_impl<double>(P, n, pos, q, (double *)potential, energy, (double *)forces, workspace,
+                               workspace_bytes, S, tr);
     else
-        rc = eval_impl<float>(P, n, pos, q, (float *)potential, energy, (float *)forces, workspace, S, tr);
+        rc = eval_impl<float>(P, n, pos, q, (float *)potential, energy, (float *)forces, workspace,
+                              workspace_bytes, S, tr);
     P->last = tr;
     if (rc) return rc;
     P->last_ws = workspace;
@@ -937,7 +854,7 @@ static int dump_bytes(fmm_plan_t P, int what, int n_eff, size_t *bytes) {
 int fmm_debug_inject(fmm_plan_t P, int what) {
     if (!P) return FMM_ERR_ARG;
     if (what != FMM_INJECT_NONE && what != FMM_INJECT_TC_STALL) return FMM_ERR_ARG;
-    if (what == FMM_INJECT_TC_STALL && !P->tc) return FMM_ERR_UNSUPPORTED;
+    if (what == FMM_INJECT_TC_STALL && (!P->tc || P->opts.precision == FMM_PREC_FP32)) return FMM_ERR_UNSUPPORTED;
     P->inject = what;
     return FMM_OK;
 }
@@ -1186,7 +1103,8 @@ int record_merged(fmm_batch_t B, const std::vector<int64_t> &n, const std::vecto
         char *pot = potential ? (char *)potential + o * 4 : nullptr;
         char *frc = forces ? (char *)forces + 3 * o * 4 : nullptr;
         double *en = energy ? energy + i : nullptr;
-        int rc = eval_impl<float>(P, n[i], pos + 3 * o, q + o, (float *)pot, en, (float *)frc, ws + wofs[i], S, tr);
+        int rc = eval_impl<float>(P, n[i], pos + 3 * o, q + o, (float *)pot, en, (float *)frc, ws + wofs[i],
+                                  SIZE_MAX, S, tr);
         if (rc) return rc;
     }
     if (tc_lmin) {
@@ -1196,27 +1114,26 @@ int record_merged(fmm_batch_t B, const std::vector<int64_t> &n, const std::vecto
         std::vector<TcXSys> xs((size_t)M0->ncomp * ns);
         std::vector<int> dep(ns);
         WsLayout W0;
+        size_t ws_bytes = 0;
         for (int i = 0; i < ns; i++) {
             WsLayout W = make_layout(B->sys[i], n[i]);
             Ptrs<float> Pi = make_ptrs<float>(W, ws + wofs[i]);
             if (i == 0) W0 = W;
+            ws_bytes = std::max(ws_bytes, wofs[i] + W.total);
             dep[i] = n[i] > 0 ? B->sys[i]->depth : 0;
             for (int c = 0; c < M0->ncomp; c++)
-                xs[(size_t)c * ns + i] = TcXSys{reinterpret_cast<const char *>(Pi.phihi),
-                                               reinterpret_cast<const char *>(Pi.philo), Pi.qlev,
-                                               Pi.loc + c * W.loc_comp};
+                xs[(size_t)c * ns + i] = TcXSys{(int)((Pi.op - ws) / 128), Pi.qsc, Pi.loc + c * W.loc_comp, Pi.tc_part};
         }
-        const void *khi[4], *klo[4];
+        const void *km[4];
         const float *kb[4];
         for (int c = 0; c < M0->ncomp; c++) {
-            khi[c] = M0->khi_map[c];
-            klo[c] = M0->klo_map[c];
+            km[c] = M0->k_map[c];
             kb[c] = (const float *)M0->Kbar_tc + (size_t)c * 343 * tc_padded(M0->geom.p3);
         }
         int *status = &reinterpret_cast<WsHeader *>(ws + wofs[0])->status;
         std::vector<LaunchRec> xr;
-        int rc = tc_cross_records(xs, dep, M0->ncomp, tc_lmin, x_lmax, M0->geom.p3, M0->tc_mode, M0->geom.power, khi,
-                                  klo, kb, W0, status, &B->d_x, &B->x_bytes, xr);
+        int rc = tc_cross_records(xs, dep, M0->ncomp, tc_lmin, x_lmax, M0->geom.p3, M0->tc_mode, M0->geom.power, km,
+                                  kb, W0, ws, ws_bytes, status, &B->d_x, &B->x_bytes, xr);
         if (rc) return rc;
         bool placed = false;
         for (int i = 0; i < ns && !placed; i++)
@@ -1406,10 +1323,10 @@ int capture_batch(fmm_batch_t B, int lanes, const std::vector<int64_t> &n,
         double *en = energy ? energy + i : nullptr;
         if (P->fp64)
             rc = eval_impl<double>(P, n[i], pos + 3 * o, q + o, (double *)pot, en, (double *)frc,
-                                   ws + wofs[i], S, tr);
+                                   ws + wofs[i], SIZE_MAX, S, tr);
         else
             rc = eval_impl<float>(P, n[i], pos + 3 * o, q + o, (float *)pot, en, (float *)frc,
-                                  ws + wofs[i], S, tr);
+                                  ws + wofs[i], SIZE_MAX, S, tr);
         total += tr.launches;
     }
     for (int k = 0; k < lanes; k++) {

@@ -74,14 +74,17 @@ struct WsLayout {
     size_t react;  // [13][cap] near-field reactions per forward direction (mutual near field)
     size_t phi, loc;                      // all levels (loc: ncomp blocks of loc_comp)
     size_t qlev;                          // total charge of every cell, padded Phi layout
-    size_t phihi, philo;                  // TF32 split of Phi (tensor-core plans)
     size_t m2l_part;                      // per-offset-group partials of the SIMT contraction
+    size_t op;                            // 16-bit split of Phi (tensor-core contraction)
+    size_t qsc;                           // per cell: charge and the split's factor
+    size_t tc_part;                       // partials of the levels whose offsets are split over blocks
     size_t occ;                           // occupied-cell lists of the contraction (tensor-core plans)
     size_t delta;                         // per emitted charge of a split particle: phi(s_k) - phi(r)
     size_t slist;                         // the split particles (count, then indices)
     size_t pord;                          // near-field launch order: class counts, fill, cells
     size_t scan_tmp, epart;
     size_t total;
+    size_t total_simt;                    // FP32 plans: enough without the tensor-core contraction
     int64_t cap;                          // charge capacity
     int64_t ncell;                        // 8^depth
     int64_t phi_level[FMM_MAXDEPTH + 2];  // element offset of each level in Phi
@@ -123,23 +126,24 @@ __host__ __device__ inline int64_t phi_level_cells(int l) {
     int64_t P = ((int64_t)1 << (l - 1)) + 2;
     return 8 * P * P * P;
 }
-// Tensor-core operand layout of the grid charges (split hi / lo copies): the
-// padded parity-major layout with at least 10 cells per axis, so that every
-// 8 x 4 x 4 box the contraction loads (starting at coarse coordinate 0..2)
-// lies inside the grid; cells beyond the padded layout hold zeros.
-__host__ __device__ inline int64_t tc_level_extent(int l) {
-    int64_t P = ((int64_t)1 << (l - 1)) + 2;
-    return P < 10 ? 10 : P;
+// Blocks that share the 189 offsets of a tile of the tensor-core contraction:
+// the levels with fewer than 8 coarse cells per axis have one tile a parity
+// (a depth-3 system: 16 tiles for 152 SMs), a depth-4 system 32 tiles at its
+// finest level.  The 9 runs of 21 offsets of levels 1 to 3 are also the runs in
+// which a batch's cross-system tiles add, so the choice depends on the level
+// and the depth alone.
+#define TC_PARTS_SMALL 9
+__host__ __device__ inline int tc_parts(int l, int depth) {
+    return l <= 3 ? TC_PARTS_SMALL : (l == 4 && depth == 4 ? 3 : 1);
 }
-__host__ __device__ inline int64_t tc_level_cells(int l) {
-    if (l == 0) return 1;
-    int64_t Pt = tc_level_extent(l);
-    return 8 * Pt * Pt * Pt;
+// partial functionals of a level with tc_parts > 1: its first value and the
+// distance between parts
+inline void tc_part_place(int l, int p3, long long *off, long long *stride) {
+    *off = l <= 3 ? (((1LL << (3 * l)) - 1) / 7) * p3 : (long long)TC_PARTS_SMALL * 585 * p3;
+    *stride = l <= 3 ? 585LL * p3 : 4096LL * p3;
 }
-__host__ __device__ inline int64_t tc_level_first(int l) {  // cells before level l
-    int64_t c = 0;
-    for (int k = 0; k < l; k++) c += tc_level_cells(k);
-    return c;
+inline long long tc_part_values(int depth, int p3) {
+    return (long long)TC_PARTS_SMALL * 585 * p3 + (depth == 4 ? 3LL * 4096 * p3 : 0);
 }
 
 // cell of level l >= 1 in the unpadded L layout
@@ -165,7 +169,7 @@ __device__ __forceinline__ bool cell_occupied(const int *leaf_start, int depth, 
 // of OCC_BLOCK coarse cells.  Ints in the workspace region `occ`:
 //   [0, nblk)                     occupied cells per block (then their prefix)
 //   [nblk, nblk + nseg)           occupied cells per segment
-//   [.., + nseg + 1)              prefix of the segments' 128-row tiles
+//   [.., + nseg + 1)              prefix of the segments' blocks, deepest level first
 //   [occ_list_offset, ..)         the lists, segment s from the number of
 //                                 cells of the segments before it
 #define OCC_BLOCK 1024
@@ -185,19 +189,14 @@ __host__ __device__ inline int64_t occ_list_offset(int depth, int lmin) {
     return ((int64_t)occ_nblk(depth, lmin) + 2 * occ_nseg(depth, lmin) + 1 + 63) / 64 * 64;
 }
 // A segment takes box tiles (each offset's A operand one TMA box of 8 x 4 x 4
-// coarse cells, empty cells included) when it has fewer than 8 coarse cells
-// per axis or when the share of its cells that hold charges reaches the
-// threshold of the tile width N (p^3 padded): the gathered tiles of narrow
-// shapes keep fewer copies in flight per MMA, so they pay off only on sparser
-// segments (measured: N = 224 gathers as fast as boxes, N = 128 at ~2/3 of
-// their rate, N <= 64 at ~2/5).
+// coarse cells, empty cells included) where nearly all of its cells hold
+// charges: a box costs one copy instead of 32 gathers a chunk, and multiplies
+// the empty cells.
 __host__ __device__ inline bool occ_box_segment(int H, int64_t count, int N) {
-    const int pct = N >= 224 ? 95 : (N >= 128 ? 70 : 40);
-    return H < 8 || count * 100 >= (int64_t)pct * H * H * H;
+    const int pct = N >= 128 ? 95 : 90;
+    return H >= 8 && count * 100 >= (int64_t)pct * H * H * H;
 }
 __host__ __device__ inline int occ_seg_tiles(int H, int64_t count, int N) {
-    if (count == 0) return 0;
-    if (H < 8) return 1;
     return occ_box_segment(H, count, N) ? (int)((int64_t)H * H * H / 128) : (int)((count + 127) / 128);
 }
 __host__ __device__ inline int64_t occ_ints(int depth, int lmin) {
@@ -262,7 +261,9 @@ struct Ptrs {
     typename Vec4<real>::T *react;
     real *phi, *loc;
     real *qlev;
-    real *phihi, *philo;
+    char *op;
+    float2 *qsc;
+    float *tc_part;
     real *m2l_part;
     int *occ;
     float *delta;  // single-precision plans of the continuous form (adjoint split forces)
@@ -287,11 +288,11 @@ struct DevTables {
     const real *Kbar[4];   // [343][a]
     const real *Klt[4];    // [a][b] lattice kernel minus its row mean (periodic form)
     const real *Klbar[4];  // [a]
-    // tensor-core contraction (TF32X3 / TF32X1 / BF16X3 plans): levels >= tc_lmin, 0 = none
+    // tensor-core contraction: levels >= tc_lmin, 0 = none
     int tc_lmin;
     int tc_mode;                          // FMM_TC_*
     int tc_inject;                        // FMM_INJECT_* test hook for this evaluation
-    const void *tc_khi_map[4], *tc_klo_map[4];  // CUtensorMap of the split unit-cell kernels
+    const void *tc_k_map[4];              // CUtensorMap of the split unit-cell kernels
     const float *tc_kbar[4];                    // [343][p3 padded to 32] row means
     // App. A.2 forms (shift-free plans), FP64: right parts K_o shift_{S->C},
     // [level pairs from sf_base[l]][n][m]; per-axis shift_{S->C} of every level
@@ -347,34 +348,46 @@ int launch_downward(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, con
                     const DevTables<real> &T, const Streams &S, Tracer &tr);
 
 // tensor-core contraction (m2l_tc.cu)
-#define FMM_TC_TF32X3 0  // 3-pass split TF32
-#define FMM_TC_TF32X1 1  // 1-pass TF32
+#define FMM_TC_F16X3 0   // 3-pass split: two 11-bit halves per operand (TF32's significand), scaled
+#define FMM_TC_F16X1 1   // 1 pass: operands rounded to 11 bits, scaled
 #define FMM_TC_BF16X3 2  // 3-pass split BF16
-// loc: the functionals to write (one kernel component); spow: forms scale by
-// 2^(l spow) at level l; split: also split the grid charges into the operand
-// copies (once per evaluation)
+#define FMM_TC_F16X3C 3  // as F16X3, the sum over the offsets compensated (plain FP32 plans)
+// factor of the scaled kernel tables: |K| <= 2 at unit cells (separation >= 1),
+// so the scaled entries stay below the half type's maximum and their lo parts
+// above its subnormal floor
+#define TC_KSCALE 16384.0f
 // one system of a batched evaluation's cross-system contraction tiles
 struct TcXSys {
-    const char *op_hi, *op_lo;  // operand copies (hi, lo) of its grid charges
-    const float *qlev;          // its cell charges
+    int op_chunk;               // its operand copy: first 128-byte chunk from the batch's workspace
+    const float2 *qsc;          // its cells' charges and operand factors
     float *loc;                 // its functionals (one kernel component)
+    float *part;                // scratch of the functionals' layout
 };
 // The launches (one per kernel component) of the cross-system tiles of a
 // batch: levels lmin..lmax of every system, all cells.  sys: ncomp x nsys
-// (component-major); depth: per system.  The lists and the per-system table
-// are written to the device buffer *dx (grown as needed, owned by the caller).
+// (component-major); depth: per system; ws: the batch's workspace.  The lists
+// and the per-system table are written to the device buffer *dx (grown as
+// needed, owned by the caller).
 int tc_cross_records(const std::vector<TcXSys> &sys, const std::vector<int> &depth, int ncomp, int lmin,
-                     int lmax, int p3, int mode, int spow0, const void *const *k_hi_maps,
-                     const void *const *k_lo_maps, const float *const *kbars, const WsLayout &W, int *status,
-                     void **dx, size_t *dx_bytes, std::vector<LaunchRec> &out);
-int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const void *k_hi_map,
-                  const void *k_lo_map, const float *kbar, int lmin, int mode, int inject,
-                  float *loc, int spow, bool split, int comp, cudaStream_t st, Tracer &tr);
-// map of a [343][p3s][pk] kernel table: fp32 (pk = p3s) or bf16 (pk = tc_padded_k)
-int tc_encode_kernel_map(void *map, const void *base, int p3s, int pk, int mode);
-int tc_padded(int p3);            // p^3 rounded up to 32 (MMA N, fp32 K)
-int tc_padded_k(int p3, int mode);  // K extent of a cell vector: 32 (fp32) or 64 (bf16) multiple
+                     int lmax, int p3, int mode, int spow0, const void *const *k_maps, const float *const *kbars,
+                     const WsLayout &W, const char *ws, size_t ws_bytes, int *status, void **dx, size_t *dx_bytes,
+                     std::vector<LaunchRec> &out);
+// loc: the functionals to write (one kernel component); spow: forms scale by
+// 2^(l spow) at level l; split: also split the grid charges into the operand
+// copy and list the occupied cells (once per evaluation)
+int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const void *k_map, const float *kbar,
+                  int lmin, int mode, int inject, float *loc, int spow, bool split, int comp, cudaStream_t st,
+                  Tracer &tr);
+// map of a [343][tc_padded] table of kernel rows
+int tc_encode_kernel_map(void *map, const void *base, int p3, int mode);
+int tc_padded(int p3);     // p^3 rounded up to 32 (MMA N)
+int tc_row_bytes(int p3);  // bytes of a cell vector's (or kernel row's) split copy
 size_t tc_map_bytes();
+// the kernel tables of a plan, computed on the device (rows, kbar_tc: tensor
+// cores, or null); asynchronous on the default stream
+template <typename real>
+int build_tables(int p, double grid_scale, int power, int ncomp, int mode, real *KtT, real *Kbar, void *rows,
+                 float *kbar_tc);
 
 // bilinear forms without shifts (shift_free.cu, App. A.2; double-precision plans)
 // table bytes and the first pair of every level (base[0..depth+1])
@@ -394,6 +407,8 @@ void launch_sf_downward(const Geom &g, const Ptrs<double> &P, const WsLayout &W,
 // the device a plan was created on (fmm_api.cu); the scratch array of
 // fmm_eval_static on the current device, looked up once per device (fmm_static.cu)
 int plan_device(const fmm_plan_s *plan);
+// the smallest workspace an evaluation of n particles accepts
+int plan_min_workspace(const fmm_plan_s *plan, int64_t n, size_t *bytes);
 int static_workspace_address(void **out);
 
 // near field + far-field evaluation at the charges (kernels_p2p.cu)

@@ -48,7 +48,7 @@ extern "C" int fmm_eval_static(fmm_plan_t plan, int64_t n, const float *pos, con
     if (cudaGetDevice(&dev) != cudaSuccess) return FMM_ERR_CUDA;
     if (dev != fmm::plan_device(plan)) return FMM_ERR_ARG;
     size_t need = 0;
-    int rc = fmm_workspace_size(plan, n, &need);
+    int rc = fmm::plan_min_workspace(plan, n, &need);
     if (rc != FMM_OK) return rc;
     if (need > (size_t)FMM_STATIC_WORKSPACE_BYTES) return FMM_ERR_WORKSPACE;
     void *ws = nullptr;

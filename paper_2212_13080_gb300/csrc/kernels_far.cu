@@ -823,7 +823,7 @@ int launch_downward(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, con
     if constexpr (std::is_same<real, float>::value) {
         if (T.tc_lmin > 0 && depth >= T.tc_lmin) {
             for (int c = 0; c < T.ncomp; c++) {
-                int rc = launch_m2l_tc(g, P, W, T.tc_khi_map[c], T.tc_klo_map[c], T.tc_kbar[c], T.tc_lmin,
+                int rc = launch_m2l_tc(g, P, W, T.tc_k_map[c], T.tc_kbar[c], T.tc_lmin,
                                        T.tc_mode, T.tc_inject, P.loc + c * W.loc_comp,
                                        c == 0 ? g.power : g.power + 1,
                                        c == 0, c, st, tr);

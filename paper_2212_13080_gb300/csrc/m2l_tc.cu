@@ -1,46 +1,51 @@
 // Bilinear forms of the interaction lists (§2.2 step 3, eq. bilinear) on the
-// 5th-generation tensor cores (tcgen05): 3-pass split TF32, 1-pass TF32 or
-// 3-pass split BF16, FP32 accumulation.
+// 5th-generation tensor cores (tcgen05): 16-bit operands in 3-pass split form
+// (half or bfloat16) or one pass, FP32 accumulation.
 //
 // Only cells that hold charges get a functional (step 4 reads no other).
 // After the sort, a list of the occupied cells of every (level, target
 // parity) segment is built in coarse Morton order; one CTA takes 128 of them
 // (the MMA's M).  For each of the 189 interaction-list offsets o, the tile's
 // contribution L[cell][a] += sum_b Phi[cell + o][b] K_o[a][b] is a
-// 128 x N x K GEMM (N = K = p^3 padded to a multiple of 32): A holds the
-// tile's 128 source vectors, B the unit-cell kernel K_o, both in 128-byte K
-// chunks staged in shared memory with the 128-byte swizzle; one thread issues
-// the MMAs into tensor memory.  A arrives in one of two ways:
-//   - box tiles (a segment whose cells mostly hold charges, or a level with
-//     fewer than 8 coarse cells per axis): the tile is 128 consecutive
-//     Morton cells, an 8 x 4 x 4 box of the padded parity-major layout, and
-//     each stage's A is one TMA box copy; one thread issues A and B into the
-//     same ring stage;
-//   - gathered tiles (sparser segments): producer warps copy each row's 128
-//     bytes with 16-byte cp.async straight into the swizzled layout, complete
-//     and fence them for the async proxy before arriving on the stage; B has
-//     its own TMA producer and ring (tile widths N >= 128), so several stages
-//     of gathered copies stay in flight.
+// 128 x N x K GEMM (N = p^3 padded to a multiple of 32, K to a multiple of
+// 16): A holds the tile's 128 source vectors, B the unit-cell kernel K_o, both
+// in 128-byte K chunks staged in shared memory with the 128-byte swizzle; one
+// thread issues the MMAs into tensor memory.  A arrives in one of two ways:
+//   - box tiles (a segment whose cells nearly all hold charges): the tile is
+//     128 consecutive Morton cells, an 8 x 4 x 4 box of the padded parity-major
+//     layout, one box copy a chunk;
+//   - gathered tiles: producer warps copy the rows with 16-byte cp.async
+//     straight into the swizzled layout (16-byte piece j of row r lands at piece
+//     j ^ (r mod 8)), complete and fence them for the async proxy before they
+//     arrive on the stage.  A lane's rows and places are fixed for the whole
+//     tile, so a row costs one address and two copies a stage; TMA row gathers
+//     (four rows each) took 65 cycles each: 79.7 against 51 ms on 8M clustered
+//     charges at p = 6.
 //
-// Accuracy.  Split precision: x = hi + lo with hi = x with its 13 low mantissa
-// bits cleared (exact in TF32); D = Ahi Bhi + Ahi Blo + Alo Bhi.  The BF16
-// form splits x = hi + lo with hi = bf16(x), lo = bf16(x - hi) (both round to
-// nearest, 8 + 8 significant bits) and takes the same three products with
-// kind::f16 MMAs (K = 16 per MMA, 64 per 128-byte chunk).  The 1-pass TF32
-// form takes Ahi Bhi alone.  The kernel
-// is split as K_o = Kbar_o[a] + Kt_o[a,b] (row mean): the tensor cores contract
-// Kt_o, the CUDA cores add Kbar_o[a] Q (Q = the source cell's total charge).
-// Each offset accumulates into a fresh TMEM region (two regions, alternating):
-// the epilogue warps read it out and add the 189 partials in FP32 registers,
-// so no FP32 accumulator in TMEM sees more than 3 * K / 8 MMAs (the tensor
-// cores' accumulation is not round-to-nearest; over 1512 MMAs it drifted by
-// ~1e-4).  A row's functional depends on its own A rows only, so it is the
-// same, bit for bit, whichever tile form computes it.  For N > 64 the
-// epilogue splits the columns over two warp groups.
+// Operands.  x = hi + lo in two halves of 11 significant bits each, after an
+// exact power-of-two scaling (per cell for the grid charges, one factor for
+// the kernels) that puts the largest value near the type's maximum: as many
+// significant bits as FP32 keeps of a value, so plain FP32 plans (p = 3..6)
+// and the split-TF32 precision use this form at twice TF32's MMA rate and half
+// its bytes.  D = Alo Bhi + Ahi Blo + Ahi Bhi.  The BF16 form has 8 + 8 bits
+// and no scaling; the 1-pass form takes Ahi Bhi alone (11 bits, TF32's).
+//
+// Accuracy.  The kernel is split as K_o = Kbar_o[a] + Kt_o[a,b] (row mean): the
+// tensor cores contract Kt_o, the CUDA cores add Kbar_o[a] Q (Q = the source
+// cell's total charge).  Each offset accumulates into a fresh TMEM region (two
+// regions, alternating), small products first; the epilogue warps read it out
+// and add the offsets in FP32 registers with Kahan compensation.  Without the
+// compensation these 189 additions were the largest error of the form
+// (potentials of a depth-4 system at p = 6: 3.2e-7 against 2.8e-7 for FP32
+// multiply-adds; draining an accumulator more often than once an offset made
+// it worse).  A row's functional depends on its own A rows only, so it is the
+// same, bit for bit, whichever tile form computes it.
 #include <algorithm>
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
+#include <type_traits>
 
 #include "fmm_internal.cuh"
 #include "launch.cuh"
@@ -49,7 +54,7 @@
 namespace fmm {
 
 #define TC_M 128
-#define TC_ABYTES (TC_M * 128)      // 128 rows x 32 fp32 (one K chunk)
+#define TC_ABYTES (TC_M * 128)      // 128 rows of one 128-byte K chunk
 #define TC_WAIT_CYCLES (4LL << 30)  // about 2 s of SM clock
 #define TC_NOFF 189
 
@@ -63,47 +68,72 @@ __device__ __forceinline__ void tc_wait_failed(int *status, int site, int level,
     }
 }
 
-// The i-th offset of the interaction list of parity (bx, by, bz), in the
-// order shared by the producer and the epilogue.
+// The interaction list of every target parity (bx, by, bz): offsets o in
+// [-2 - b, 3 - b]^3 without [-1, 1]^3, ordered by the source's parity, then by
+// its coarse shift (x fastest): a tile's source cells of one parity (a few
+// hundred cells, used by up to 27 offsets) are read in one stretch of the
+// walk, so that the tiles in flight find them in L2 (152 tiles x 0.3 MB at
+// p = 6, against 2.6 MB a tile for all eight parities: measured 54.6 ms with
+// the offsets in x, y, z order).  An entry packs the index of
+// the offset in the 7^3 kernel tables, the source's parity block and its
+// coarse shift (-1..1 per axis).
+struct OffTable {
+    uint32_t v[8][TC_NOFF];
+};
+constexpr OffTable make_off_table() {
+    OffTable t{};
+    for (int par = 0; par < 8; par++) {
+        const int b[3] = {par & 1, (par >> 1) & 1, par >> 2};
+        int n = 0;
+        for (int sp = 0; sp < 8; sp++)
+            for (int dz = -1; dz <= 1; dz++)
+                for (int dy = -1; dy <= 1; dy++)
+                    for (int dx = -1; dx <= 1; dx++) {
+                        const int ox = 2 * dx + (sp & 1) - b[0], oy = 2 * dy + ((sp >> 1) & 1) - b[1],
+                                  oz = 2 * dz + (sp >> 2) - b[2];
+                        if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1) continue;
+                        t.v[par][n++] = (uint32_t)(((oz + 3) * 7 + (oy + 3)) * 7 + (ox + 3)) | (uint32_t)sp << 9 |
+                                        (uint32_t)(dx + 1) << 12 | (uint32_t)(dy + 1) << 14 | (uint32_t)(dz + 1) << 16;
+                    }
+    }
+    return t;
+}
+__constant__ const OffTable c_off = make_off_table();
 struct Off {
     int oi, spar, dX, dY, dZ;
 };
-__device__ __forceinline__ bool next_offset(int bx, int by, int bz, int &ox, int &oy, int &oz) {
-    do {
-        if (++ox > 3 - bx) {
-            ox = -2 - bx;
-            if (++oy > 3 - by) {
-                oy = -2 - by;
-                if (++oz > 3 - bz) return false;
-            }
-        }
-    } while (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1);
-    return true;
-}
-__device__ __forceinline__ Off make_off(int bx, int by, int bz, int ox, int oy, int oz) {
-    Off f;
-    const int sx = bx + ox, sy = by + oy, sz = bz + oz;
-    f.spar = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
-    f.dX = sx >> 1;
-    f.dY = sy >> 1;
-    f.dZ = sz >> 1;
-    f.oi = ((oz + 3) * 7 + (oy + 3)) * 7 + (ox + 3);
-    return f;
+__device__ __forceinline__ Off list_offset(int par, int i) {
+    const uint32_t v = c_off.v[par][i];
+    return Off{(int)(v & 511u), (int)((v >> 9) & 7u), (int)((v >> 12) & 3u) - 1, (int)((v >> 14) & 3u) - 1,
+               (int)(v >> 16) - 1};
 }
 
-#define TC_TF32X3 0
-#define TC_TF32X1 1
-#define TC_BF16X3 2
+#define TC_F16X3 FMM_TC_F16X3
+#define TC_F16X1 FMM_TC_F16X1
+#define TC_BF16X3 FMM_TC_BF16X3
+#define TC_F16X3C FMM_TC_F16X3C
 
+// A cell vector (and a kernel row) in 128-byte chunks of 64 values: the hi and
+// the lo part of every 64 values in two chunks; a tail of at most 32 values has
+// both in one (hi in its first half).  p = 3: 27 values, one chunk; 4: 64, two;
+// 5: 125, four; 6: 216, seven.
 template <int N, int MODE>
 struct TcShape {
     static constexpr int CH = N > 64 ? 2 : 1;           // epilogue column groups
     static constexpr int EPI = 4 * CH;                  // epilogue warps
-    static constexpr int KE = MODE == TC_BF16X3 ? 64 : 32;  // K elements per 128-byte chunk
-    static constexpr int KC = (N + KE - 1) / KE;        // 128-byte K chunks
-    static constexpr bool LO = MODE != TC_TF32X1;       // lo parts loaded and used
-    static constexpr int BBYTES = N * 128;              // one K chunk of K_o (hi or lo)
-    static constexpr int TCOLS = 2 * N <= 64 ? 64 : (2 * N <= 128 ? 128 : (2 * N <= 256 ? 256 : 512));
+    static constexpr int KS = N == 32 ? 2 : (N == 64 ? 4 : (N == 128 ? 8 : 14));  // MMA steps of 16 values
+    static constexpr int FC = KS / 4;                   // stages of whole chunks (hi, lo)
+    static constexpr int KC = (KS + 3) / 4;             // stages per offset
+    static constexpr int RC = 2 * FC + (KC - FC);       // chunks per cell vector
+    static constexpr bool LO = MODE != TC_F16X1;        // lo parts loaded and used
+    static constexpr bool SCALED = MODE != TC_BF16X3;   // operands scaled by powers of two
+    static constexpr bool COMP = MODE == TC_F16X3C;     // compensated sum over the offsets
+    static constexpr int BBYTES = N * 128;              // one chunk of K_o
+    // cross-system tiles keep the totals of their runs of offsets in TMEM, the
+    // widest tile (two accumulators fill it) in the output
+    static constexpr bool RMW = N == 224;
+    static constexpr int TUSED = RMW ? 2 * N : 4 * N;
+    static constexpr int TCOLS = TUSED <= 128 ? 128 : (TUSED <= 256 ? 256 : 512);
     static constexpr int COLS = N / CH;                 // columns per epilogue thread
 };
 
@@ -208,7 +238,7 @@ __global__ void k_occ_offsets(const __grid_constant__ KOccOffsets k) {
 }
 
 // the list entries: coarse coordinates X | Y << 10 | Z << 20 of each occupied
-// cell; block 0 also writes the prefix of the segments' 128-row tiles
+// cell; block 0 also writes the prefix of the segments' blocks
 struct KOccScatter {
     static constexpr int BS = OCC_BLOCK / 4, MINB = 0;  // bounds on the block size only
     OccParams op;
@@ -229,9 +259,10 @@ struct KOccScatter {
             const int *cnt = op.occ + op.nblk;
             int *tiles = op.occ + op.nblk + op.nseg;
             int t = 0;
-            for (int k = 0; k < op.nseg; k++) {
+            for (int k = 0; k < op.nseg; k++) {  // the deepest level's blocks first
+                const int sg = op.nseg - 1 - k, lv = op.lmin + sg / 8;
                 tiles[k] = t;
-                t += occ_seg_tiles(1 << (op.lmin + k / 8 - 1), cnt[k], op.N);
+                t += occ_seg_tiles(1 << (lv - 1), cnt[sg], op.N) * tc_parts(lv, op.depth);
             }
             tiles[op.nseg] = t;
         }
@@ -242,30 +273,29 @@ __global__ void __launch_bounds__(KOccScatter::BS) k_occ_scatter(const __grid_co
 }
 
 // ---------------------------------------------------------------------------
-// The contraction over the occupied-cell lists.  One CTA per 128-row tile of a
-// segment (level l, target parity b): row r is the tile's r-th occupied
-// target cell; for offset o its A operand row is the source cell (target + o)
-// of the operand layout, gathered by the producer warps with 16-byte
-// cp.async copies straight into the 128-byte-swizzled K-major layout (the
-// 16-byte chunk j of row r lands at chunk j ^ (r mod 8)); the kernel matrix B
-// arrives by TMA as in the box form.  The copies of a stage are complete and
-// fenced for the async proxy before the producers arrive on its barrier.  MMA
-// issue, TMEM regions and the epilogue are those of the box form, so every
-// row is summed over the offsets in the same order: a row's functional is the
-// box form's bit for bit.
+// The contraction over the occupied-cell lists.  A block takes one 128-row tile
+// of a segment (level l, target parity b): row r is the tile's r-th occupied
+// target cell, and its A operand row for offset o is the source cell (target +
+// o), copied by TMA gathers (or one box copy); the kernel matrix B arrives by
+// TMA box copies.  Levels with few tiles split the 189 offsets over tc_parts
+// blocks, whose partial functionals k_tc_reduce adds.
+//
+// What bounds it (GB300): p = 4 the shared-memory traffic of operands and MMAs
+// (N = 64 reads 6 KB per 32-cycle MMA), p = 5 and 6 the tensor pipe and the
+// operand copies.
 // ---------------------------------------------------------------------------
 struct TcgParams {
-    CUtensorMap k_hi, k_lo;
-    CUtensorMap phi_hi[FMM_MAXDEPTH + 1], phi_lo[FMM_MAXDEPTH + 1];  // box maps of the operand layout
-    const char *op_hi, *op_lo;  // operand copies of the grid charges (every level)
-    int row_bytes;              // bytes of one cell vector in the operand layout
+    CUtensorMap k;                        // kernel tables: [343][N] rows of chunks
+    CUtensorMap phi[FMM_MAXDEPTH + 1];    // box maps of the operand copy, per level
+    const char *op;                       // the operand copy
     int lmin, depth, p3, spow, nseg;
     const int *occ;             // occupied-cell lists
-    long long op_cell0[FMM_MAXDEPTH + 2];  // first operand cell of each level
     long long loc_off[FMM_MAXDEPTH + 1];
-    long long q_off[FMM_MAXDEPTH + 1];
+    long long q_off[FMM_MAXDEPTH + 1];    // first cell of a level in the padded layout
+    long long part_off[FMM_MAXDEPTH + 1], part_stride[FMM_MAXDEPTH + 1];  // partials of levels with tc_parts > 1
     float *loc;
-    const float *qlev;
+    float *part;
+    const float2 *qsc;  // per cell: total charge, factor of its scaled operands (see KSplit)
     const float *kbar;  // [343][N], zero padded
     int *status;
     int inject_stall;   // test hook: the first stage's kernel copies are withheld
@@ -274,74 +304,91 @@ struct TcgParams {
     // per axis, every cell of every system one row, gathered.  xseg: [nseg]
     // rows per segment, [nseg + 1] prefix of their tiles, [nseg] first list
     // entry, then the list (system << 12 | Z << 8 | Y << 4 | X); xsys: per
-    // system its operand copies, charges and functionals (op_hi, op_lo, qlev,
-    // loc above are unused).
+    // system its operand copy, charges and functionals (qsc, loc above are
+    // unused; op is the start of the batch's workspace).
     const TcXSys *xsys;
     const int *xseg;
 };
 
-// Ring depths per tile shape.  N >= 128: the gathered A stages (32 KB each)
-// and the kernel-matrix B stages (2 N 128 bytes) are separate rings with their
-// own producers, so the gather keeps G = SA - 1 stages of copies in flight per
-// producer thread; one CTA per SM (N = 224: 3 A + 2 B stages, 208 KB; N = 128:
-// 3 + 3, 192 KB).  Dynamic plus static shared memory stays below 227 KB.  N <= 64 (UNI): one ring whose stages hold A and B, one
-// producer warp whose first lane also issues the B copies, six warps and two
-// CTAs per SM (each CTA's barrier round trips and epilogue hide under the
-// other's MMAs).
-template <int N, int MODE, bool CROSS = false>
+// Ring depths per tile shape.  N >= 128: the A stages (32 KB) and the kernel
+// stages (N 256 bytes) are separate rings with their own producers, one CTA per
+// SM (N = 224: 3 A + 2 B stages, 208 KB; N = 128: 3 + 3, 192 KB).  Dynamic plus
+// static shared memory stays below 227 KB.  N <= 64 (UNI): one ring whose
+// stages hold A and B, six warps and two CTAs per SM (each CTA's barrier round
+// trips and epilogue hide under the other's MMAs).  N = 224 needs about 210
+// registers per epilogue thread (112 sums and their compensations): the other
+// warpgroup gives its share up (216 x 256 + 72 x 128 = 168 x 384).
+template <int N, int MODE>
 struct TcgShape {
     typedef TcShape<N, MODE> B;
     static constexpr bool UNI = N <= 64;
-    // producer (gather) warps: cross-system tiles of the narrow shapes gather
-    // every row (no box copies), with two warps
-    static constexpr int PW = UNI ? (CROSS ? 2 : 1) : 2;
-    static_assert(32 % PW == 0, "the gather's row groups: 32 per stage, PW warps");
-    static constexpr int NPROD = 32 * PW;
-    static constexpr int SA = UNI ? 2 : 3;
-    static constexpr int SB = N == 128 ? 3 : 2;
-    static constexpr int G = SA - 1;                 // copy groups in flight per producer thread
-    static constexpr int ASTAGE = 2 * TC_ABYTES;     // hi, lo
-    static constexpr int BSTAGE = 2 * B::BBYTES;     // hi, lo
-    static constexpr int WB = B::EPI + PW;           // kernel-matrix TMA warp (split rings)
+    static constexpr int SA = N == 32 ? 4 : (N == 64 ? 2 : 3);
+    static constexpr int SB = N == 224 ? 2 : (N == 128 ? 3 : SA);
+    static constexpr int ASTAGE = (B::FC ? 2 : 1) * TC_ABYTES;
+    static constexpr int BSTAGE = (B::FC ? 2 : 1) * B::BBYTES;
+    static constexpr int PW = UNI ? 1 : 2;           // A warps
+    static constexpr int G = SA - 1;                 // stages of copies in flight per gathering thread
+    static constexpr int WA = B::EPI;
+    static constexpr int WB = WA + PW;               // kernel-matrix warp (split rings)
     static constexpr int WM = UNI ? WB : WB + 1;     // MMA warp
+    static constexpr bool SETREG = N == 224 && B::COMP;
     static constexpr int THREADS = 32 * (WM + 1);
+    static_assert(!SETREG || THREADS == 384, "three warpgroups");
     static constexpr int MINB = UNI ? 2 : 1;
-    // rings, barriers, the rows' tables (cross-system tiles: also each row's
-    // system and its operand addresses)
-    static constexpr int SMEM = 1024 + SA * ASTAGE + SB * BSTAGE + 256 + 3 * TC_M * 4 + (CROSS ? TC_M * 4 + 2 * TC_M * 8 : 0);
+    // rings, barriers, two offsets' row means, the rows' tables
+    static constexpr int SMEM = 1024 + SA * ASTAGE + SB * BSTAGE + 256 + 2 * N * 4 + 4 * TC_M * 4;
     static_assert(SMEM + 1024 <= 227 * 1024, "shared memory of one CTA");
 };
 
-template <int G>
-__device__ __forceinline__ void cp_async_wait_pending() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(G) : "memory");
+// one step of a compensated sum of pairs: run += t, the rounding error of the
+// addition carried to the next step in comp (two bfloat16: eight bits of it)
+__device__ __forceinline__ void kahan_add(float2 &run, uint32_t &comp, float2 t) {
+    const float2 y = __fadd2_rn(t, make_float2(__uint_as_float(comp << 16), __uint_as_float(comp & 0xFFFF0000u)));
+    const float2 s = __fadd2_rn(run, y);
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    const float2 z = __ffma2_rn(run, m1, s);
+    const float2 e = __ffma2_rn(z, m1, y);
+    const __nv_bfloat162 c = __floats2bfloat162_rn(e.x, e.y);
+    comp = *reinterpret_cast<const uint32_t *>(&c);
+    run = s;
+}
+
+// The next part of a sum of several runs: (h, w) += t with the rounding error
+// of the addition kept in w; after the last part h is the sum.
+__device__ __forceinline__ void part_add(float &h, float &w, float t, bool last) {
+    const float s = h + t, b = s - h;
+    w += (h - (s - b)) + (t - b);
+    h = last ? s + w : s;
 }
 
 template <int N, int MODE, bool CROSS = false>
 struct KM2LTcg {
-    static constexpr int BS = TcgShape<N, MODE, CROSS>::THREADS, MINB = TcgShape<N, MODE, CROSS>::MINB;
-    static constexpr int SMEM = TcgShape<N, MODE, CROSS>::SMEM;
+    static constexpr int BS = TcgShape<N, MODE>::THREADS, MINB = TcgShape<N, MODE>::MINB;
+    static constexpr int SMEM = TcgShape<N, MODE>::SMEM;
     TcgParams prm;
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
         typedef TcShape<N, MODE> Sh;
-        typedef TcgShape<N, MODE, CROSS> Gh;
-        // the segments' counts and tile prefix, read once into shared memory
-        __shared__ int seg_cnt[8 * (FMM_MAXDEPTH + 1)], seg_tiles[8 * (FMM_MAXDEPTH + 1) + 1];
+        typedef TcgShape<N, MODE> Gh;
+        // the segments' counts and block prefix, read once into shared memory
+        __shared__ int seg_cnt[8 * (FMM_MAXDEPTH + 1)], seg_first[8 * (FMM_MAXDEPTH + 1) + 1];
         constexpr bool cross = CROSS;
         {
-            const int *cnt_g = cross ? prm.xseg : prm.occ + occ_nblk(prm.depth, prm.lmin), *tiles_g = cnt_g + prm.nseg;
-            if ((int)threadIdx.x <= prm.nseg) seg_tiles[threadIdx.x] = tiles_g[threadIdx.x];
+            const int *cnt_g = cross ? prm.xseg : prm.occ + occ_nblk(prm.depth, prm.lmin), *first_g = cnt_g + prm.nseg;
+            if ((int)threadIdx.x <= prm.nseg) seg_first[threadIdx.x] = first_g[threadIdx.x];
             if ((int)threadIdx.x < prm.nseg) seg_cnt[threadIdx.x] = cnt_g[threadIdx.x];
             __syncthreads();
         }
-        if ((int)bid_ >= seg_tiles[prm.nseg]) return;  // past the last occupied tile
-        int sg = 0;
-        while (sg + 1 < prm.nseg && (int)bid_ >= seg_tiles[sg + 1]) sg++;
+        if ((int)bid_ >= seg_first[prm.nseg]) return;  // past the last occupied tile
+        int k = 0;
+        while (k + 1 < prm.nseg && (int)bid_ >= seg_first[k + 1]) k++;
+        const int sg = cross ? k : prm.nseg - 1 - k;  // a system's own blocks: the deepest level first
         const int l = prm.lmin + sg / 8, par = sg & 7;
-        const int bx = par & 1, by = (par >> 1) & 1, bz = par >> 2;
-        const int H = 1 << (l - 1), P = H + 2, Pt = (int)tc_level_extent(l);
+        const int H = 1 << (l - 1), P = H + 2;
         const int count = seg_cnt[sg];
-        const int r0 = ((int)bid_ - seg_tiles[sg]) * TC_M;  // first list entry of the tile
+        const int parts = cross ? 1 : tc_parts(l, prm.depth);
+        const int tile = ((int)bid_ - seg_first[k]) / parts, part = ((int)bid_ - seg_first[k]) % parts;
+        const int i0 = part * (TC_NOFF / parts), i1 = i0 + TC_NOFF / parts;  // this block's offsets
+        const int r0 = tile * TC_M;  // first list entry of the tile
         const int *lst = cross ? prm.xseg + 3 * prm.nseg + 1 + prm.xseg[2 * prm.nseg + 1 + sg]
                                : prm.occ + occ_list_offset(prm.depth, prm.lmin) + occ_seg_first(prm.lmin, sg);
 
@@ -356,39 +403,29 @@ struct KM2LTcg {
         const uint32_t done = rfree0 + 16;
         const uint32_t tslot = done + 8;
         volatile uint32_t *tslot_ptr = reinterpret_cast<volatile uint32_t *>(smraw + (tslot - raw));
-        // per row: source-cell base in the operand layout, cell in the padded
-        // Phi layout (charges Q), target cell in the L layout (-1: past the
-        // list); cross-system tiles: its system and the addresses of its source
-        // cell in that system's hi / lo operand copies
-        int *rowA = reinterpret_cast<int *>(smraw + (bars - raw) + 256);
-        int *rowQ = rowA + TC_M, *rowL = rowQ + TC_M, *rowS = rowL + TC_M;
-        const char **rowBh = reinterpret_cast<const char **>(rowS + TC_M), **rowBl = rowBh + TC_M;
+        float *kbs = reinterpret_cast<float *>(smraw + (bars - raw) + 256);  // row means of two offsets
+        // per row: first chunk of its own cell in the operand copy, cell in the
+        // padded layout, target cell in the L layout (-1: past the list), system
+        int *rowG = reinterpret_cast<int *>(kbs + 2 * N);
+        int *rowQ = rowG + TC_M, *rowL = rowQ + TC_M, *rowS = rowL + TC_M;
 
-        // Box tiles (occ_box_segment: a level with fewer than 8 coarse cells per
-        // axis, or a segment whose cells mostly hold charges): tile t is the 128
-        // consecutive Morton cells [128 t, 128 t + 128), one 8 x 4 x 4 box, and
-        // each offset's A operand is one TMA box copy (row r = x + 8 y + 32 z of
-        // the box) instead of 128 gathered rows.  A level with fewer than 8 coarse
-        // cells per axis takes one box at the origin, partly outside the grid (the
-        // operand layout holds zeros there; those rows are not stored).
+        // Box tiles (occ_box_segment): tile t is the 128 consecutive Morton cells
+        // [128 t, 128 t + 128), one 8 x 4 x 4 box, and each chunk's A operand is
+        // one TMA box copy (row r = x + 8 y + 32 z of the box).
         const bool box = !cross && occ_box_segment(H, count, N);
-        // one ring whose stages hold A and B, filled by one thread (box tiles, and
-        // every tile of the narrow shapes), or split rings (gathered tiles of N >= 128)
-        const bool uni = Gh::UNI || box;
-        const int SU = Gh::SA < Gh::SB ? Gh::SA : Gh::SB;
-        const int ra = uni ? SU : Gh::SA, rb = uni ? SU : Gh::SB;  // ring depths of A and B
+        // rows past the list hold no operand: their groups of four are not copied
+        const int ngroups = box ? TC_M / 4 : (min(TC_M, count - r0) + 3) / 4;
         int X0 = 0, Y0 = 0, Z0 = 0;
         if (box) morton_decode((uint32_t)r0, X0, Y0, Z0);
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         if (threadIdx.x < TC_M) {
             const int r = threadIdx.x;
-            int X, Y, Z;
-            bool in;
+            int X, Y, Z, sys = 0;
+            bool in = true;
             if (box) {
                 X = X0 + (r & 7);
                 Y = Y0 + ((r >> 3) & 3);
                 Z = Z0 + (r >> 5);
-                in = X < H && Y < H && Z < H;
             } else {
                 in = r0 + r < count;
                 const int pk = lst[in ? r0 + r : r0];  // rows past the list repeat the tile's first cell
@@ -396,27 +433,23 @@ struct KM2LTcg {
                     X = pk & 15;
                     Y = (pk >> 4) & 15;
                     Z = (pk >> 8) & 15;
-                    rowS[r] = pk >> 12;
+                    sys = pk >> 12;
                 } else {
                     X = pk & 1023;
                     Y = (pk >> 10) & 1023;
                     Z = pk >> 20;
                 }
             }
-            rowA[r] = ((Z + 1) * Pt + Y + 1) * Pt + X + 1;
             rowQ[r] = ((Z + 1) * P + Y + 1) * P + X + 1;
             rowL[r] = in ? ((par * H + Z) * H + Y) * H + X : -1;
-            if (cross) {
-                const TcXSys &xs = prm.xsys[rowS[r]];
-                rowBh[r] = xs.op_hi + (int64_t)rowA[r] * prm.row_bytes;
-                rowBl[r] = xs.op_lo + (int64_t)rowA[r] * prm.row_bytes;
-            }
+            rowS[r] = sys;
+            rowG[r] = (cross ? prm.xsys[sys].op_chunk : 0) + (int)(prm.q_off[l] + rowQ[r]) * Sh::RC;
         }
         if (threadIdx.x == 0) {
             for (int s = 0; s < Gh::SA; s++) {
-                // arrivals: the box copies' issuer, or every gather thread (plus the
-                // issuer of the B copies when they share the ring)
-                tc::mbar_init(afull0 + 8 * s, box ? 1 : Gh::NPROD + (uni ? 1 : 0));
+                // arrivals: the copies' issuer (box), or every gathering thread (and
+                // the issuer of the B copies that share the ring)
+                tc::mbar_init(afull0 + 8 * s, box ? 1 : 32 * Gh::PW + (Gh::UNI ? 1 : 0));
                 tc::mbar_init(aempty0 + 8 * s, 1);
             }
             for (int s = 0; s < Gh::SB; s++) {
@@ -435,212 +468,56 @@ struct KM2LTcg {
         __syncthreads();
         tc::fence_after_sync();
         const uint32_t tmem = *tslot_ptr;
-
-        if (warp >= Sh::EPI && warp < Sh::EPI + Gh::PW && (!box || (warp == Sh::EPI && lane == 0))) {
-            // ---- A producers.  Box tiles: the first lane issues one TMA box (hi,
-            //      lo) per stage.  Otherwise the gather: lane = (row within a group
-            //      of four) * 8 + 16-byte chunk, warp pw takes rows 4 (pw + PW i) +
-            //      lane / 8; a stage is signalled once its copies are complete and
-            //      fenced for the async proxy, G - 1 stages later (G stages of copies
-            //      in flight).  With one ring (UNI) the first lane also issues the
-            //      stage's B copies. ----
-            const int pw = warp - Sh::EPI;
-            const bool lead = pw == 0 && lane == 0;
-            if (lead) {
-                if (box) {
-                    tc::tensormap_acquire(&prm.phi_hi[l]);
-                    if (Sh::LO) tc::tensormap_acquire(&prm.phi_lo[l]);
-                }
-                if (uni) {
-                    tc::tensormap_acquire(&prm.k_hi);
-                    if (Sh::LO) tc::tensormap_acquire(&prm.k_lo);
-                }
-            }
-            const int j = lane & 7, rsub = lane >> 3;
-            constexpr uint32_t ABYTES = Sh::LO ? 2 * TC_ABYTES : TC_ABYTES;
-            constexpr uint32_t BBYTES = Sh::LO ? 2 * Sh::BBYTES : Sh::BBYTES;
-            bool failed = false;
-            int last_phase[8] = {-1, -1, -1, -1, -1, -1, -1, -1};
-            int sig = 0;  // next gathered stage to signal
-            const int64_t lvl0 = prm.op_cell0[l];
-            const int64_t pt3 = (int64_t)Pt * Pt * Pt;
-            int ox = -2 - bx - 1, oy = -2 - by, oz = -2 - bz, it = 0;
-            while (!failed && next_offset(bx, by, bz, ox, oy, oz)) {
-                const Off f = make_off(bx, by, bz, ox, oy, oz);
-                const int64_t delta = lvl0 + f.spar * pt3 + ((int64_t)f.dZ * Pt + f.dY) * Pt + f.dX;
-                const int cX = X0 + 1 + f.dX, cY = Y0 + 1 + f.dY, cZ = Z0 + 1 + f.dZ;
-                for (int kc = 0; kc < Sh::KC; kc++, it++) {
-                    const int s = it % ra;
-                    const uint32_t ph = (uint32_t)(it / ra) & 1u;
-                    if (!tc::mbar_wait(aempty0 + 8 * s, ph ^ 1u, TC_WAIT_CYCLES)) {
-                        if (lane == 0) tc_wait_failed(prm.status, 1, l, it);
-                        failed = true;
-                        break;
-                    }
-                    const uint32_t st = abase + s * Gh::ASTAGE;
-                    const uint32_t fb = afull0 + 8 * s;
-                    // TMA bytes of this stage (an arrival of its own; none when the
-                    // lead only gathers)
-                    const uint32_t tx = (box ? ABYTES : 0u) + (uni ? BBYTES : 0u);
-                    if (lead && tx) {
-                        tc::mbar_expect_tx(fb, tx);
-                        last_phase[s] = (int)ph;
-                        if (box) {
-                            tc::tma_load_5d(st, &prm.phi_hi[l], fb, kc * Sh::KE, cX, cY, cZ, f.spar);
-                            if (Sh::LO) tc::tma_load_5d(st + TC_ABYTES, &prm.phi_lo[l], fb, kc * Sh::KE, cX, cY, cZ, f.spar);
-                        }
-                        if (uni && !(prm.inject_stall && it == 0)) {  // inject: armed, never filled
-                            const uint32_t stb = bbase + s * Gh::BSTAGE;
-                            tc::tma_load_3d(stb, &prm.k_hi, fb, kc * Sh::KE, 0, f.oi);
-                            if (Sh::LO) tc::tma_load_3d(stb + Sh::BBYTES, &prm.k_lo, fb, kc * Sh::KE, 0, f.oi);
-                        }
-                    }
-                    if (box) continue;
-                    const int64_t cb = (int64_t)kc * 128 + j * 16;
-                    if (cross) {  // each row from its system's operand copies
-                        const int64_t src = delta * prm.row_bytes + cb;
-#pragma unroll 4
-                        for (int i = 0; i < 32 / Gh::PW; i++) {
-                            const int r = 4 * (pw + Gh::PW * i) + rsub;
-                            const uint32_t d = st + r * 128 + ((j ^ (r & 7)) << 4);
-                            tc::cp_async16(d, rowBh[r] + src);
-                            if (Sh::LO) tc::cp_async16(d + TC_ABYTES, rowBl[r] + src);
-                        }
-                    } else {
-#pragma unroll 4
-                        for (int i = 0; i < 32 / Gh::PW; i++) {
-                            const int r = 4 * (pw + Gh::PW * i) + rsub;
-                            const int64_t src = (delta + rowA[r]) * prm.row_bytes + cb;
-                            const uint32_t d = st + r * 128 + ((j ^ (r & 7)) << 4);
-                            tc::cp_async16(d, prm.op_hi + src);
-                            if (Sh::LO) tc::cp_async16(d + TC_ABYTES, prm.op_lo + src);
-                        }
-                    }
-                    tc::cp_async_commit();
-                    cp_async_wait_pending<Gh::G - 1>();  // stages <= it - G + 1 have landed
-                    if (it - Gh::G + 1 >= sig) {
-                        tc::fence_proxy_async_smem();
-                        for (; sig <= it - Gh::G + 1; sig++) tc::mbar_arrive(afull0 + 8 * (sig % ra));
-                    }
-                }
-            }
-            if (!box) {
-                tc::cp_async_wait_all();  // no copy outlives the CTA
-                if (!failed) {
-                    tc::fence_proxy_async_smem();
-                    for (; sig < it; sig++) tc::mbar_arrive(afull0 + 8 * (sig % ra));
-                }
-            }
-            if (failed) {
-                if (lane == 0) atomicOr(prm.status, ST_TIMEOUT);
-                if (lead)  // the TMA copies already issued land before the CTA can exit
-                    for (int s = 0; s < ra; s++)
-                        if (last_phase[s] >= 0) tc::mbar_wait(afull0 + 8 * s, (uint32_t)last_phase[s], TC_WAIT_CYCLES);
-            }
-        } else if (!uni && warp == Gh::WB && lane == 0) {
-            tc::tensormap_acquire(&prm.k_hi);
-            if (Sh::LO) tc::tensormap_acquire(&prm.k_lo);
-            // ---- kernel-matrix producer (split rings): K chunk kc of K_o by TMA ----
-            bool failed = false;
-            int last_phase[4] = {-1, -1, -1, -1};
-            int ox = -2 - bx - 1, oy = -2 - by, oz = -2 - bz, it = 0;
-            while (!failed && next_offset(bx, by, bz, ox, oy, oz)) {
-                const Off f = make_off(bx, by, bz, ox, oy, oz);
-                for (int kc = 0; kc < Sh::KC; kc++, it++) {
-                    const int s = it % Gh::SB;
-                    const uint32_t ph = (uint32_t)(it / Gh::SB) & 1u;
-                    if (!tc::mbar_wait(bempty0 + 8 * s, ph ^ 1u, TC_WAIT_CYCLES)) {
-                        tc_wait_failed(prm.status, 1, l, it);
-                        failed = true;
-                        break;
-                    }
-                    const uint32_t st = bbase + s * Gh::BSTAGE;
-                    const uint32_t fb = bfull0 + 8 * s;
-                    tc::mbar_expect_tx(fb, Sh::LO ? 2 * Sh::BBYTES : Sh::BBYTES);
-                    last_phase[s] = (int)ph;
-                    if (prm.inject_stall && it == 0) continue;  // armed, never filled (test hook)
-                    tc::tma_load_3d(st, &prm.k_hi, fb, kc * Sh::KE, 0, f.oi);
-                    if (Sh::LO) tc::tma_load_3d(st + Sh::BBYTES, &prm.k_lo, fb, kc * Sh::KE, 0, f.oi);
-                }
-            }
-            if (failed) {
-                atomicOr(prm.status, ST_TIMEOUT);
-                // the copies already issued land before the CTA can exit
-                for (int s = 0; s < Gh::SB; s++)
-                    if (last_phase[s] >= 0) tc::mbar_wait(bfull0 + 8 * s, (uint32_t)last_phase[s], TC_WAIT_CYCLES);
-            }
-        } else if (warp == Gh::WM && lane == 0) {
-            // ---- MMA issuer: offset i accumulates into TMEM region i & 1 ----
-            const uint32_t idesc = MODE == TC_BF16X3 ? tc::idesc_bf16(TC_M, N) : tc::idesc_tf32(TC_M, N);
-            bool failed = false;
-            for (int i = 0; i < TC_NOFF && !failed; i++) {
-                const int r = i & 1;
-                const uint32_t u = (uint32_t)(i >> 1) & 1u;
-                if (!tc::mbar_wait(rfree0 + 8 * r, u ^ 1u, TC_WAIT_CYCLES)) {
-                    tc_wait_failed(prm.status, 2, l, i);
-                    failed = true;
-                    break;
-                }
-                const uint32_t d = tmem + (uint32_t)(r * N);
-                for (int kc = 0; kc < Sh::KC; kc++) {
-                    const int it = Sh::KC * i + kc;
-                    const int sa = it % ra, sb = it % rb;
-                    if (!tc::mbar_wait(afull0 + 8 * sa, (uint32_t)(it / ra) & 1u, TC_WAIT_CYCLES) ||
-                        (!uni && !tc::mbar_wait(bfull0 + 8 * sb, (uint32_t)(it / rb) & 1u, TC_WAIT_CYCLES))) {
-                        tc_wait_failed(prm.status, 3, l, it);
-                        failed = true;
-                        break;
-                    }
-                    tc::fence_after_sync();
-                    const uint32_t sta = abase + sa * Gh::ASTAGE, stb = bbase + sb * Gh::BSTAGE;
-#pragma unroll
-                    for (int k = 0; k < 4; k++) {  // 32 bytes of K per MMA (8 tf32 or 16 bf16)
-                        const uint64_t ah = tc::desc_sw128(sta + 32 * k);
-                        const uint64_t al = tc::desc_sw128(sta + TC_ABYTES + 32 * k);
-                        const uint64_t bh = tc::desc_sw128(stb + 32 * k);
-                        const uint64_t bl = tc::desc_sw128(stb + Sh::BBYTES + 32 * k);
-                        if (MODE == TC_BF16X3) {
-                            tc::mma_bf16(d, ah, bh, idesc, (kc | k) != 0);
-                            tc::mma_bf16(d, ah, bl, idesc, 1u);
-                            tc::mma_bf16(d, al, bh, idesc, 1u);
-                        } else {
-                            tc::mma_tf32(d, ah, bh, idesc, (kc | k) != 0);
-                            if (MODE == TC_TF32X3) {
-                                tc::mma_tf32(d, ah, bl, idesc, 1u);
-                                tc::mma_tf32(d, al, bh, idesc, 1u);
-                            }
-                        }
-                    }
-                    tc::mma_commit(aempty0 + 8 * sa);
-                    if (!uni) tc::mma_commit(bempty0 + 8 * sb);
-                }
-                if (!failed) tc::mma_commit(rfull0 + 8 * r);
-            }
-            if (failed) atomicOr(prm.status, ST_TIMEOUT);
-            tc::mma_commit(done);  // always: the deallocation waits on it
-        } else if (warp < Sh::EPI) {
+        // Register shares (SETREG): whole warpgroups 0-3 and 4-7 (epilogue) and 8-11,
+        // each group's change one instruction, its role inside the branch.
+        if (warp < Sh::EPI) {
+            if constexpr (Gh::SETREG) tc::setmaxnreg_inc<216>();
             // ---- epilogue: TMEM lane = row; columns [c0, c0 + COLS) ----
             const int sub = warp & 3, cgrp = warp >> 2;
             const int c0 = cgrp * Sh::COLS;
             const int row = sub * 32 + lane;
             const int lrow = rowL[row];
             const bool valid = lrow >= 0;
-            const float *q = (cross ? prm.xsys[rowS[row]].qlev : prm.qlev) + prm.q_off[l] + rowQ[row];
-            const int64_t pp3 = (int64_t)P * P * P;
-            float tot[Sh::COLS];
+            const float2 *q = (cross ? prm.xsys[rowS[row]].qsc : prm.qsc) + prm.q_off[l] + rowQ[row];
+            const int p3 = prm.p3;
+            float *out = (cross ? prm.xsys[rowS[row]].loc + prm.loc_off[l]
+                          : parts > 1 ? prm.part + prm.part_off[l] + part * prm.part_stride[l] : prm.loc + prm.loc_off[l]) +
+                         (int64_t)(valid ? lrow : 0) * p3 + c0;
+            // the totals' low parts of the widest cross-system tile
+            float *out_lo = cross && Sh::RMW
+                                ? prm.xsys[rowS[row]].part + prm.loc_off[l] + (int64_t)(valid ? lrow : 0) * p3 + c0 : nullptr;
+            const float scale = (float)(1 << (l * prm.spow));
+            // where the totals of a cross-system tile's runs wait (this thread's columns)
+            const uint32_t ttot = tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(2 * N + c0);
+            float2 run[Sh::COLS / 2];
+            uint32_t comp[Sh::COMP ? Sh::COLS / 2 : 1];
 #pragma unroll
-            for (int j = 0; j < Sh::COLS; j++) tot[j] = 0.0f;
+            for (int j = 0; j < Sh::COLS / 2; j++) {
+                run[j] = make_float2(0.0f, 0.0f);
+                if (Sh::COMP) comp[j] = 0u;
+            }
             bool ok = true;
-            int ox = -2 - bx - 1, oy = -2 - by, oz = -2 - bz;
-            for (int i = 0; i < TC_NOFF; i++) {
-                next_offset(bx, by, bz, ox, oy, oz);
-                const Off f = make_off(bx, by, bz, ox, oy, oz);
-                const float Qs = valid ? q[f.spar * pp3 + ((int64_t)f.dZ * P + f.dY) * P + f.dX] : 0.0f;
-                const float4 *kb = reinterpret_cast<const float4 *>(prm.kbar + (int64_t)f.oi * N + c0);
-                const int r = i & 1;
-                const uint32_t u = (uint32_t)(i >> 1) & 1u;
+            // the row's source charge and factor, and the row means Kbar_o, are
+            // fetched one offset ahead: the charge into registers, the means by the
+            // epilogue's threads into a shared row
+            auto source = [&](int i) {
+                const Off f = list_offset(par, i);
+                return valid ? q[((f.spar * P + f.dZ) * P + f.dY) * P + f.dX] : make_float2(0.0f, 0.0f);
+            };
+            const int et = threadIdx.x;  // epilogue thread (the epilogue warps come first)
+            float2 qs = source(i0);
+            if (et < N) kbs[et] = prm.kbar[list_offset(par, i0).oi * N + et];
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * Sh::EPI) : "memory");
+            for (int i = i0; i < i1; i++) {
+                const int j = i - i0, in = i + 1 < i1 ? i + 1 : i;
+                const float2 qn = source(in);
+                const float kn = et < N ? prm.kbar[list_offset(par, in).oi * N + et] : 0.0f;
+                const float2 Q2 = make_float2(qs.x, qs.x), inv2 = make_float2(qs.y, qs.y);
+                const float *kb = kbs + (j & 1) * N + c0;
+                const int r = j & 1;
+                const uint32_t u = (uint32_t)(j >> 1) & 1u;
                 if (ok && !tc::mbar_wait(rfull0 + 8 * r, u, TC_WAIT_CYCLES)) {
-                    if (lane == 0) tc_wait_failed(prm.status, 4, l, i);
+                    if (lane == 0) tc_wait_failed(prm.status, 4, l, j);
                     ok = false;
                 }
                 tc::fence_after_sync();
@@ -650,28 +527,274 @@ struct KM2LTcg {
                     uint32_t v[16];
                     tc::tmem_ld16(taddr + c * 16, v);
 #pragma unroll
-                    for (int j = 0; j < 16; j += 4) {
-                        const float4 m = kb[(c * 16 + j) >> 2];
-                        tot[c * 16 + j] += __uint_as_float(v[j]) + m.x * Qs;
-                        tot[c * 16 + j + 1] += __uint_as_float(v[j + 1]) + m.y * Qs;
-                        tot[c * 16 + j + 2] += __uint_as_float(v[j + 2]) + m.z * Qs;
-                        tot[c * 16 + j + 3] += __uint_as_float(v[j + 3]) + m.w * Qs;
+                    for (int e = 0; e < 16; e += 4) {
+                        // the offset's contribution with its monopole term Kbar Q
+                        const float4 m = *reinterpret_cast<const float4 *>(kb + c * 16 + e);
+                        const float2 m0 = make_float2(m.x, m.y), m1 = make_float2(m.z, m.w);
+                        float2 d0 = make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+                        float2 d1 = make_float2(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
+                        if (Sh::SCALED) {
+                            d0 = __ffma2_rn(d0, inv2, __fmul2_rn(m0, Q2));
+                            d1 = __ffma2_rn(d1, inv2, __fmul2_rn(m1, Q2));
+                        } else {
+                            d0 = __ffma2_rn(m0, Q2, d0);
+                            d1 = __ffma2_rn(m1, Q2, d1);
+                        }
+                        const int x = (c * 16 + e) / 2;
+                        if constexpr (Sh::COMP) {
+                            kahan_add(run[x], comp[x], d0);
+                            kahan_add(run[x + 1], comp[x + 1], d1);
+                        } else {
+                            run[x] = __fadd2_rn(run[x], d0);
+                            run[x + 1] = __fadd2_rn(run[x + 1], d1);
+                        }
                     }
                 }
                 tc::fence_before_sync();
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(rfree0 + 8 * r) : "memory");
-            }
-            const int p3 = prm.p3;
-            float *out = (cross ? prm.xsys[rowS[row]].loc : prm.loc) + prm.loc_off[l] + (int64_t)(valid ? lrow : 0) * p3 + c0;
-            const float scale = (float)(1 << (l * prm.spow));
-            if (ok) {
-                if (valid) {
+                tc::mbar_arrive(rfree0 + 8 * r);
+                qs = qn;
+                if (et < N) kbs[((j + 1) & 1) * N + et] = kn;
+                asm volatile("bar.sync 1, %0;" ::"n"(32 * Sh::EPI) : "memory");
+                // a cross-system tile adds its offsets in the same runs as a system's
+                // own blocks of these levels do (one run per block, added by
+                // k_tc_reduce in order), for the same sums bit for bit
+                if (cross && (j + 1) % (TC_NOFF / TC_PARTS_SMALL) == 0) {
+                    const bool first = j + 1 == TC_NOFF / TC_PARTS_SMALL, last = j + 1 == TC_NOFF;
+                    if constexpr (Sh::RMW) {  // p^3 = 216 values: rows of whole, aligned float4
+                        if (ok && valid) {
 #pragma unroll
-                    for (int j = 0; j < Sh::COLS; j++)
-                        if (c0 + j < p3) out[j] = scale * tot[j];
+                            for (int e = 0; e < Sh::COLS; e += 4) {
+                                if (c0 + e >= p3) break;
+                                float4 *h4 = reinterpret_cast<float4 *>(out + e), *w4 = reinterpret_cast<float4 *>(out_lo + e);
+                                const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                                float4 h = first ? z : *h4, w = first ? z : *w4;
+                                part_add(h.x, w.x, scale * run[e / 2].x, last);
+                                part_add(h.y, w.y, scale * run[e / 2].y, last);
+                                part_add(h.z, w.z, scale * run[e / 2 + 1].x, last);
+                                part_add(h.w, w.w, scale * run[e / 2 + 1].y, last);
+                                *h4 = h;
+                                if (!last) *w4 = w;
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < Sh::COLS / 16; c++) {
+                            uint32_t h[16], w[16];
+#pragma unroll
+                            for (int e = 0; e < 16; e++) h[e] = w[e] = 0u;
+                            if (!first) {
+                                tc::tmem_ld16(ttot + c * 16, h);
+                                tc::tmem_ld16(ttot + N + c * 16, w);
+                            }
+#pragma unroll
+                            for (int e = 0; e < 16; e++) {
+                                float &t = e & 1 ? run[c * 8 + e / 2].y : run[c * 8 + e / 2].x;
+                                float hf = __uint_as_float(h[e]), wf = __uint_as_float(w[e]);
+                                part_add(hf, wf, t, last);
+                                if (last) t = hf;
+                                h[e] = __float_as_uint(hf);
+                                w[e] = __float_as_uint(wf);
+                            }
+                            if (!last) {
+                                tc::tmem_st16(ttot + c * 16, h);
+                                tc::tmem_st16(ttot + N + c * 16, w);
+                            }
+                        }
+                        tc::tmem_wait_st();
+                    }
+                    if (j + 1 < TC_NOFF) {
+#pragma unroll
+                        for (int e = 0; e < Sh::COLS / 2; e++) {
+                            run[e] = make_float2(0.0f, 0.0f);
+                            if (Sh::COMP) comp[e] = 0u;
+                        }
+                    }
+                }
+            }
+            if (ok) {
+                if (!(cross && Sh::RMW) && valid) {
+#pragma unroll
+                    for (int e = 0; e < Sh::COLS; e++)
+                        if (c0 + e < p3) out[e] = scale * (e & 1 ? run[e / 2].y : run[e / 2].x);
                 }
             } else if (lane == 0) {
                 atomicOr(prm.status, ST_TIMEOUT);
+            }
+        } else {
+            if constexpr (Gh::SETREG) tc::setmaxnreg_dec<72>();
+            if (warp < Gh::WA + Gh::PW) {
+                // ---- A producers; with one ring (UNI) the first lane also issues the
+                //      stage's B copies.  Gather: lane = 8 (row within a group of four) +
+                //      16-byte piece; warp pw takes the groups pw + PW i.  A stage is
+                //      signalled once its copies are complete and fenced, G - 1 stages
+                //      later. ----
+                const int pw = warp - Gh::WA;
+                const bool lead = pw == 0 && lane == 0;
+                if (lead) {
+                    if (box) tc::tensormap_acquire(&prm.phi[l]);
+                    if (Gh::UNI) tc::tensormap_acquire(&prm.k);
+                }
+                constexpr int RI = 32 / Gh::PW;
+                const int piece = lane & 7, rsub = lane >> 3;
+                // groups of this warp that hold rows of the tile
+                const int ni = box ? 0 : (ngroups - pw + Gh::PW - 1) / Gh::PW;
+                int g[RI];
+                uint32_t place[2 / Gh::PW];  // of the groups i (mod 2 / PW), 1 KB a further pair of groups
+                if (!box) {
+#pragma unroll
+                    for (int i = 0; i < RI; i++) g[i] = rowG[4 * (pw + Gh::PW * i) + rsub];
+#pragma unroll
+                    for (int i = 0; i < 2 / Gh::PW; i++) {
+                        const int r = 4 * (pw + Gh::PW * i) + rsub;
+                        place[i] = (uint32_t)(r * 128 + ((piece ^ (r & 7)) << 4));
+                    }
+                }
+                const char *src0 = prm.op + 16 * piece;
+                bool failed = false;
+                int last_phase[4] = {-1, -1, -1, -1};
+                int it = 0, sig = 0;  // sig: next gathered stage to signal
+                for (int i = i0; i < i1 && !failed; i++) {
+                    const Off f = list_offset(par, i);
+                    const int delta = (((f.spar * P + f.dZ) * P + f.dY) * P + f.dX) * Sh::RC;
+                    for (int kc = 0; kc < Sh::KC; kc++, it++) {
+                        const int s = it % Gh::SA;
+                        const uint32_t ph = (uint32_t)(it / Gh::SA) & 1u;
+                        if (!tc::mbar_wait(aempty0 + 8 * s, ph ^ 1u, TC_WAIT_CYCLES)) {
+                            if (lane == 0) tc_wait_failed(prm.status, 1, l, it);
+                            failed = true;
+                            break;
+                        }
+                        const uint32_t st = abase + s * Gh::ASTAGE, fb = afull0 + 8 * s;
+                        const int nch = kc < Sh::FC && Sh::LO ? 2 : 1;  // chunks of this stage (a tail holds hi and lo)
+                        if (lead && (box || Gh::UNI)) {
+                            tc::mbar_expect_tx(fb, (uint32_t)(nch * ((box ? TC_ABYTES : 0) + (Gh::UNI ? Sh::BBYTES : 0))));
+                            last_phase[s] = (int)ph;
+                            if (box) {
+                                const int cX = X0 + 1 + f.dX, cY = Y0 + 1 + f.dY, cZ = Z0 + 1 + f.dZ;
+                                tc::tma_load_5d(st, &prm.phi[l], fb, 128 * kc, cX, cY, cZ, f.spar);
+                                if (nch == 2) tc::tma_load_5d(st + TC_ABYTES, &prm.phi[l], fb, 128 * kc + 64, cX, cY, cZ, f.spar);
+                            }
+                            if (Gh::UNI && !(prm.inject_stall && it == 0)) {  // inject: armed, never filled
+                                const uint32_t stb = bbase + s * Gh::BSTAGE;
+                                tc::tma_load_3d(stb, &prm.k, fb, 128 * kc, 0, f.oi);
+                                if (nch == 2) tc::tma_load_3d(stb + Sh::BBYTES, &prm.k, fb, 128 * kc + 64, 0, f.oi);
+                            }
+                        }
+                        if (box) continue;
+                        const int d = delta + 2 * kc;
+#pragma unroll
+                        for (int i = 0; i < RI; i++) {
+                            if (i >= ni) break;
+                            const char *src = src0 + (int64_t)(g[i] + d) * 128;
+                            const uint32_t to = st + place[i % (2 / Gh::PW)] + 1024 * (i / (2 / Gh::PW));
+                            tc::cp_async16(to, src);
+                            if (nch == 2) tc::cp_async16(to + TC_ABYTES, src + 128);
+                        }
+                        tc::cp_async_commit();
+                        tc::cp_async_wait_pending<Gh::G - 1>();  // stages <= it - G + 1 have landed
+                        if (it - Gh::G + 1 >= sig) {
+                            tc::fence_proxy_async_smem();
+                            for (; sig <= it - Gh::G + 1; sig++) tc::mbar_arrive(afull0 + 8 * (sig % Gh::SA));
+                        }
+                    }
+                }
+                if (!box) {
+                    tc::cp_async_wait_all();  // no copy outlives the CTA
+                    if (!failed) {
+                        tc::fence_proxy_async_smem();
+                        for (; sig < it; sig++) tc::mbar_arrive(afull0 + 8 * (sig % Gh::SA));
+                    }
+                }
+                if (failed) {
+                    if (lane == 0) atomicOr(prm.status, ST_TIMEOUT);
+                    if (lead)  // the TMA copies already issued land before the CTA can exit
+                        for (int s = 0; s < Gh::SA; s++)
+                            if (last_phase[s] >= 0) tc::mbar_wait(afull0 + 8 * s, (uint32_t)last_phase[s], TC_WAIT_CYCLES);
+                }
+            } else if (!Gh::UNI && warp == Gh::WB) {
+                // ---- kernel-matrix producer (split rings): the chunks of K_o by TMA ----
+                if (lane == 0) {
+                    tc::tensormap_acquire(&prm.k);
+                    bool failed = false;
+                    int last_phase[4] = {-1, -1, -1, -1};
+                    int it = 0;
+                    for (int i = i0; i < i1 && !failed; i++) {
+                        const int oi = list_offset(par, i).oi;
+                        for (int kc = 0; kc < Sh::KC; kc++, it++) {
+                            const int s = it % Gh::SB;
+                            const uint32_t ph = (uint32_t)(it / Gh::SB) & 1u;
+                            if (!tc::mbar_wait(bempty0 + 8 * s, ph ^ 1u, TC_WAIT_CYCLES)) {
+                                tc_wait_failed(prm.status, 1, l, it);
+                                failed = true;
+                                break;
+                            }
+                            const uint32_t st = bbase + s * Gh::BSTAGE, fb = bfull0 + 8 * s;
+                            const int nch = kc < Sh::FC && Sh::LO ? 2 : 1;
+                            tc::mbar_expect_tx(fb, (uint32_t)(nch * Sh::BBYTES));
+                            last_phase[s] = (int)ph;
+                            if (prm.inject_stall && it == 0) continue;  // armed, never filled (test hook)
+                            tc::tma_load_3d(st, &prm.k, fb, 128 * kc, 0, oi);
+                            if (nch == 2) tc::tma_load_3d(st + Sh::BBYTES, &prm.k, fb, 128 * kc + 64, 0, oi);
+                        }
+                    }
+                    if (failed) {
+                        atomicOr(prm.status, ST_TIMEOUT);
+                        // the copies already issued land before the CTA can exit
+                        for (int s = 0; s < Gh::SB; s++)
+                            if (last_phase[s] >= 0) tc::mbar_wait(bfull0 + 8 * s, (uint32_t)last_phase[s], TC_WAIT_CYCLES);
+                    }
+                }
+            } else if (warp == Gh::WM) {
+                // ---- MMA issuer: the j-th offset of the block accumulates into TMEM region j & 1 ----
+                if (lane == 0) {
+                    const uint32_t idesc = MODE == TC_BF16X3 ? tc::idesc_bf16(TC_M, N) : tc::idesc_f16(TC_M, N);
+                    bool failed = false;
+                    for (int j = 0; j < i1 - i0 && !failed; j++) {
+                        const int r = j & 1;
+                        const uint32_t u = (uint32_t)(j >> 1) & 1u;
+                        if (!tc::mbar_wait(rfree0 + 8 * r, u ^ 1u, TC_WAIT_CYCLES)) {
+                            tc_wait_failed(prm.status, 2, l, j);
+                            failed = true;
+                            break;
+                        }
+                        const uint32_t d = tmem + (uint32_t)(r * N);
+    #pragma unroll
+                        for (int kc = 0; kc < Sh::KC; kc++) {
+                            const int it = Sh::KC * j + kc;
+                            const int sa = it % Gh::SA, sb = it % Gh::SB;
+                            if (!tc::mbar_wait(afull0 + 8 * sa, (uint32_t)(it / Gh::SA) & 1u, TC_WAIT_CYCLES) ||
+                                (!Gh::UNI && !tc::mbar_wait(bfull0 + 8 * sb, (uint32_t)(it / Gh::SB) & 1u, TC_WAIT_CYCLES))) {
+                                tc_wait_failed(prm.status, 3, l, it);
+                                failed = true;
+                                break;
+                            }
+                            tc::fence_after_sync();
+                            // the stage's hi and lo parts: two chunks, or the halves of a tail chunk
+                            const bool full = kc < Sh::FC;
+                            const int ks = full ? 4 : 2;
+                            const uint32_t ah = abase + sa * Gh::ASTAGE, al = ah + (full ? TC_ABYTES : 64);
+                            const uint32_t bh = bbase + sb * Gh::BSTAGE, bl = bh + (full ? Sh::BBYTES : 64);
+                            // 32 bytes of K (16 values) per MMA; the small products of the
+                            // stage first, so that they meet an accumulator of their own size
+                            if (Sh::LO) {
+    #pragma unroll
+                                for (int s = 0; s < ks; s++) {
+                                    tc::mma_f16(d, tc::desc_sw128(ah + 32 * s), tc::desc_sw128(bl + 32 * s), idesc, (kc | s) != 0);
+                                    tc::mma_f16(d, tc::desc_sw128(al + 32 * s), tc::desc_sw128(bh + 32 * s), idesc, 1u);
+                                }
+                            }
+    #pragma unroll
+                            for (int s = 0; s < ks; s++)
+                                tc::mma_f16(d, tc::desc_sw128(ah + 32 * s), tc::desc_sw128(bh + 32 * s), idesc,
+                                            Sh::LO || (kc | s) != 0);
+                            tc::mma_commit(aempty0 + 8 * sa);
+                            if (!Gh::UNI) tc::mma_commit(bempty0 + 8 * sb);
+                        }
+                        if (!failed) tc::mma_commit(rfull0 + 8 * r);
+                    }
+                    if (failed) atomicOr(prm.status, ST_TIMEOUT);
+                    tc::mma_commit(done);  // always: the deallocation waits on it
+                }
             }
         }
         tc::fence_before_sync();
@@ -694,128 +817,161 @@ __global__ void __launch_bounds__(KM2LTcg<N, MODE, true>::BS, KM2LTcg<N, MODE, t
     k.run(blockIdx.x, gridDim.x);
 }
 
-// Levels lmin..lmax of the grid charges, remapped from the padded layout (P =
-// H + 2 per axis) into the operand layout (tc_level_extent per axis, zeros
-// outside) and split into hi / lo parts.  One element = one (cell, b) of the
-// operand layout.
-struct SplitLevels {
-    int lmin, lmax;
-    long long src[FMM_MAXDEPTH + 2];  // first value of level l in the padded layout
-    long long dst[FMM_MAXDEPTH + 2];  // first cell of level l in the operand layout
-    long long cst[FMM_MAXDEPTH + 2];  // first visited cell of level l (from lmin; see split_cell)
-};
-__device__ __forceinline__ bool split_source(const SplitLevels &L, int64_t c, int &l, int64_t &src_cell) {
-    l = L.lmin;
-    while (l < L.lmax && c >= L.dst[l + 1]) l++;
-    const int r = (int)(c - L.dst[l]);  // < 8 * 130^3
-    const int Pt = (int)tc_level_extent(l), P = (1 << (l - 1)) + 2;
-    if (Pt == P) {  // levels with at least 8 coarse cells per axis: same layout
-        src_cell = r;
-        return true;
-    }
-    const int x = r % Pt, y = (r / Pt) % Pt, z = (r / (Pt * Pt)) % Pt, par = r / (Pt * Pt * Pt);
-    if (x >= P || y >= P || z >= P) return false;
-    src_cell = ((int64_t)(par * P + z) * P + y) * P + x;
-    return true;
-}
-
-// TF32: hi = x with the 13 low mantissa bits cleared (exact in TF32), lo = x - hi;
-// with `nearest` (the 1-pass form, which has no lo term) hi is x rounded to the
-// nearest TF32 value (ties away from zero) instead of truncated.  One thread per
-// 4 consecutive values of a cell (p3s % 32 == 0).
-// Visited cell k -> level l, operand cell c and padded-layout cell src_cell;
-// false: c lies outside the padded layout (written as zeros).  Levels below
-// lpad visit the padded layout's cells only (no box copy reads the rest of
-// their operand layout); the others every operand cell.
-__device__ __forceinline__ bool split_cell(const SplitLevels &L, int lpad, int64_t k, int &l, int64_t &c,
-                                           int64_t &src_cell) {
-    l = L.lmin;
-    while (l < L.lmax && k >= L.cst[l + 1]) l++;
-    const int64_t r = k - L.cst[l];
-    if (l < lpad) {
-        const int Pt = (int)tc_level_extent(l), P = (1 << (l - 1)) + 2;
-        const int x = (int)(r % P), y = (int)((r / P) % P), z = (int)((r / (P * P)) % P), par = (int)(r / (P * P * P));
-        c = L.dst[l] + ((int64_t)(par * Pt + z) * Pt + y) * Pt + x;
-        src_cell = r;
-        return true;
-    }
-    c = L.dst[l] + r;
-    int l2;
-    return split_source(L, c, l2, src_cell);
-}
-
-struct KSplitTf32 {
-    static constexpr int BS = 0, MINB = 0;
-    const float *__restrict__ phi;
-    SplitLevels L;
-    float *__restrict__ hi;
-    float *__restrict__ lo;
-    int p3;
-    int p3s;
-    int nearest;
-    int lpad;  // levels below lpad: cells outside the padded layout are not visited (no box reads them)
+// The partials of the levels whose offsets are split over blocks, added in
+// order of the offsets (every cell of those levels; cells without charges hold
+// no partials and their sums are never read).
+struct KTcReduce {
+    static constexpr int BS = 256, MINB = 0;
+    const float *__restrict__ part;
+    float *__restrict__ loc;
+    int nlev;
+    int parts[4];
+    long long first[5];  // prefix of the levels' values
+    long long part_off[4], part_stride[4], loc_off[4];
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
-        const int q4 = p3s / 4;
-        const int64_t n = L.cst[L.lmax + 1] * q4;
-        for (int64_t i = bid_ * (int64_t)blockDim.x + threadIdx.x; i < n;
-             i += (int64_t)nblk_ * blockDim.x) {
-            const int b0 = (int)(i % q4) * 4;
-            int l;
-            int64_t c, sc;
-            const bool in = split_cell(L, lpad, i / q4, l, c, sc);
-            const float *src = phi + L.src[l] + sc * p3;
-            float v[4], h[4], w[4];
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                v[j] = (in && b0 + j < p3) ? src[b0 + j] : 0.0f;
-                const uint32_t u = __float_as_uint(v[j]) + (nearest ? 0x1000u : 0u);
-                h[j] = __uint_as_float(u & 0xFFFFE000u);
-                w[j] = v[j] - h[j];
-            }
-            *reinterpret_cast<float4 *>(hi + c * p3s + b0) = make_float4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<float4 *>(lo + c * p3s + b0) = make_float4(w[0], w[1], w[2], w[3]);
+        for (int64_t i = (int64_t)bid_ * BS + threadIdx.x; i < first[nlev]; i += (int64_t)nblk_ * BS) {
+            int v = 0;
+            while (i >= first[v + 1]) v++;
+            const int64_t e = i - first[v];
+            const float *p = part + part_off[v] + e;
+            float h = 0.0f, w = 0.0f;
+            for (int k = 0; k < parts[v]; k++) part_add(h, w, p[k * part_stride[v]], k + 1 == parts[v]);
+            loc[loc_off[v] + e] = h;
         }
     }
 };
-__global__ void k_split_tf32(const __grid_constant__ KSplitTf32 k) {
+__global__ void __launch_bounds__(KTcReduce::BS) k_tc_reduce(const __grid_constant__ KTcReduce k) {
     k.run(blockIdx.x, gridDim.x);
 }
 
-// BF16: hi = bf16(x), lo = bf16(x - hi), both rounded to nearest even; cell
-// vectors of p3k values (zero padded, p3k % 64 == 0).  One thread per 4 values.
-struct KSplitBf16 {
-    static constexpr int BS = 0, MINB = 0;
-    const float *__restrict__ phi;
-    SplitLevels L;
-    __nv_bfloat16 *__restrict__ hi;
-    __nv_bfloat16 *__restrict__ lo;
+// Split of the grid charges into 16-bit parts, one warp per cell of the padded
+// layout (cells [c0, c1), all levels in one stretch).
+// F16: x s = hi + lo with hi = half(x s), lo = half(x s - hi), both rounded to
+// nearest, s the power of two that takes the cell's largest |x| into [2^14,
+// 2^15): 11 + 11 significant bits, and an absolute floor of 2^-25 against that
+// maximum, so every value keeps an error below 2^-24 of itself or 2^-39 of the
+// cell's largest.  The accumulated products are scaled back by the cell's
+// factor 1/(s TC_KSCALE) where they are added up, all exact powers of two.
+// BF16: hi = bf16(x), lo = bf16(x - hi), unscaled (the type has FP32's range).
+// qsc: per cell (total charge, factor).  Infinite or NaN grid charges stay so.
+template <int MODE>
+struct KSplit {
+    static constexpr int BS = 256, MINB = 0;
+    const float *__restrict__ phi;   // the cells' values from cell 0 of the layout
+    const float *__restrict__ qlev;
+    float2 *__restrict__ qsc;
+    char *__restrict__ op;
+    long long c0, c1;
     int p3;
-    int p3k;
-    int lpad;  // as KSplitTf32
+    int fc;     // whole stages (64 values) of a row
+    int tail;   // values of the last, shorter stage (0 or 32)
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
-        const int q4 = p3k / 4;
-        const int64_t n = L.cst[L.lmax + 1] * q4;
-        for (int64_t i = bid_ * (int64_t)blockDim.x + threadIdx.x; i < n;
-             i += (int64_t)nblk_ * blockDim.x) {
-            const int b0 = (int)(i % q4) * 4;
-            int l;
-            int64_t c, sc;
-            const bool in = split_cell(L, lpad, i / q4, l, c, sc);
-            const float *src = phi + L.src[l] + sc * p3;
-            __nv_bfloat16 h[4], w[4];
+        typedef typename std::conditional<MODE == TC_BF16X3, __nv_bfloat162, __half2>::type T2;
+        const int lane = threadIdx.x & 31;
+        const int row_bytes = 256 * fc + (tail ? 128 : 0);
+        for (int64_t c = c0 + ((bid_ * (int64_t)BS + threadIdx.x) >> 5); c < c1; c += ((int64_t)nblk_ * BS) >> 5) {
+            const float *src = phi + c * p3;
+            float2 v[4];
+            uint32_t m = 0;
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const float v = (in && b0 + j < p3) ? src[b0 + j] : 0.0f;
-                h[j] = __float2bfloat16_rn(v);
-                w[j] = __float2bfloat16_rn(v - __bfloat162float(h[j]));
+            for (int k = 0; k < 4; k++) {
+                const int b = 2 * lane + 64 * k;
+                v[k].x = b < p3 ? src[b] : 0.0f;
+                v[k].y = b + 1 < p3 ? src[b + 1] : 0.0f;
+                m = max(m, max(__float_as_uint(v[k].x) & 0x7FFFFFFFu, __float_as_uint(v[k].y) & 0x7FFFFFFFu));
             }
-            *reinterpret_cast<uint2 *>(hi + c * p3k + b0) = *reinterpret_cast<const uint2 *>(h);
-            *reinterpret_cast<uint2 *>(lo + c * p3k + b0) = *reinterpret_cast<const uint2 *>(w);
+            float s = 1.0f, inv = 1.0f;
+            if (MODE != TC_BF16X3) {
+                // biased exponent e of the largest: s = 2^(14 - (e - 127)), capped at 2^127
+                const int e = (int)(__reduce_max_sync(0xffffffffu, m) >> 23);
+                const int f = min(268 - e, 254);
+                s = __uint_as_float((uint32_t)f << 23);
+                // 2^(127 - f) / TC_KSCALE, subnormal for the smallest cells: two exact factors
+                inv = __uint_as_float((uint32_t)(254 - min(f, 253)) << 23) * (f > 253 ? 0.5f / TC_KSCALE : 1.0f / TC_KSCALE);
+            }
+            if (lane == 0) qsc[c] = make_float2(qlev[c], inv);
+            char *dst = op + c * row_bytes + 4 * lane;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const bool full = k < fc;
+                if (!full && !(k == fc && tail && lane < 16)) break;
+                T2 a, r;
+                const float x = v[k].x * s, y = v[k].y * s;
+                if constexpr (MODE == TC_BF16X3) {
+                    a = __floats2bfloat162_rn(x, y);
+                    const float2 f = __bfloat1622float2(a);
+                    r = __floats2bfloat162_rn(x - f.x, y - f.y);
+                } else {
+                    a = __floats2half2_rn(x, y);
+                    const float2 f = __half22float2(a);
+                    r = __floats2half2_rn(x - f.x, y - f.y);
+                }
+                *reinterpret_cast<T2 *>(dst + 256 * k) = a;
+                *reinterpret_cast<T2 *>(dst + 256 * k + (full ? 128 : 64)) = r;
+            }
         }
     }
 };
-__global__ void k_split_bf16(const __grid_constant__ KSplitBf16 k) {
+template <int MODE>
+__global__ void __launch_bounds__(KSplit<MODE>::BS) k_split(const __grid_constant__ KSplit<MODE> k) {
     k.run(blockIdx.x, gridDim.x);
+}
+
+// Kernel tables of a plan, K_o[a,b] of eq. (bilinear) at unit cells with its row
+// mean split off, computed in FP64: one warp per (offset, a).  KtT: Kt_o^T
+// [o][b][a] and Kbar [o][a] in the plan's type (SIMT contraction); row: the
+// row's chunks for the tensor cores (hi, lo as the operand copy's, scaled by
+// TC_KSCALE or in bfloat16), kbar_tc [o][p3s].  Offsets of adjacent cells stay
+// zero (the tables are cleared first).
+template <typename real>
+struct KTables {
+    double tau[FMM_MAXP];
+    int p, power, ncomp, bf16, p3s, fc, tail;
+    real *KtT, *Kbar;
+    char *row;       // nullptr: no tensor-core tables
+    float *kbar_tc;
+};
+__device__ __forceinline__ double table_value(int comp, int power, double dx, double dy, double dz) {
+    // comp 0: 1/r^power; comps 1..3: the components of its force kernel
+    const double r2 = dx * dx + dy * dy + dz * dz, r = sqrt(r2);
+    const double d = comp == 1 ? dx : comp == 2 ? dy : dz;
+    if (power == 2) return comp == 0 ? 1.0 / r2 : 2.0 * d / (r2 * r2);
+    return comp == 0 ? 1.0 / r : d / (r2 * r);
+}
+template <typename real>
+__global__ void __launch_bounds__(256) k_tables(const __grid_constant__ KTables<real> t) {
+    const int p = t.p, p3 = p * p * p, lane = threadIdx.x & 31;
+    const int a = blockIdx.y * 8 + (threadIdx.x >> 5), oc = blockIdx.x, c = oc / 343, oi = oc % 343;
+    const int ox = oi % 7 - 3, oy = (oi / 7) % 7 - 3, oz = oi / 49 - 3;
+    if (a >= p3 || (abs(ox) <= 1 && abs(oy) <= 1 && abs(oz) <= 1)) return;
+    const double ax = t.tau[a % p] - ox, ay = t.tau[(a / p) % p] - oy, az = t.tau[a / (p * p)] - oz;
+    auto value = [&](int b) {
+        return table_value(c, t.power, ax - t.tau[b % p], ay - t.tau[(b / p) % p], az - t.tau[b / (p * p)]);
+    };
+    double mean = 0.0;
+    for (int b = lane; b < p3; b += 32) mean += value(b);
+    for (int o = 16; o >= 1; o >>= 1) mean += __shfl_xor_sync(0xffffffffu, mean, o);
+    mean /= p3;
+    if (lane == 0) t.Kbar[(int64_t)oc * p3 + a] = (real)mean;
+    for (int b = lane; b < p3; b += 32) t.KtT[((int64_t)oc * p3 + b) * p3 + a] = (real)(value(b) - mean);
+    if (!t.row) return;
+    if (lane == 0) t.kbar_tc[oc * t.p3s + a] = (float)mean;
+    char *row = t.row + ((int64_t)oc * t.p3s + a) * (256 * t.fc + (t.tail ? 128 : 0));
+    for (int b = lane; b < p3; b += 32) {
+        const double v = value(b) - mean;
+        const bool full = b < 64 * t.fc;
+        char *h = row + (b / 64) * 256 + (b % 64) * 2, *w = h + (full ? 128 : 64);
+        if (t.bf16) {
+            const __nv_bfloat16 x = __float2bfloat16_rn((float)v);
+            *reinterpret_cast<__nv_bfloat16 *>(h) = x;
+            *reinterpret_cast<__nv_bfloat16 *>(w) = __float2bfloat16_rn((float)(v - (double)__bfloat162float(x)));
+        } else {
+            const double u = v * (double)TC_KSCALE;
+            const __half x = __float2half_rn((float)u);
+            *reinterpret_cast<__half *>(h) = x;
+            *reinterpret_cast<__half *>(w) = __float2half_rn((float)(u - (double)__half2float(x)));
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -835,49 +991,76 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 int tc_padded(int p3) { return (p3 + 31) / 32 * 32; }
-int tc_padded_k(int p3, int mode) {
-    return mode == FMM_TC_BF16X3 ? (p3 + 63) / 64 * 64 : tc_padded(p3);
-}
+// a cell vector's (and kernel row's) chunks: stages of 64 values (two chunks),
+// a rest of at most 32 values in one chunk
+static int tc_full(int p3) { return p3 % 64 == 0 || p3 % 64 > 32 ? (p3 + 63) / 64 : p3 / 64; }
+static int tc_tail(int p3) { return p3 > 64 * tc_full(p3) ? 32 : 0; }
+int tc_row_bytes(int p3) { return 256 * tc_full(p3) + (tc_tail(p3) ? 128 : 0); }
 
-// Grid-charge box map of level l (operand layout): dims (pk b, Pt x, Pt y, Pt z,
-// 8 parity), box (one 128-byte chunk of b, 8, 4, 4, 1); fp32 (pk = p3s) or bf16
-// (pk = p3k) elements.  Every box the kernel loads lies inside the map.
-static int encode_phi_map(CUtensorMap *m, const void *base, int l, int pk, bool bf16) {
+static CUtensorMapDataType op_type(int mode) {
+    return mode == FMM_TC_BF16X3 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+}
+static int encode(CUtensorMap *m, int mode, int rank, const void *base, const cuuint64_t *dims,
+                  const cuuint64_t *strides, const cuuint32_t *box) {
     auto enc = encode_fn();
     if (!enc) return FMM_ERR_CUDA;
-    const cuuint64_t es_b = bf16 ? 2 : 4;
-    const cuuint64_t P = (cuuint64_t)tc_level_extent(l), rb = (cuuint64_t)pk * es_b;
-    cuuint64_t dims[5] = {(cuuint64_t)pk, P, P, P, 8};
-    cuuint64_t strides[4] = {rb, rb * P, rb * P * P, rb * P * P * P};
-    cuuint32_t box[5] = {(cuuint32_t)(128 / es_b), 8, 4, 4, 1};
-    cuuint32_t es[5] = {1, 1, 1, 1, 1};
-    CUresult r = enc(m, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5,
-                     (void *)base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    CUresult r = enc(m, op_type(mode), rank, (void *)base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? FMM_OK : FMM_ERR_CUDA;
 }
 
-// Kernel-table map: dims (pk b, p3s a, 343 offsets), box (one 128-byte chunk of b,
-// p3s, 1); fp32 tables have pk = p3s, bf16 tables pk = p3k.
-int tc_encode_kernel_map(void *map, const void *base, int p3s, int pk, int mode) {
-    auto enc = encode_fn();
-    if (!enc) return FMM_ERR_CUDA;
-    const bool bf16 = mode == FMM_TC_BF16X3;
-    const cuuint64_t es_b = bf16 ? 2 : 4;
-    cuuint64_t dims[3] = {(cuuint64_t)pk, (cuuint64_t)p3s, 343};
-    cuuint64_t strides[2] = {(cuuint64_t)pk * es_b, (cuuint64_t)pk * p3s * es_b};
-    cuuint32_t box[3] = {(cuuint32_t)(128 / es_b), (cuuint32_t)p3s, 1};
-    cuuint32_t es[3] = {1, 1, 1};
-    CUresult r = enc((CUtensorMap *)map,
-                     bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
-                     (void *)base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? FMM_OK : FMM_ERR_CUDA;
+// Box map of level l of the operand copy: dims (row values, P x, P y, P z, 8
+// parity), box (one chunk, 8, 4, 4, 1).  Every box the kernel loads lies inside.
+static int encode_phi_map(CUtensorMap *m, const void *base, int l, int row_bytes, int mode) {
+    const cuuint64_t P = ((cuuint64_t)1 << (l - 1)) + 2, rb = (cuuint64_t)row_bytes;
+    const cuuint64_t dims[5] = {rb / 2, P, P, P, 8}, strides[4] = {rb, rb * P, rb * P * P, rb * P * P * P};
+    const cuuint32_t box[5] = {64, 8, 4, 4, 1};
+    return encode(m, mode, 5, base, dims, strides, box);
+}
+
+// Kernel-table map: dims (row values, p3s a, 343 offsets), box (one chunk, p3s, 1).
+int tc_encode_kernel_map(void *map, const void *base, int p3, int mode) {
+    const cuuint64_t rb = (cuuint64_t)tc_row_bytes(p3), p3s = (cuuint64_t)tc_padded(p3);
+    const cuuint64_t dims[3] = {rb / 2, p3s, 343}, strides[2] = {rb, rb * p3s};
+    const cuuint32_t box[3] = {64, (cuuint32_t)p3s, 1};
+    return encode((CUtensorMap *)map, mode, 3, base, dims, strides, box);
 }
 
 size_t tc_map_bytes() { return sizeof(CUtensorMap); }
+
+template <typename real>
+int build_tables(int p, double grid_scale, int power, int ncomp, int mode, real *KtT, real *Kbar, void *rows,
+                 float *kbar_tc) {
+    KTables<real> t;
+    memset(&t, 0, sizeof(t));
+    const int p3 = p * p * p;
+    // §2.1.2: the p-division points; §4.1's reduced arrangement
+    for (int i = 0; i < p; i++) t.tau[i] = 0.5 + grid_scale * ((double)i / (double)(p - 1) - 0.5);
+    t.p = p;
+    t.power = power;
+    t.ncomp = ncomp;
+    t.bf16 = mode == FMM_TC_BF16X3;
+    t.p3s = tc_padded(p3);
+    t.fc = tc_full(p3);
+    t.tail = tc_tail(p3);
+    t.KtT = KtT;
+    t.Kbar = Kbar;
+    t.row = (char *)rows;
+    t.kbar_tc = kbar_tc;
+    const size_t no = (size_t)343 * ncomp;
+    if (cudaMemset(KtT, 0, no * p3 * p3 * sizeof(real)) != cudaSuccess ||
+        cudaMemset(Kbar, 0, no * p3 * sizeof(real)) != cudaSuccess)
+        return FMM_ERR_CUDA;
+    if (rows && (cudaMemset(rows, 0, no * t.p3s * tc_row_bytes(p3)) != cudaSuccess ||
+                 cudaMemset(kbar_tc, 0, no * t.p3s * sizeof(float)) != cudaSuccess))
+        return FMM_ERR_CUDA;
+    k_tables<real><<<dim3((unsigned)no, (p3 + 7) / 8), 256>>>(t);
+    return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+}
+template int build_tables<float>(int, double, int, int, int, float *, float *, void *, float *);
+template int build_tables<double>(int, double, int, int, int, double *, double *, void *, float *);
 
 template <int N, int MODE>
 static int launch_tcg_kernel(const TcgParams &prm, int blocks, int comp, cudaStream_t st, Tracer &tr) {
@@ -925,43 +1108,25 @@ static int launch_tcg_mode(int p3s, const TcgParams &prm, int blocks, int comp, 
     }
 }
 
-int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const void *k_hi_map,
-                  const void *k_lo_map, const float *kbar, int lmin, int mode, int inject,
-                  float *loc, int spow, bool split, int comp, cudaStream_t st, Tracer &tr) {
-    const int depth = g.depth, p3 = g.p3, p3s = tc_padded(p3), pk = tc_padded_k(p3, mode);
-    const bool bf16 = mode == FMM_TC_BF16X3;
-    // the grid charges of levels lmin..depth in the operand layout, split into
-    // hi / lo parts (the bf16 parts are stored in the same buffers, pk <= 2 p3s)
-    SplitLevels SL;
-    memset(&SL, 0, sizeof(SL));
-    SL.lmin = lmin;
-    SL.lmax = depth;
-    for (int l = 0; l <= depth + 1; l++) {
-        SL.src[l] = l <= depth ? W.phi_level[l] : 0;
-        SL.dst[l] = tc_level_first(l);
-    }
-    // a batch whose small levels run as cross-system (gathered) tiles reads
-    // none of their padding
-    const int lpad = tr.rec ? tr.tc_lbig : 0;
-    SL.cst[lmin] = 0;
-    for (int l = lmin; l <= depth; l++) {
-        const int64_t P = ((int64_t)1 << (l - 1)) + 2;
-        SL.cst[l + 1] = SL.cst[l] + (l < lpad ? 8 * P * P * P : SL.dst[l + 1] - SL.dst[l]);
-    }
+template <int MODE>
+static void launch_split(const Ptrs<float> &P, int64_t c0, int64_t c1, int p3, int blocks, cudaStream_t st, Tracer &tr) {
+    launch_k(tr, FMM_TAG(S_SPLIT_TC, 0), k_split<MODE>,
+             KSplit<MODE>{P.phi, P.qlev, P.qsc, P.op, c0, c1, p3, tc_full(p3), tc_tail(p3)}, blocks, KSplit<MODE>::BS, 0,
+             st);
+}
+
+int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const void *k_map, const float *kbar,
+                  int lmin, int mode, int inject, float *loc, int spow, bool split, int comp, cudaStream_t st,
+                  Tracer &tr) {
+    const int depth = g.depth, p3 = g.p3, p3s = tc_padded(p3), rb = tc_row_bytes(p3);
     tr.begin(FMM_STAGE_M2L, st);
-    __nv_bfloat16 *hi16 = reinterpret_cast<__nv_bfloat16 *>(P.phihi);
-    __nv_bfloat16 *lo16 = reinterpret_cast<__nv_bfloat16 *>(P.philo);
     if (split) {
-        // grid-stride over the levels' (cell, 4 values); small systems take a
-        // small grid, so that other work keeps the SMs
-        const int64_t units = SL.cst[depth + 1] * ((bf16 ? pk : p3s) / 4);
-        const int nbs = (int)std::min<int64_t>(152 * 8, std::max<int64_t>(1, (units + 255) / 256));
-        if (bf16)
-            launch_k(tr, FMM_TAG(S_SPLIT_TC, 0), k_split_bf16, KSplitBf16{P.phi, SL, hi16, lo16, p3, pk, lpad}, nbs,
-                     256, 0, st);
-        else
-            launch_k(tr, FMM_TAG(S_SPLIT_TC, 0), k_split_tf32,
-                     KSplitTf32{P.phi, SL, P.phihi, P.philo, p3, p3s, mode == FMM_TC_TF32X1, lpad}, nbs, 256, 0, st);
+        // grid-stride over the cells, a warp each; small systems take a small
+        // grid, so that other work keeps the SMs
+        const int64_t c0 = W.q_level[lmin], c1 = W.q_level[depth + 1];
+        const int nbs = (int)std::min<int64_t>(152 * 8, std::max<int64_t>(1, (c1 - c0 + 7) / 8));
+        if (mode == FMM_TC_BF16X3) launch_split<TC_BF16X3>(P, c0, c1, p3, nbs, st, tr);
+        else launch_split<TC_F16X3>(P, c0, c1, p3, nbs, st, tr);
         tr.count();
     }
     // a batch whose small levels run as cross-system tiles: this system's own
@@ -986,7 +1151,8 @@ int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const 
     for (int s = 0; s < op.nseg; s++) {
         op.bfirst[s] = nb;
         nb += (int)((occ_seg_cells(lmin, s) + OCC_BLOCK - 1) / OCC_BLOCK);
-        blocks += (int)((occ_seg_cells(lmin, s) + TC_M - 1) / TC_M);  // tiles if every cell holds charges
+        // blocks if every cell holds charges
+        blocks += (int)((occ_seg_cells(lmin, s) + TC_M - 1) / TC_M) * tc_parts(lmin + s / 8, depth);
     }
     op.bfirst[op.nseg] = nb;
     op.nblk = nb;
@@ -998,59 +1164,67 @@ int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const 
     }
     TcgParams prm;
     memset(&prm, 0, sizeof(prm));
-    memcpy(&prm.k_hi, k_hi_map, sizeof(CUtensorMap));
-    memcpy(&prm.k_lo, k_lo_map, sizeof(CUtensorMap));
-    const size_t es = bf16 ? 2 : 4;
-    prm.op_hi = reinterpret_cast<const char *>(P.phihi);
-    prm.op_lo = reinterpret_cast<const char *>(P.philo);
-    prm.row_bytes = (int)((bf16 ? pk : p3s) * es);
+    memcpy(&prm.k, k_map, sizeof(CUtensorMap));
     prm.lmin = lmin;
     prm.depth = depth;
     prm.p3 = p3;
     prm.spow = spow;
     prm.nseg = op.nseg;
     prm.occ = P.occ;
-    for (int l = 0; l <= depth + 1; l++) prm.op_cell0[l] = tc_level_first(l);
-    for (int l = lmin; l <= depth; l++) {
+    prm.op = P.op;
+    int rc = FMM_OK;
+    KTcReduce red;
+    memset(&red, 0, sizeof(red));
+    for (int l = lmin; l <= depth && !rc; l++) {
         prm.loc_off[l] = W.loc_level[l];
         prm.q_off[l] = W.q_level[l];
-        {  // box maps of the operand layout
-            const int64_t cl = tc_level_first(l);
-            const void *bh = bf16 ? (const void *)(hi16 + cl * pk) : (const void *)(P.phihi + cl * p3s);
-            const void *bl = bf16 ? (const void *)(lo16 + cl * pk) : (const void *)(P.philo + cl * p3s);
-            int rc = encode_phi_map(&prm.phi_hi[l], bh, l, pk, bf16);
-            if (!rc) rc = encode_phi_map(&prm.phi_lo[l], bl, l, pk, bf16);
-            if (rc) return rc;
+        if (l >= 4) rc = encode_phi_map(&prm.phi[l], P.op + W.q_level[l] * rb, l, rb, mode);
+        if (tc_parts(l, depth) > 1) {
+            const int v = red.nlev++;
+            tc_part_place(l, p3, &prm.part_off[l], &prm.part_stride[l]);
+            red.parts[v] = tc_parts(l, depth);
+            red.first[v + 1] = red.first[v] + ((long long)p3 << (3 * l));
+            red.part_off[v] = prm.part_off[l];
+            red.part_stride[v] = prm.part_stride[l];
+            red.loc_off[v] = W.loc_level[l];
         }
     }
+    if (rc) return rc;
     prm.loc = loc;
-    prm.qlev = P.qlev;
+    prm.part = P.tc_part;
+    prm.qsc = P.qsc;
     prm.kbar = kbar;
     prm.status = &P.hdr->status;
     prm.inject_stall = inject == FMM_INJECT_TC_STALL;
-    prm.xsys = nullptr;
-    prm.xseg = nullptr;
-    int rc = mode == FMM_TC_BF16X3   ? launch_tcg_mode<TC_BF16X3>(p3s, prm, blocks, comp, st, tr)
-             : mode == FMM_TC_TF32X1 ? launch_tcg_mode<TC_TF32X1>(p3s, prm, blocks, comp, st, tr)
-                                     : launch_tcg_mode<TC_TF32X3>(p3s, prm, blocks, comp, st, tr);
+    rc = mode == FMM_TC_BF16X3  ? launch_tcg_mode<TC_BF16X3>(p3s, prm, blocks, comp, st, tr)
+         : mode == FMM_TC_F16X1 ? launch_tcg_mode<TC_F16X1>(p3s, prm, blocks, comp, st, tr)
+         : mode == FMM_TC_F16X3C ? launch_tcg_mode<TC_F16X3C>(p3s, prm, blocks, comp, st, tr)
+                                : launch_tcg_mode<TC_F16X3>(p3s, prm, blocks, comp, st, tr);
     tr.count();
+    if (!rc && red.nlev > 0) {
+        red.part = P.tc_part;
+        red.loc = loc;
+        const int nbr = (int)std::min<int64_t>(152 * 4, (red.first[red.nlev] + KTcReduce::BS - 1) / KTcReduce::BS);
+        launch_k(tr, FMM_TAG(S_TC_REDUCE, comp), k_tc_reduce, red, nbr, KTcReduce::BS, 0, st);
+        tr.count();
+    }
     tr.end();
     return rc;
 }
 
 int tc_cross_records(const std::vector<TcXSys> &sys, const std::vector<int> &depth, int ncomp, int lmin,
-                     int lmax, int p3, int mode, int spow0, const void *const *k_hi_maps,
-                     const void *const *k_lo_maps, const float *const *kbars, const WsLayout &W, int *status,
-                     void **dx, size_t *dx_bytes, std::vector<LaunchRec> &out) {
+                     int lmax, int p3, int mode, int spow0, const void *const *k_maps, const float *const *kbars,
+                     const WsLayout &W, const char *ws, size_t ws_bytes, int *status, void **dx, size_t *dx_bytes,
+                     std::vector<LaunchRec> &out) {
     const int ns = (int)depth.size();
-    const int p3s = tc_padded(p3), pk = tc_padded_k(p3, mode);
-    const bool bf16 = mode == FMM_TC_BF16X3;
+    const int p3s = tc_padded(p3);
     const int nseg = 8 * (lmax - lmin + 1);
-    if (lmax >= 5 || ns >= (1 << 19)) return FMM_ERR_UNSUPPORTED;  // coordinates and systems fit the entries
+    // coordinates and systems fit the list's entries, chunks of the workspace a gather's row index
+    if (lmax >= 5 || ns >= (1 << 19) || ws_bytes / 128 > INT32_MAX) return FMM_ERR_UNSUPPORTED;
     // the lists: every cell of every system with that level, system-major
     std::vector<int> cnt(nseg, 0), tiles(nseg + 1, 0), first(nseg, 0), list;
     for (int sg = 0; sg < nseg; sg++) {
-        const int l = lmin + sg / 8, par = sg & 7, H = 1 << (l - 1);
+        const int l = lmin + sg / 8, H = 1 << (l - 1);
         first[sg] = (int)list.size();
         for (int i = 0; i < ns; i++) {
             if (depth[i] < l) continue;
@@ -1060,7 +1234,6 @@ int tc_cross_records(const std::vector<TcXSys> &sys, const std::vector<int> &dep
         }
         cnt[sg] = (int)list.size() - first[sg];
         tiles[sg + 1] = tiles[sg] + (cnt[sg] + TC_M - 1) / TC_M;
-        (void)par;
     }
     // device buffer: the segment table and list, then the systems' table per component
     std::vector<int> seg;
@@ -1085,15 +1258,13 @@ int tc_cross_records(const std::vector<TcXSys> &sys, const std::vector<int> &dep
     for (int c = 0; c < ncomp; c++) {
         TcgParams prm;
         memset(&prm, 0, sizeof(prm));
-        memcpy(&prm.k_hi, k_hi_maps[c], sizeof(CUtensorMap));
-        memcpy(&prm.k_lo, k_lo_maps[c], sizeof(CUtensorMap));
-        prm.row_bytes = (int)((bf16 ? pk : p3s) * (bf16 ? 2 : 4));
+        memcpy(&prm.k, k_maps[c], sizeof(CUtensorMap));
+        prm.op = ws;
         prm.lmin = lmin;
         prm.depth = lmax;
         prm.p3 = p3;
         prm.spow = c == 0 ? spow0 : spow0 + 1;
         prm.nseg = nseg;
-        for (int l = 0; l <= lmax + 1; l++) prm.op_cell0[l] = tc_level_first(l);
         for (int l = lmin; l <= lmax; l++) {
             prm.loc_off[l] = W.loc_level[l];
             prm.q_off[l] = W.q_level[l];
@@ -1105,9 +1276,10 @@ int tc_cross_records(const std::vector<TcXSys> &sys, const std::vector<int> &dep
         Tracer t;
         std::vector<LaunchRec> one;
         t.rec = &one;
-        int rc = mode == FMM_TC_BF16X3   ? record_tcx_mode<TC_BF16X3>(p3s, prm, tiles[nseg], c, t)
-                 : mode == FMM_TC_TF32X1 ? record_tcx_mode<TC_TF32X1>(p3s, prm, tiles[nseg], c, t)
-                                         : record_tcx_mode<TC_TF32X3>(p3s, prm, tiles[nseg], c, t);
+        int rc = mode == FMM_TC_BF16X3  ? record_tcx_mode<TC_BF16X3>(p3s, prm, tiles[nseg], c, t)
+             : mode == FMM_TC_F16X1 ? record_tcx_mode<TC_F16X1>(p3s, prm, tiles[nseg], c, t)
+             : mode == FMM_TC_F16X3C ? record_tcx_mode<TC_F16X3C>(p3s, prm, tiles[nseg], c, t)
+                                    : record_tcx_mode<TC_F16X3>(p3s, prm, tiles[nseg], c, t);
         if (rc) return rc;
         out.push_back(std::move(one[0]));
     }
