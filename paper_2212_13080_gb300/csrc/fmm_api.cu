@@ -464,7 +464,7 @@ int eval_impl(fmm_plan_t P, int64_t n, const float *pos, const float *q, real *p
         cudaStreamWaitEvent(S.near, S.sorted, 0);
     }
     tr.near = S.near;
-    launch_p2p<real>(g, ptr, W, forces != nullptr, S.near, tr);
+    launch_p2p<real>(g, ptr, W, n, forces != nullptr, S.near, tr);
     tr.near = nullptr;
     if (!tr.rec) cudaEventRecord(S.near_done, S.near);
     // the far field runs on a high-priority stream when one is given, so that
@@ -505,7 +505,7 @@ int eval_impl(fmm_plan_t P, int64_t n, const float *pos, const float *q, real *p
     }
     if (!tr.rec) cudaStreamWaitEvent(st, S.near_done, 0);
     else record_marker(tr, FMM_TAG(S_JOIN_NEAR, 0));
-    launch_l2p<real>(g, C, ptr, W, forces != nullptr, st, tr);
+    launch_l2p<real>(g, C, ptr, W, n, forces != nullptr, st, tr);
     launch_unsplit<real>(g, ptr, W, (int)n, q, potential, energy, forces, nullptr, nullptr, false,
                          st, tr);
     launch_k(tr, FMM_TAG(S_MARK_VALID, 0), k_mark_valid, KMarkValid{ptr.hdr, eval_tag(P, n)}, 1, KMarkValid::BS, 0,
@@ -527,8 +527,8 @@ int backward_impl(fmm_plan_t P, int64_t n, const float *pos, const float *q, con
     tr.count();
     // the gradient of the energy: adjoint forces whatever the forward mode
     if (g.force_mode == FMM_FORCE_KERNEL) g.force_mode = FMM_FORCE_ADJOINT;
-    launch_p2p<real>(g, ptr, W, true, st, tr);
-    launch_l2p<real>(g, C, ptr, W, true, st, tr);
+    launch_p2p<real>(g, ptr, W, n, true, st, tr);
+    launch_l2p<real>(g, C, ptr, W, n, true, st, tr);
     if constexpr (std::is_same<real, float>::value)
         if (g.continuous && g.force_mode == FMM_FORCE_ADJOINT)
             launch_split_delta(g, P->cd, ptr, W, (int)n, pos, st, tr);

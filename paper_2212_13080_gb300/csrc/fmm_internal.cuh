@@ -412,13 +412,13 @@ int plan_min_workspace(const fmm_plan_s *plan, int64_t n, size_t *bytes);
 int static_workspace_address(void **out);
 
 // near field + far-field evaluation at the charges (kernels_p2p.cu)
-// near field: writes out_pt (assigns) and the reaction slots; far field at the
+// near field (of n particles): writes out_pt (assigns) and the reaction slots; far field at the
 // charges: adds them and the far field, stores the totals to out_e[perm[slot]]
 template <typename real>
-void launch_p2p(const Geom &g, const Ptrs<real> &P, const WsLayout &W, bool forces,
+void launch_p2p(const Geom &g, const Ptrs<real> &P, const WsLayout &W, int64_t n, bool forces,
                 cudaStream_t st, Tracer &tr);
 template <typename real>
-void launch_l2p(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, const WsLayout &W,
+void launch_l2p(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, const WsLayout &W, int64_t n,
                 bool forces, cudaStream_t st, Tracer &tr);
 
 }  // namespace fmm

@@ -2,13 +2,16 @@
 // cell and its 26 neighbours) and far field (§2.2 step 4 and the far-field force
 // at the end of §2.2).  Results in unit-box units, (phi, F_x, F_y, F_z) with phi
 // per unit charge and F with the charge.
-// The near-field kernel evaluates every pair of neighbouring cells once for
-// both partners (mutual form): it writes the target cell's own sums to
-// out_pt[slot] (sorted order) and the partners' reactions to one slot per
+// The near field evaluates every pair of neighbouring cells once for both
+// partners (mutual form; where light cells are told apart, their pairs are taken
+// one-sided): it writes the charges' own sums
+// to out_pt[slot] (sorted order) and the partners' reactions to one slot per
 // direction; the far-field kernel adds the slots in a fixed order and the far
 // field, and stores the total by emitted index, out_e[perm[slot]], where the
 // recombination reads each particle's charges in a row.  The near field needs
 // only the sorted charges and runs beside the far field.
+#include <algorithm>
+
 #include "fmm_internal.cuh"
 #include "lagrange.cuh"
 #include "launch.cuh"
@@ -29,6 +32,10 @@ __device__ __forceinline__ double4 make_vec4(double a, double b, double c, doubl
 // after it in (z, y, x) order.  Every unordered pair of neighbouring cells
 // {A, A + delta_d} is evaluated once, by the CTA of A.
 #define NF_SEGS 14
+// A cell with fewer than `light` charges is light (NF_LIGHT in single-precision
+// calls on sparse deep trees, see launch_p2p; else 1: none is): its pairs are
+// taken one-sided.
+#define NF_LIGHT 24
 __host__ __device__ __forceinline__ void nf_delta(int d, int &dx, int &dy, int &dz) {
     const int i = 13 + d;
     dx = i % 3 - 1;
@@ -86,6 +93,7 @@ struct KL2P {
     const typename Vec4<real>::T *__restrict__ out_pt;
     const int *__restrict__ perm;
     typename Vec4<real>::T *__restrict__ out_e;
+    int light;
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
         typedef typename Vec4<real>::T real4;
         constexpr int P3 = P * P * P;
@@ -109,14 +117,14 @@ struct KL2P {
             if (c == 0 && o < 3) org[j][o] = sf ? (real)(o == 0 ? cx : o == 1 ? cy : cz) / (real)(1 << depth) : real(0);
         }
         // slot d - 1 of a cell's charges was written by the cell (that cell -
-        // delta_d), d = 1..13, if it exists and holds charges
+        // delta_d), d = 1..13, if it exists and neither is light (or empty)
         if (threadIdx.x < nleaf * (NF_SEGS - 1)) {
             const int j = threadIdx.x / (NF_SEGS - 1), d = threadIdx.x % (NF_SEGS - 1);
             int cx, cy, cz, dx, dy, dz;
             morton_decode((uint32_t)(k0 + j), cx, cy, cz);
             nf_delta(d + 1, dx, dy, dz);
             const int64_t a = nf_cell(cx, cy, cz, -dx, -dy, -dz, 1 << depth, periodic);
-            slot_ok[j][d] = a >= 0 && leaf_start[a + 1] > leaf_start[a];
+            slot_ok[j][d] = a >= 0 && min(leaf_start[a + 1] - leaf_start[a], lst[j + 1] - lst[j]) >= light;
         }
         __syncthreads();
         const real S = (real)(1 << depth);
@@ -269,15 +277,16 @@ __global__ void __launch_bounds__(KL2P<real, P, FORCES, KF>::BS) k_l2p(const __g
 // Launch order of the near field: the occupied cells, heaviest first.  A
 // cell's work grows with its charge count T (T times its own and its 13
 // forward neighbours' charges), so the cells go in seven classes by T, the
-// largest first, and within a class in the order the atomics hand out (a
+// largest first (the last two are the light cells, where there are any), and within a class in the order the atomics hand out (a
 // cell's sums do not depend on when its CTA runs: the results are the same
 // bit for bit).  Clustered inputs put a few hundred cells with up to ~1000
 // charges each among many light ones; launched in cell order they would
 // start late and run alone at the end.  pord[0..6]: class sizes; pord[8..14]:
 // fill counters; pord[16..]: the cells (zeroed before the count).
 #define NF_NCLS 7
+#define NF_DENSE 5  // the first classes: dense cells
 __device__ __forceinline__ int nf_class(int T) {
-    return T >= 512 ? 0 : T >= 256 ? 1 : T >= 128 ? 2 : T >= 64 ? 3 : T >= 32 ? 4 : T >= 16 ? 5 : T > 0 ? 6 : -1;
+    return T >= 512 ? 0 : T >= 256 ? 1 : T >= 128 ? 2 : T >= 64 ? 3 : T >= NF_LIGHT ? 4 : T >= 8 ? 5 : T > 0 ? 6 : -1;
 }
 
 struct KNfOrderCount {
@@ -463,7 +472,8 @@ __device__ __forceinline__ void nf_targets2(const float4 *tpa, const float4 *tpb
     }
 }
 
-template <typename real, bool FORCES, int CK, int POW>
+// LT: light cells are told apart (single precision)
+template <typename real, bool FORCES, int CK, int POW, bool LT>
 struct KP2P {
     static constexpr int BS = NF_BS, MINB = sizeof(real) == 4 ? NF_MINB : 1;
     int depth;
@@ -495,6 +505,8 @@ struct KP2P {
         // seg_off: prefix of the 13 forward segments' sizes, then sentinels up to
         // index 16 for the 4-step search of a slot's segment
         __shared__ int seg_start[NF_SEGS], seg_off[NF_SEGS + 3];
+        __shared__ int lseg[2][LT ? 32 : 1], nlight;  // LT: the light neighbours
+        constexpr int light = LT ? NF_LIGHT : 1;
 
         // the cell of this CTA: the launch order's entry (occupied cells, heaviest
         // first), or the block index where there is no order (small grids)
@@ -502,12 +514,12 @@ struct KP2P {
         if (pord) {
             int nocc = 0;
 #pragma unroll
-            for (int k = 0; k < NF_NCLS; k++) nocc += pord[k];
+            for (int k = 0; k < NF_NCLS; k++) nocc += k < NF_DENSE || light == 1 ? pord[k] : 0;
             if ((int)bid_ >= nocc) return;
             key = (uint32_t)pord[16 + bid_];
         }
         const int t0 = leaf_start[key], T = leaf_start[key + 1] - t0;
-        if (T == 0) return;
+        if (T < light) return;
         const int S = 1 << depth;
         int cx, cy, cz;
         morton_decode(key, cx, cy, cz);
@@ -545,6 +557,7 @@ struct KP2P {
                 if (b >= 0) {
                     st = leaf_start[b];
                     cnt = leaf_start[b + 1] - st;
+                    if (cnt < light) cnt = 0;
                 }
                 seg_start[l] = st;
             }
@@ -556,6 +569,28 @@ struct KP2P {
             if (l == 0) seg_off[0] = 0;
             if (l < NF_SEGS - 1) seg_off[l + 1] = cnt;
             else if (l < NF_SEGS + 2) seg_off[l + 1] = 0x7fffffff;
+        } else if (LT && threadIdx.x < 64) {
+            // the light neighbours, on either side (index of the 3x3x3 block, x
+            // fastest), for the own phase: the second warp
+            const int l = threadIdx.x - 32;
+            int st = 0, cnt = 0;
+            if (l < 27 && l != 13) {
+                const int64_t b = nf_cell(cx, cy, cz, l % 3 - 1, (l / 3) % 3 - 1, l / 9 - 1, S, periodic);
+                if (b >= 0) {
+                    st = leaf_start[b];
+                    cnt = leaf_start[b + 1] - st;
+                    if (cnt >= light) cnt = 0;
+                }
+            }
+            int inc = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (l >= o) inc += v;
+            }
+            lseg[0][l] = st - (inc - cnt);  // slot of source f: lseg[0] + f
+            lseg[1][l] = inc - cnt;
+            if (l == 31) nlight = inc;
         }
         __syncthreads();
         const int Ns = seg_off[NF_SEGS - 1];
@@ -808,6 +843,47 @@ struct KP2P {
                     }
                 }
             }
+            // the light neighbours' charges, the same way (staged in
+            // tbuf, which the passes above no longer need)
+            if constexpr (LT) {
+                constexpr int LB = 256;
+                float4 *lpos = reinterpret_cast<float4 *>(&tbuf[0][0]);
+                int *lori = reinterpret_cast<int *>(lpos + LB);
+                for (int sb = 0; sb < nlight; sb += LB) {
+                    const int ns = min(LB, nlight - sb);
+                    __syncthreads();
+                    for (int i = threadIdx.x; i < ns; i += NF_BS) {
+                        int d = 0;  // the last segment that starts at or before the source
+#pragma unroll
+                        for (int b = 16; b >= 1; b >>= 1)
+                            if (lseg[1][d + b] <= sb + i) d += b;
+                        const int j = lseg[0][d] + sb + i;
+                        const float4 v = s_pt[j];
+                        lpos[i] = make_float4(v.x + (float)(d % 3 - 1), v.y + (float)((d / 3) % 3 - 1),
+                                              v.z + (float)(d / 9 - 1), v.w);
+                        lori[i] = s_origin[j];
+                    }
+                    __syncthreads();
+                    if (act) {
+#pragma unroll 4
+                        for (int j = warp; j < ns; j += NW) {
+                            const float4 sv = lpos[j];
+                            const float dx = tv.x - sv.x, dy = tv.y - sv.y, dz = tv.z - sv.z;
+                            const float r2 = dx * dx + dy * dy + dz * dz;
+                            float ri = rsqrt_pair<float>(r2);
+                            if (CK >= 1) ri = (lori[j] != to && (CK < 2 || r2 > 0.0f)) ? ri : 0.0f;
+                            const float pf = POW == 2 ? ri * ri : ri;
+                            pa += sv.w * pf;
+                            if (FORCES) {
+                                const float q3 = sv.w * (POW == 2 ? 2.0f * pf * pf : ri * ri * ri);
+                                xa += q3 * dx;
+                                ya += q3 * dy;
+                                za += q3 * dz;
+                            }
+                        }
+                    }
+                }
+            }
             wpart[warp][lane * 4 + 0] = pa;
             wpart[warp][lane * 4 + 1] = xa;
             wpart[warp][lane * 4 + 2] = ya;
@@ -838,22 +914,256 @@ struct KP2P {
         }
     }
 };
-template <typename real, bool FORCES, int CK, int POW>
-__global__ void __launch_bounds__(KP2P<real, FORCES, CK, POW>::BS, KP2P<real, FORCES, CK, POW>::MINB) k_p2p(const __grid_constant__ KP2P<real, FORCES, CK, POW> k) {
+template <typename real, bool FORCES, int CK, int POW, bool LT>
+__global__ void __launch_bounds__(KP2P<real, FORCES, CK, POW, LT>::BS, KP2P<real, FORCES, CK, POW, LT>::MINB) k_p2p(const __grid_constant__ KP2P<real, FORCES, CK, POW, LT> k) {
     k.run(blockIdx.x, gridDim.x);
 }
 
+// ---------------------------------------------------------------------------
+// near field of the light cells in single precision, one-sided: one warp per
+// cell, all charges of its 27 cells as sources.  Lane = (target, phase): T
+// targets, 32 / T phases that take every 32/T-th source pair; two sources per
+// packed FP32x2 instruction, broadcast from the warp's own staging buffer, the
+// next NEAR_CH sources in flight to registers meanwhile.  No block barriers, no
+// sums across lanes inside the loop, no reactions.
+//
+// Why not the mutual form: its 128-thread block per cell has 512 source places
+// for the 13 T sources and sums its targets across four warps; with T = 8 it
+// ran at a sixth of its rate at T = 64.  The one-sided step (two pairs) is 13
+// packed operations against 18 for two mutual pairs, which count double.
+// Water at 8 charges a cell (water2m): 1.13 ms against 2.04 for the mutual form
+// alone; which calls take it: nf_light.
+//
+// Sums: at most NEAR_CH / 2 additions in a row, the chunks' sums added with
+// compensation, the phases in order.
+// ---------------------------------------------------------------------------
+#define NEAR_CH 128   // sources staged at a time
+#define NEAR_BS 128   // four independent warps
+#ifndef NEAR_MINB
+#define NEAR_MINB 5
+#endif
+#define NEAR_PAIRS (NEAR_CH / 2 + 32)  // and padding that the last step of a phase may read
+
+template <bool FORCES, int CK, int POW>
+struct KNear {
+    static constexpr int BS = NEAR_BS, MINB = NEAR_MINB;
+    int depth;
+    int periodic;
+    int ncell;
+    const int *__restrict__ leaf_start;
+    const float4 *__restrict__ s_pt;
+    const int *__restrict__ s_origin;
+    float4 *__restrict__ out_pt;
+    const int *__restrict__ pord;       // launch order (its last classes), or null
+
+    // the cell's neighbour d (x fastest, 13 the cell itself): its first slot and count
+    __device__ __forceinline__ void neighbour(uint32_t key, int d, int &start, int &cnt) const {
+        // one axis of a Morton key is an integer whose carries skip the other axes' bits
+        const uint32_t full = 0x09249249u & ((1u << (3 * depth)) - 1u);
+        uint32_t nk = 0;
+        bool in = true;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const uint32_t m = full << a, k = key & m;
+            const int s = (a == 0 ? d % 3 : a == 1 ? (d / 3) % 3 : d / 9) - 1;
+            if (!periodic && ((s < 0 && k == 0u) || (s > 0 && k == m))) in = false;
+            nk |= (s == 0 ? k : s > 0 ? (k | ~m) + (1u << a) : k - (1u << a)) & m;
+        }
+        start = in ? leaf_start[nk] : 0;
+        cnt = in ? leaf_start[nk + 1] - start : 0;
+    }
+
+    // Sums of this lane's target over one staged chunk of npair source pairs, its
+    // phase of nph.  src: per pair (x0 x1 y0 y1), (z0 z1 q0 q1).  OWN: the cell's
+    // own charges (the target itself and coincident charges are skipped).
+    template <bool OWN>
+    __device__ __forceinline__ void chunk(const float4 *src, const int2 *sor, int npair, int ph, int nph, float2 tx,
+                                          float2 ty, float2 tz, int to, float (&tot)[4], float (&cmp)[4]) const {
+        float2 ap = make_float2(0.0f, 0.0f), ax = ap, ay = ap, az = ap;
+        const int steps = (npair + nph - 1) / nph;
+        const float4 *p = src + 2 * ph;
+        const int2 *po = sor + ph;
+#pragma unroll 2
+        for (int s = 0; s < steps; s++, p += 2 * nph) {
+            const float4 A = p[0], B = p[1];
+            const float2 q = make_float2(B.z, B.w);
+            const float2 dx = __fadd2_rn(tx, make_float2(A.x, A.y)), dy = __fadd2_rn(ty, make_float2(A.z, A.w)),
+                         dz = __fadd2_rn(tz, make_float2(B.x, B.y));
+            const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+            float2 ri = make_float2(rsqrt_pair<float>(r2.x), rsqrt_pair<float>(r2.y));
+            if (OWN || CK >= 1) {
+                const int2 o = *po;
+                po += nph;
+                ri.x = (o.x != to && (!(OWN || CK >= 2) || r2.x > 0.0f)) ? ri.x : 0.0f;
+                ri.y = (o.y != to && (!(OWN || CK >= 2) || r2.y > 0.0f)) ? ri.y : 0.0f;
+            }
+            const float2 ri2 = __fmul2_rn(ri, ri);
+            const float2 pf = POW == 2 ? ri2 : ri;  // the pair function
+            const float2 qp = __fmul2_rn(q, pf);
+            ap = __fadd2_rn(ap, qp);
+            if (FORCES) {  // |force| / (q q' r): r^-3, or 2 r^-4
+                const float2 f = POW == 2 ? __fmul2_rn(__fadd2_rn(qp, qp), ri2) : __fmul2_rn(qp, ri2);
+                ax = __ffma2_rn(f, dx, ax);
+                ay = __ffma2_rn(f, dy, ay);
+                az = __ffma2_rn(f, dz, az);
+            }
+        }
+        const float v[4] = {ap.x + ap.y, ax.x + ax.y, ay.x + ay.y, az.x + az.y};
+#pragma unroll
+        for (int c = 0; c < (FORCES ? 4 : 1); c++) {
+            const float y = v[c] - cmp[c], t = tot[c] + y;
+            cmp[c] = (t - tot[c]) - y;
+            tot[c] = t;
+        }
+    }
+
+    __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
+        __shared__ float4 s_src[NEAR_BS / 32][2 * NEAR_PAIRS];
+        __shared__ int2 s_or[NEAR_BS / 32][NEAR_PAIRS];
+        __shared__ int s_seg[NEAR_BS / 32][2][32];
+        const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+        const int w = bid_ * (NEAR_BS / 32) + wl;
+        uint32_t key = (uint32_t)w;
+        if (pord) {
+            int first = 0, nlight = 0;
+#pragma unroll
+            for (int k = 0; k < NF_NCLS; k++) (k < NF_DENSE ? first : nlight) += pord[k];
+            if (w >= nlight) return;
+            key = (uint32_t)pord[16 + first + w];
+        } else if (w >= ncell) {
+            return;
+        }
+        const int t0 = leaf_start[key], T = leaf_start[key + 1] - t0;
+        if (T == 0 || T >= NF_LIGHT) return;
+        float4 *src = s_src[wl];
+        int2 *sor = s_or[wl];
+        int *seg0 = s_seg[wl][0], *pre = s_seg[wl][1];
+        // the 26 neighbours: first slots and the prefix of their counts
+        int Ns;
+        {
+            int st = 0, cnt = 0;
+            if (lane < 27 && lane != 13) neighbour(key, lane, st, cnt);
+            int inc = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += v;
+            }
+            Ns = __shfl_sync(0xffffffffu, inc, 31);
+            seg0[lane] = st - (inc - cnt);  // slot of source f of this segment: seg0 + f
+            pre[lane] = inc - cnt;          // first source of the segment (lanes 27..31: Ns)
+        }
+        const float S = (float)(1 << depth), far = 4.0f * S + 16.0f;
+        const float Sp = POW == 2 ? S * S : S;  // unit-box scale of the pair function
+        for (int i = NEAR_CH / 2 + lane; i < NEAR_PAIRS; i += 32) {  // the padding: no charge, far away
+            src[2 * i] = make_float4(far, far, far, far);
+            src[2 * i + 1] = make_float4(far, far, 0.0f, 0.0f);
+            sor[i] = make_int2(-1, -1);
+        }
+        __syncwarp();
+        constexpr int NL = NEAR_CH / 32;
+        float4 rv[NL];
+        int ro[NL];
+        // sources f0 + lane + 32 k into registers (own: the cell's charges; else the
+        // neighbours', shifted into the cell's frame), coordinates negated
+        auto load = [&](int f0, int n, bool own) {
+#pragma unroll
+            for (int k = 0; k < NL; k++) {
+                const int f = f0 + lane + 32 * k;
+                rv[k] = make_float4(far, far, far, 0.0f);
+                ro[k] = -1;
+                if (f < n) {
+                    int j = t0 + f, d = 13;
+                    if (!own) {
+                        d = 0;  // the last segment that starts at or before f
+#pragma unroll
+                        for (int b = 16; b >= 1; b >>= 1)
+                            if (pre[d + b] <= f) d += b;
+                        j = seg0[d] + f;
+                    }
+                    const float4 v = s_pt[j];
+                    rv[k] = make_float4(-(v.x + (float)(d % 3 - 1)), -(v.y + (float)((d / 3) % 3 - 1)),
+                                        -(v.z + (float)(d / 9 - 1)), v.w);
+                    if (own || CK >= 1) ro[k] = s_origin[j];
+                }
+            }
+        };
+        auto store = [&](bool origins) {
+            float *a = reinterpret_cast<float *>(src);
+            int *o = reinterpret_cast<int *>(sor);
+#pragma unroll
+            for (int k = 0; k < NL; k++) {
+                const int f = lane + 32 * k, e = 8 * (f >> 1) + (f & 1);
+                a[e] = rv[k].x;
+                a[e + 2] = rv[k].y;
+                a[e + 4] = rv[k].z;
+                a[e + 6] = rv[k].w;
+                if (origins) o[f] = ro[k];
+            }
+        };
+        // lanes past T nph repeat a phase and are not summed
+        const int nph = 32 / T, t = lane % T, ph = lane / T;
+        const float4 tv = s_pt[t0 + t];
+        const int to = s_origin[t0 + t];
+        const float2 tx = make_float2(tv.x, tv.x), ty = make_float2(tv.y, tv.y), tz = make_float2(tv.z, tv.z);
+        float tot[4] = {0.0f, 0.0f, 0.0f, 0.0f}, cmp[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        load(0, T, true);  // the cell itself: one chunk
+        store(true);
+        __syncwarp();
+        load(0, Ns, false);
+        chunk<true>(src, sor, (T + 1) >> 1, ph, nph, tx, ty, tz, to, tot, cmp);
+        for (int f0 = 0; f0 < Ns; f0 += NEAR_CH) {
+            __syncwarp();
+            store(CK >= 1);
+            __syncwarp();
+            if (f0 + NEAR_CH < Ns) load(f0 + NEAR_CH, Ns, false);
+            chunk<false>(src, sor, (min(NEAR_CH, Ns - f0) + 1) >> 1, ph, nph, tx, ty, tz, to, tot, cmp);
+        }
+        // the phases of a target, in order
+        float v[4];
+#pragma unroll
+        for (int c = 0; c < (FORCES ? 4 : 1); c++) {
+            v[c] = tot[c];
+            for (int k = 1; k < nph; k++) v[c] += __shfl_sync(0xffffffffu, tot[c], t + k * T);
+        }
+        if (lane < T) {
+            const float qs = tv.w * Sp * S;  // forces: S^(k+1)
+            out_pt[t0 + t] = FORCES ? make_float4(Sp * v[0], qs * v[1], qs * v[2], qs * v[3])
+                                    : make_float4(Sp * v[0], 0.0f, 0.0f, 0.0f);
+        }
+    }
+};
+static_assert(NF_LIGHT <= 33 && NF_LIGHT <= NEAR_CH, "a light cell: one target per lane, one chunk of its own charges");
+template <bool FORCES, int CK, int POW>
+__global__ void __launch_bounds__(KNear<FORCES, CK, POW>::BS, KNear<FORCES, CK, POW>::MINB)
+    k_near(const __grid_constant__ KNear<FORCES, CK, POW> k) {
+    k.run(blockIdx.x, gridDim.x);
+}
+
+// Cells that count as light, of a call with n particles.  One-sided pairs of
+// light cells pay where most cells are light and there are enough of them to
+// fill the chip with a warp each: trees of at least 64^3 cells with fewer than
+// 16 particles a cell (water2m, 8 a cell: near field 2.04 -> 1.13 ms; plummer8m,
+// 4 a cell: 20.3 -> 18.0 ms).  Elsewhere the mutual form takes every pair: with
+// 32 a cell (uniform1m) the split took 0.76 against 0.62 ms, with 8 a cell in
+// 16^3 cells 0.088 against 0.054 ms.
 template <typename real>
-void launch_l2p(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, const WsLayout &W,
+static int nf_light(const WsLayout &W, int64_t n) {
+    return sizeof(real) == 4 && W.ncell >= 262144 && n < 16 * W.ncell ? NF_LIGHT : 1;
+}
+
+template <typename real>
+void launch_l2p(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, const WsLayout &W, int64_t n,
                 bool forces, cudaStream_t st, Tracer &tr) {
     const int ncell = (int)W.ncell, depth = g.depth;
     const real *loc_leaf = P.loc + W.loc_level[depth];
     const bool kf = forces && g.force_mode == FMM_FORCE_KERNEL;
+    const int light = nf_light<real>(W, n);
     tr.begin(FMM_STAGE_L2P, st);
 #define L2P(PP, F, K)                                                                              \
     launch_k(tr, FMM_TAG(S_L2P, 0), k_l2p<real, PP, F, K>,                                          \
              KL2P<real, PP, F, K>{C, depth, g.periodic, ncell, g.shift_free, P.leaf_start, P.s_pt, loc_leaf, \
-                                  W.loc_comp, P.react, W.cap, P.out_pt, P.perm, P.out_e},            \
+                                  W.loc_comp, P.react, W.cap, P.out_pt, P.perm, P.out_e, light},     \
              (ncell + l2p_lpc<real, PP, K>() - 1) / l2p_lpc<real, PP, K>(), L2P_BS, 0, st)
     switch (g.p) {
 #define CASE(PP)                                                                                 \
@@ -871,9 +1181,9 @@ void launch_l2p(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, const W
 }
 
 template <typename real>
-void launch_p2p(const Geom &g, const Ptrs<real> &P, const WsLayout &W, bool forces,
+void launch_p2p(const Geom &g, const Ptrs<real> &P, const WsLayout &W, int64_t n, bool forces,
                 cudaStream_t st, Tracer &tr) {
-    const int ncell = (int)W.ncell, depth = g.depth;
+    const int ncell = (int)W.ncell, depth = g.depth, light = nf_light<real>(W, n);
     tr.begin(FMM_STAGE_P2P, st);
     // pairs to skip (see k_p2p): none in the plain form; charges of the same
     // particle in the continuous form; also coincident charges there with odd p
@@ -892,18 +1202,20 @@ void launch_p2p(const Geom &g, const Ptrs<real> &P, const WsLayout &W, bool forc
                  st);
         tr.count();
     }
+#define LAUNCH_LT(F, CK, POW, LT)                                                                  \
+    launch_k(tr, FMM_TAG(S_P2P, 0), k_p2p<real, F, CK, POW, LT>,                                    \
+             KP2P<real, F, CK, POW, LT>{depth, g.periodic, P.leaf_start, P.s_pt, P.s_origin, P.out_pt, P.react, W.cap, \
+                                        pord},                                                     \
+             ncell, NF_BS, 0, st)
+#define LAUNCH_POW(F, CK, POW)                                                                     \
+    do {                                                                                           \
+        if (sizeof(real) == 4 && light > 1) LAUNCH_LT(F, CK, POW, sizeof(real) == 4);              \
+        else LAUNCH_LT(F, CK, POW, false);                                                         \
+    } while (0)
 #define LAUNCH(F, CK)                                                                              \
     do {                                                                                           \
-        if (g.power == 2)                                                                          \
-            launch_k(tr, FMM_TAG(S_P2P, 0), k_p2p<real, F, CK, 2>,                                 \
-                     KP2P<real, F, CK, 2>{depth, g.periodic, P.leaf_start, P.s_pt, P.s_origin, P.out_pt, \
-                                          P.react, W.cap, pord},                                   \
-                     ncell, NF_BS, 0, st);                                                         \
-        else                                                                                       \
-            launch_k(tr, FMM_TAG(S_P2P, 0), k_p2p<real, F, CK, 1>,                                 \
-                     KP2P<real, F, CK, 1>{depth, g.periodic, P.leaf_start, P.s_pt, P.s_origin, P.out_pt, \
-                                          P.react, W.cap, pord},                                   \
-                     ncell, NF_BS, 0, st);                                                         \
+        if (g.power == 2) LAUNCH_POW(F, CK, 2);                                                    \
+        else LAUNCH_POW(F, CK, 1);                                                                 \
     } while (0)
     if (forces) {
         if (ck == 2) LAUNCH(true, 2);
@@ -915,17 +1227,49 @@ void launch_p2p(const Geom &g, const Ptrs<real> &P, const WsLayout &W, bool forc
         else LAUNCH(false, 0);
     }
 #undef LAUNCH
+#undef LAUNCH_POW
+#undef LAUNCH_LT
     tr.count();
+    if constexpr (sizeof(real) == 4) {
+        if (light == 1) {
+            tr.end();
+            return;
+        }
+        // the light cells: a warp each, as many as the list may hold
+        const int64_t nwarp = pord ? std::min<int64_t>(W.ncell, W.cap) : W.ncell;
+        const int nblk = (int)((nwarp + NEAR_BS / 32 - 1) / (NEAR_BS / 32));
+#define LAUNCH_POW(F, CK, POW)                                                                     \
+    launch_k(tr, FMM_TAG(S_NEAR_LIGHT, 0), k_near<F, CK, POW>,                                      \
+             KNear<F, CK, POW>{depth, g.periodic, ncell, P.leaf_start, P.s_pt, P.s_origin, P.out_pt, pord}, nblk, \
+             NEAR_BS, 0, st)
+#define LAUNCH(F, CK)                                                                              \
+    do {                                                                                           \
+        if (g.power == 2) LAUNCH_POW(F, CK, 2);                                                    \
+        else LAUNCH_POW(F, CK, 1);                                                                 \
+    } while (0)
+        if (forces) {
+            if (ck == 2) LAUNCH(true, 2);
+            else if (ck == 1) LAUNCH(true, 1);
+            else LAUNCH(true, 0);
+        } else {
+            if (ck == 2) LAUNCH(false, 2);
+            else if (ck == 1) LAUNCH(false, 1);
+            else LAUNCH(false, 0);
+        }
+#undef LAUNCH
+#undef LAUNCH_POW
+        tr.count();
+    }
     tr.end();
 }
 
 template void launch_l2p<float>(const Geom &, const Coef<float> &, const Ptrs<float> &,
-                                const WsLayout &, bool, cudaStream_t, Tracer &);
+                                const WsLayout &, int64_t, bool, cudaStream_t, Tracer &);
 template void launch_l2p<double>(const Geom &, const Coef<double> &, const Ptrs<double> &,
-                                 const WsLayout &, bool, cudaStream_t, Tracer &);
-template void launch_p2p<float>(const Geom &, const Ptrs<float> &, const WsLayout &, bool,
+                                 const WsLayout &, int64_t, bool, cudaStream_t, Tracer &);
+template void launch_p2p<float>(const Geom &, const Ptrs<float> &, const WsLayout &, int64_t, bool,
                                 cudaStream_t, Tracer &);
-template void launch_p2p<double>(const Geom &, const Ptrs<double> &, const WsLayout &, bool,
+template void launch_p2p<double>(const Geom &, const Ptrs<double> &, const WsLayout &, int64_t, bool,
                                  cudaStream_t, Tracer &);
 
 }  // namespace fmm

@@ -93,7 +93,7 @@ enum LaunchSite {
     S_P2M, S_HALO, S_M2M, S_LATTICE, S_M2L_SIMT, S_M2L_REDUCE,
     S_SPLIT_TC, S_OCC_COUNT, S_OCC_OFFSETS, S_OCC_SCATTER, S_M2L_TC,
     S_L2L, S_ZERO_SLIST, S_SPLIT_LIST, S_SPLIT_DELTA, S_L2P,
-    S_ZERO_ENERGY, S_UNSPLIT, S_ENERGY_FINAL, S_MARK_VALID, S_JOIN_NEAR, S_M2L_TCX, S_TC_REDUCE
+    S_ZERO_ENERGY, S_UNSPLIT, S_ENERGY_FINAL, S_MARK_VALID, S_JOIN_NEAR, S_M2L_TCX, S_TC_REDUCE, S_NEAR_LIGHT
 };
 
 template <class K>
