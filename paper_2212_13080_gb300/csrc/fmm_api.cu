@@ -333,7 +333,7 @@ WsLayout make_layout(const fmm_plan_t P, int64_t n) {
     const bool simt = !P->tc || P->opts.precision == FMM_PREC_FP32;
     size_t part = 0;
     for (int l = P->periodic ? 1 : 2; l <= P->depth && simt; l++) {
-        const int G = m2l_groups(l, p3);
+        const int G = m2l_groups(l, p3, P->fp64);
         if (G > 1) part = std::max(part, (size_t)G * ((size_t)1 << (3 * l)) * p3);
     }
     const size_t o0 = o;

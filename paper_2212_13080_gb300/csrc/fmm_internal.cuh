@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "../../include/fmm_gb300.h"
@@ -305,12 +306,26 @@ struct DevTables {
 
 // Offset groups of the SIMT contraction at level l: the 189 offsets of a
 // target tile are split over G CTAs when a level has too few tiles to fill
-// the GPU; each CTA writes a partial, summed afterwards in a fixed order.
-__host__ __device__ inline int m2l_groups(int l, int p3) {
-    int H = 1 << (l - 1), T = H < 4 ? H : 4;
-    int ctas = (H / T) * (H / T) * (H / T) * 8 * ((p3 + 63) / 64);
-    int G = (2 * 152 + ctas - 1) / ctas;
-    return G < 1 ? 1 : (G > 27 ? 27 : G);
+// the GPU; each CTA writes a partial, summed afterwards in a fixed order.  G is
+// the split with the shortest schedule, waves of `slots` resident CTAs (152 in
+// double precision, 304 in single) times offsets per CTA: 8 tiles in double
+// precision take 19 groups of 10 offsets in one wave, not 27 of 7 in two
+// (uniform23k, levels 2 and 3: 2.07 -> 0.87 ms with the tiles of few cells).
+inline int m2l_groups(int l, int p3, bool fp64) {
+    const int H = 1 << (l - 1), T = H < 4 ? H : 4, slots = fp64 ? 152 : 304;
+    const long long ctas = (long long)(H / T) * (H / T) * (H / T) * 8 * ((p3 + 63) / 64);
+    // no more than two CTAs per SM ask for (the partials take G level sizes)
+    const long long most = std::min<long long>(27, (304 + ctas - 1) / ctas);
+    int best = 1;
+    long long cost = -1;
+    for (int G = 1; G <= most; G++) {
+        const long long c = (ctas * G + slots - 1) / slots * ((189 + G - 1) / G);
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = G;
+        }
+    }
+    return best;
 }
 
 // tree / bookkeeping stage (kernels_tree.cu)

@@ -441,6 +441,12 @@ struct KM2LSimt {
         // per-offset partial sums (64 terms) are added into the totals with Kahan
         // compensation: one FP32 accumulator over all 189 x 64 terms would lose
         // ~sqrt(12096/2) ulps
+        // Tiles of at most 8 cells (T <= 2): a thread takes output a = threadIdx %
+        // 64 of cells threadIdx / 64 and + 4 (in acc[0][0..1]), so that no thread
+        // works on cells that the level does not have (8 of 64 at level 2, which took as
+        // long as level 3).
+        const bool small = T <= 2;
+        const int sa = threadIdx.x % M2L_T, sc = threadIdx.x / M2L_T;
         real acc[4][4], tot[4][4], cmp[4][4];
 #pragma unroll
         for (int i = 0; i < 4; i++)
@@ -508,6 +514,15 @@ struct KM2LSimt {
                         __syncthreads();
                         const int bn = min(M2L_T, p3 - b0);
                         int bb = 0;
+                        if (small) {
+                            const real *p0 = Ps + sc * M2L_PS, *p1 = p0 + 4 * M2L_PS;
+#pragma unroll 4
+                            for (; bb < bn; bb++) {
+                                const real kc = Ks[bb * M2L_T + sa];
+                                acc[0][0] += p0[bb] * kc;
+                                acc[0][1] += p1[bb] * kc;
+                            }
+                        }
                         for (; bb + 4 <= bn; bb += 4) {  // four values b of four cells per load
                             real pv[4][4];
 #pragma unroll
@@ -544,7 +559,8 @@ struct KM2LSimt {
                     for (int i = 0; i < 4; i++)
 #pragma unroll
                         for (int j = 0; j < 4; j++) {
-                            acc[i][j] += Kb[ag * 4 + j] * Qs[cg * 4 + i];
+                            if (small && (i > 0 || j > 1)) continue;
+                            acc[i][j] += small ? Kb[sa] * Qs[sc + 4 * j] : Kb[ag * 4 + j] * Qs[cg * 4 + i];
                             real y = acc[i][j] - cmp[i][j];
                             real t = tot[i][j] + y;
                             cmp[i][j] = (t - tot[i][j]) - y;
@@ -554,6 +570,13 @@ struct KM2LSimt {
         // ngroups > 1: loc_l is the partial buffer of this group (level layout)
         const real scale = (real)(1 << (l * spow));  // unit cells -> unit box: 2^l (1/r), 4^l (r/|r|^3)
         real *dst = loc_l + (int64_t)grp * ((int64_t)1 << (3 * l)) * p3;
+#pragma unroll
+        for (int j = 0; small && j < 2; j++) {
+            const int ci = sc + 4 * j, tx = ci % T, ty = (ci / T) % T, tz = ci / (T * T);
+            if (ci < ncell && a0 + sa < p3)
+                dst[loc_cell(l, 2 * (TX + tx) + bx, 2 * (TY + ty) + by, 2 * (TZ + tz) + bz) * p3 + a0 + sa] = scale * tot[0][j];
+        }
+        if (small) return;
 #pragma unroll
         for (int i = 0; i < 4; i++) {
             int ci = cg * 4 + i;
@@ -800,7 +823,7 @@ int launch_downward(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, con
             const int H = 1 << (l - 1);
             const int Tt = H < 4 ? H : 4;
             const int ntiles = (H / Tt) * (H / Tt) * (H / Tt);
-            const int G = m2l_groups(l, p3);
+            const int G = m2l_groups(l, p3, sizeof(real) == 8);
             real *dst = G > 1 ? P.m2l_part : loc_c + W.loc_level[l];
             tr.begin(FMM_STAGE_M2L, S.coarse);
             launch_k(tr, FMM_TAG(S_M2L_SIMT, 4 * l + c), k_m2l_simt<real>,

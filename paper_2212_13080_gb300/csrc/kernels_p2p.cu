@@ -336,14 +336,25 @@ __global__ void k_nf_order_fill(const __grid_constant__ KNfOrderFill k) {
 
 // 1/sqrt(r2): single precision uses the SFU reciprocal square root directly
 // (r2 is never subnormal here: it is 0 or a squared distance of FP32 charges
-// inside a few cells); double precision the correctly rounded form.
+// inside a few cells).  Double precision starts from the SFU value (relative
+// error below 2^-22) and takes one step of Halley's iteration for x^(-1/2),
+// y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2, which leaves 5 e^3/16 < 2^-64 before
+// rounding: five FP64 operations and two conversions in place of a square root
+// and a division, on the pipe that bounds the kernel (uniform23k near field:
+// 1.67 -> 1.48 ms, and 1.00 ms with empty source slots left out).  Squared distances outside the single-precision range (and 0)
+// take the quotient.
 template <typename real> __device__ __forceinline__ real rsqrt_pair(real x);
 template <> __device__ __forceinline__ float rsqrt_pair<float>(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-template <> __device__ __forceinline__ double rsqrt_pair<double>(double x) { return 1.0 / sqrt(x); }
+template <> __device__ __forceinline__ double rsqrt_pair<double>(double x) {
+    if (!(x >= 1e-30 && x <= 1e30)) return 1.0 / sqrt(x);
+    const double y = (double)rsqrt_pair<float>((float)x);
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
 
 // One (target, source) pair of the forward phase: target sums (p, x, y, z) in
 // a, the source's reaction in r.  FIRST assigns a instead of adding.  POW: the
@@ -677,11 +688,11 @@ struct KP2P {
                 // block); the previous pass's reads of wpart done
                 if (!one_block || pass > 0) __syncthreads();
                 int g0 = 0;
+                // the source slots that hold a source in this pass (the same for the
+                // whole CTA: slot k of thread t is source k NF_BS + t)
+                const int rem = Ns - pass * NF_BS * NF_KS;
+                const int kv = rem <= NF_BS ? 1 : (rem <= 2 * NF_BS ? 2 : (rem <= 3 * NF_BS && sizeof(real) == 8 ? 3 : NF_KS));
                 if constexpr (sizeof(real) == 4) {
-                    // the source slots that hold a source in this pass (the same for
-                    // the whole CTA: slot k of thread t is source k NF_BS + t)
-                    const int rem = Ns - pass * NF_BS * NF_KS;
-                    const int kv = rem <= NF_BS ? 1 : (rem <= 2 * NF_BS ? 2 : NF_KS);
 #define NF_GROUPS(KV)                                                                                           \
     do {                                                                                                        \
         for (; g0 + TG <= nt; g0 += TG)                                                                         \
@@ -706,8 +717,9 @@ struct KP2P {
                                                            rp[0], rx[0], ry[0], rz[0]);
 #pragma unroll
                         for (int k = 1; k < NF_KS; k++)
-                            nf_pair<real, FORCES, CK, false, POW>(tv, to, sx[k], sy[k], sz[k], sq[k], so[k],
-                                                                acc + u * NC, rp[k], rx[k], ry[k], rz[k]);
+                            if (k < kv)
+                                nf_pair<real, FORCES, CK, false, POW>(tv, to, sx[k], sy[k], sz[k], sq[k], so[k],
+                                                                      acc + u * NC, rp[k], rx[k], ry[k], rz[k]);
                     }
                     // transpose through shared memory: lane l sums value l over the lanes in order
                     __syncwarp();
@@ -730,8 +742,9 @@ struct KP2P {
                                                            rp[0], rx[0], ry[0], rz[0]);
 #pragma unroll
                         for (int k = 1; k < NF_KS; k++)
-                            nf_pair<real, FORCES, CK, false, POW>(tv, to, sx[k], sy[k], sz[k], sq[k], so[k],
-                                                                acc + u * NC, rp[k], rx[k], ry[k], rz[k]);
+                            if (k < kv)
+                                nf_pair<real, FORCES, CK, false, POW>(tv, to, sx[k], sy[k], sz[k], sq[k], so[k],
+                                                                      acc + u * NC, rp[k], rx[k], ry[k], rz[k]);
                     }
                     __syncwarp();
 #pragma unroll
