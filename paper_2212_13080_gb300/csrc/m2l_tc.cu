@@ -34,11 +34,11 @@
 // tensor cores contract Kt_o, the CUDA cores add Kbar_o[a] Q (Q = the source
 // cell's total charge).  Each offset accumulates into a fresh TMEM region (two
 // regions, alternating), small products first; the epilogue warps read it out
-// and add the offsets in FP32 registers with Kahan compensation.  Without the
-// compensation these 189 additions were the largest error of the form
-// (potentials of a depth-4 system at p = 6: 3.2e-7 against 2.8e-7 for FP32
-// multiply-adds; draining an accumulator more often than once an offset made
-// it worse).  A row's functional depends on its own A rows only, so it is the
+// and add the offsets in FP32 registers, for plain FP32 plans with Kahan
+// compensation: without it these 189 additions are the largest error of the
+// form (potentials of a depth-4 system at p = 6: 3.2e-7 against 2.8e-7 for FP32
+// multiply-adds), and it costs the reduced-precision plans more than they need
+// (uniform1m: 0.36 against 0.24 ms).  A row's functional depends on its own A rows only, so it is the
 // same, bit for bit, whichever tile form computes it.
 #include <algorithm>
 #include <cuda.h>
@@ -128,6 +128,13 @@ struct TcShape {
     static constexpr bool LO = MODE != TC_F16X1;        // lo parts loaded and used
     static constexpr bool SCALED = MODE != TC_BF16X3;   // operands scaled by powers of two
     static constexpr bool COMP = MODE == TC_F16X3C;     // compensated sum over the offsets
+    // Accumulators per offset, of KC / ND stages each.  The tensor cores' FP32
+    // additions do not round to nearest; with the compensated sum two
+    // accumulators of half the length keep plain FP32's errors at p = 5, 6
+    // (potentials of a clustered system at p = 6: 2.54e-7 against 2.81e-7 with one
+    // and 2.59e-7 for FP32 multiply-adds; contraction of plummer1m 6.2 -> 7.3 ms)
+    static constexpr int ND = COMP && N >= 128 ? 2 : 1;
+    static_assert(KC % ND == 0, "whole stages per accumulator");
     static constexpr int BBYTES = N * 128;              // one chunk of K_o
     // cross-system tiles keep the totals of their runs of offsets in TMEM, the
     // widest tile (two accumulators fill it) in the output
@@ -514,8 +521,10 @@ struct KM2LTcg {
                 const float kn = et < N ? prm.kbar[list_offset(par, in).oi * N + et] : 0.0f;
                 const float2 Q2 = make_float2(qs.x, qs.x), inv2 = make_float2(qs.y, qs.y);
                 const float *kb = kbs + (j & 1) * N + c0;
-                const int r = j & 1;
-                const uint32_t u = (uint32_t)(j >> 1) & 1u;
+#pragma unroll 1
+                for (int h = 0; h < Sh::ND; h++) {
+                const int r = (j * Sh::ND + h) & 1;
+                const uint32_t u = (uint32_t)((j * Sh::ND + h) >> 1) & 1u;
                 if (ok && !tc::mbar_wait(rfull0 + 8 * r, u, TC_WAIT_CYCLES)) {
                     if (lane == 0) tc_wait_failed(prm.status, 4, l, j);
                     ok = false;
@@ -533,7 +542,10 @@ struct KM2LTcg {
                         const float2 m0 = make_float2(m.x, m.y), m1 = make_float2(m.z, m.w);
                         float2 d0 = make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
                         float2 d1 = make_float2(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
-                        if (Sh::SCALED) {
+                        if (h > 0) {
+                            d0 = __fmul2_rn(d0, inv2);
+                            d1 = __fmul2_rn(d1, inv2);
+                        } else if (Sh::SCALED) {
                             d0 = __ffma2_rn(d0, inv2, __fmul2_rn(m0, Q2));
                             d1 = __ffma2_rn(d1, inv2, __fmul2_rn(m1, Q2));
                         } else {
@@ -552,6 +564,7 @@ struct KM2LTcg {
                 }
                 tc::fence_before_sync();
                 tc::mbar_arrive(rfree0 + 8 * r);
+                }
                 qs = qn;
                 if (et < N) kbs[((j + 1) & 1) * N + et] = kn;
                 asm volatile("bar.sync 1, %0;" ::"n"(32 * Sh::EPI) : "memory");
@@ -745,11 +758,11 @@ struct KM2LTcg {
                     }
                 }
             } else if (warp == Gh::WM) {
-                // ---- MMA issuer: the j-th offset of the block accumulates into TMEM region j & 1 ----
+                // ---- MMA issuer: the j-th accumulator of the block is TMEM region j & 1 ----
                 if (lane == 0) {
                     const uint32_t idesc = MODE == TC_BF16X3 ? tc::idesc_bf16(TC_M, N) : tc::idesc_f16(TC_M, N);
                     bool failed = false;
-                    for (int j = 0; j < i1 - i0 && !failed; j++) {
+                    for (int j = 0; j < (i1 - i0) * Sh::ND && !failed; j++) {
                         const int r = j & 1;
                         const uint32_t u = (uint32_t)(j >> 1) & 1u;
                         if (!tc::mbar_wait(rfree0 + 8 * r, u ^ 1u, TC_WAIT_CYCLES)) {
@@ -758,9 +771,9 @@ struct KM2LTcg {
                             break;
                         }
                         const uint32_t d = tmem + (uint32_t)(r * N);
-    #pragma unroll
-                        for (int kc = 0; kc < Sh::KC; kc++) {
-                            const int it = Sh::KC * j + kc;
+#pragma unroll
+                        for (int ks0 = 0; ks0 < Sh::KC / Sh::ND; ks0++) {
+                            const int it = Sh::KC / Sh::ND * j + ks0, kc = it % Sh::KC;
                             const int sa = it % Gh::SA, sb = it % Gh::SB;
                             if (!tc::mbar_wait(afull0 + 8 * sa, (uint32_t)(it / Gh::SA) & 1u, TC_WAIT_CYCLES) ||
                                 (!Gh::UNI && !tc::mbar_wait(bfull0 + 8 * sb, (uint32_t)(it / Gh::SB) & 1u, TC_WAIT_CYCLES))) {
@@ -771,22 +784,23 @@ struct KM2LTcg {
                             tc::fence_after_sync();
                             // the stage's hi and lo parts: two chunks, or the halves of a tail chunk
                             const bool full = kc < Sh::FC;
-                            const int ks = full ? 4 : 2;
                             const uint32_t ah = abase + sa * Gh::ASTAGE, al = ah + (full ? TC_ABYTES : 64);
                             const uint32_t bh = bbase + sb * Gh::BSTAGE, bl = bh + (full ? Sh::BBYTES : 64);
                             // 32 bytes of K (16 values) per MMA; the small products of the
                             // stage first, so that they meet an accumulator of their own size
                             if (Sh::LO) {
-    #pragma unroll
-                                for (int s = 0; s < ks; s++) {
-                                    tc::mma_f16(d, tc::desc_sw128(ah + 32 * s), tc::desc_sw128(bl + 32 * s), idesc, (kc | s) != 0);
+#pragma unroll
+                                for (int s = 0; s < 4; s++) {
+                                    if (s >= 2 && !full) break;
+                                    tc::mma_f16(d, tc::desc_sw128(ah + 32 * s), tc::desc_sw128(bl + 32 * s), idesc, (ks0 | s) != 0);
                                     tc::mma_f16(d, tc::desc_sw128(al + 32 * s), tc::desc_sw128(bh + 32 * s), idesc, 1u);
                                 }
                             }
-    #pragma unroll
-                            for (int s = 0; s < ks; s++)
-                                tc::mma_f16(d, tc::desc_sw128(ah + 32 * s), tc::desc_sw128(bh + 32 * s), idesc,
-                                            Sh::LO || (kc | s) != 0);
+#pragma unroll
+                            for (int s = 0; s < 4; s++)
+                                if (s < 2 || full)
+                                    tc::mma_f16(d, tc::desc_sw128(ah + 32 * s), tc::desc_sw128(bh + 32 * s), idesc,
+                                                Sh::LO || (ks0 | s) != 0);
                             tc::mma_commit(aempty0 + 8 * sa);
                             if (!Gh::UNI) tc::mma_commit(bempty0 + 8 * sb);
                         }
