@@ -987,6 +987,14 @@ struct Lane {
 const int kMaxLanes = 32;
 const int kLaneChoices[5] = {2, 4, 8, 16, 32};
 
+// the caller's arrays of a batched call, into the table its graph reads
+struct IoArrays {
+    void *p[IO_N];
+};
+__global__ void k_set_io(IoArrays a, void **io) {
+    if (threadIdx.x < IO_N) io[threadIdx.x] = a.p[threadIdx.x];
+}
+
 // OR of the status words of every system's workspace header
 __global__ void k_batch_status(const char *ws, const long long *off, int nsys, int *out) {
     __shared__ int acc;
@@ -1033,6 +1041,7 @@ struct fmm_batch_s {
     cudaEvent_t near_fork, near_join;
     char *d_tab;      // per merged launch: the systems' functors and block prefix
     size_t tab_bytes;
+    void **d_io;      // the caller's arrays of the call (IoPlace)
     void *d_x;        // cross-system contraction tiles: lists and the systems' table
     size_t x_bytes;
 };
@@ -1097,6 +1106,9 @@ int record_merged(fmm_batch_t B, const std::vector<int64_t> &n, const std::vecto
     for (int i = 0; i < ns; i++) {
         Tracer tr;
         tr.rec = &recs[i];
+        tr.io = B->d_io;
+        const void *base[IO_N] = {pos, q, potential, forces, energy};
+        for (int k = 0; k < IO_N; k++) tr.io_base[k] = base[k];
         tr.tc_lbig = tc_lmin ? x_lmax + 1 : 0;
         fmm_plan_t P = B->sys[i];
         const int64_t o = pofs[i];
@@ -1419,7 +1431,8 @@ int fmm_batch_create(fmm_batch_t *out, int nsys, const double *boxes, const int 
             cudaEventCreateWithFlags(&B->out_ev, cudaEventDisableTiming) != cudaSuccess ||
             cudaMalloc(&B->d_status, sizeof(int)) != cudaSuccess ||
             cudaMallocHost(&B->h_status, sizeof(int)) != cudaSuccess ||
-            cudaMalloc(&B->d_off, sizeof(long long) * nsys) != cudaSuccess)
+            cudaMalloc(&B->d_off, sizeof(long long) * nsys) != cudaSuccess ||
+            cudaMalloc(&B->d_io, sizeof(void *) * IO_N) != cudaSuccess)
             rc = FMM_ERR_OOM;
     }
     B->merged = true;
@@ -1466,6 +1479,7 @@ void fmm_batch_destroy(fmm_batch_t B) {
     if (B->d_off) cudaFree(B->d_off);
     if (B->d_tab) cudaFree(B->d_tab);
     if (B->d_x) cudaFree(B->d_x);
+    if (B->d_io) cudaFree(B->d_io);
     if (B->near) cudaStreamDestroy(B->near);
     if (B->near_fork) cudaEventDestroy(B->near_fork);
     if (B->near_join) cudaEventDestroy(B->near_join);
@@ -1514,12 +1528,17 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
     cudaEventRecord(B->in_ev, caller);
     cudaStreamWaitEvent(st, B->in_ev, 0);
     char *ws = (char *)workspace;
-    // what a captured graph is valid for: pointers and counts
-    std::vector<int64_t> key = {(int64_t)(uintptr_t)pos, (int64_t)(uintptr_t)q,
-                                (int64_t)(uintptr_t)potential, (int64_t)(uintptr_t)energy,
-                                (int64_t)(uintptr_t)forces, (int64_t)(uintptr_t)workspace};
+    // what a captured graph is valid for: the workspace, the counts and which
+    // outputs are wanted; a merged graph reads the arrays' addresses from a table
+    // (recording, capturing and instantiating again for every new set of arrays
+    // took 4.5 ms a call with 512 systems), the stream lanes hold them
+    IoArrays io = {{(void *)pos, (void *)q, potential, forces, energy}};
+    const bool by_table = B->merged && B->opts.precision != FMM_PREC_FP64;
+    std::vector<int64_t> key = {(int64_t)by_table, (int64_t)(uintptr_t)workspace};
+    for (int k = 0; k < IO_N; k++) key.push_back(by_table ? io.p[k] != nullptr : (int64_t)(uintptr_t)io.p[k]);
     key.insert(key.end(), n.begin(), n.end());
     cudaGetLastError();
+    if (by_table) k_set_io<<<1, 32, 0, st>>>(io, B->d_io);
     B->last_graph = true;
     std::vector<MergedLaunch> ml;
     if (!B->gexec || key != B->key || (!B->merged && B->lanes && B->glanes != B->lanes)) {
@@ -1633,7 +1652,7 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
 int fmm_batch_get_stats(fmm_batch_t B, fmm_batch_stats_t *out) {
     if (!B || !out) return FMM_ERR_ARG;
     memset(out, 0, sizeof(*out));
-    out->launches = B->launches;
+    out->launches = B->launches + (B->merged && B->opts.precision != FMM_PREC_FP64 ? 1 : 0);  // and the table's
     out->lanes = B->merged ? 0 : B->lanes;
     out->graph = B->last_graph ? 1 : 0;
     for (int c = 0; c < 8; c++) out->tune_ms[c] = B->tune_ms[c];

@@ -221,6 +221,10 @@ struct Tracer {
     // while recording a batch whose small levels run as cross-system tiles:
     // the first level of a system's own tensor-core contraction
     int tc_lbig = 0;
+    // while recording: the device table of the caller's arrays (launch.cuh) and
+    // the addresses that the recorded calls were given for them
+    void **io = nullptr;
+    const void *io_base[5] = {};
     bool on = false;
     cudaStream_t st = 0;
     int launches = 0;

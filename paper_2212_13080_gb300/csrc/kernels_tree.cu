@@ -156,8 +156,7 @@ struct KEmit {
     Geom g;
     Coef<real> C;
     int n;
-    const float *__restrict__ pos;
-    const float *__restrict__ q;
+    IoRef<const float> pos_, q_;
     const int *__restrict__ offset;
     uint32_t *__restrict__ e_key;
     typename Vec4<real>::T *__restrict__ e_pt;
@@ -167,6 +166,7 @@ struct KEmit {
     int *__restrict__ leaf_count;
     WsHeader *hdr;
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
+        const float *__restrict__ pos = pos_.get(), *__restrict__ q = q_.get();
         int st = 0;
         const int ne = offset ? hdr->n_eff : n;
         if (!offset && bid_ == 0 && threadIdx.x == 0) hdr->n_eff = n;
@@ -286,13 +286,14 @@ struct KSplitCount {
     static constexpr int BS = 0, MINB = 0;
     Geom g;
     int n;
-    const float *__restrict__ pos;
+    IoRef<const float> pos_;
     int *__restrict__ count;
     unsigned char *__restrict__ axes;
     int *__restrict__ bsum;
     WsHeader *hdr;
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
         __shared__ int sh[32];
+        const float *__restrict__ pos = pos_.get();
         const int base = bid_ * SCAN_TILE;
         int s = 0, st = 0;
         for (int k = 0; k < SCAN_IPT; k++) {
@@ -494,7 +495,7 @@ void launch_bin_emit(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, co
         // charges per particle, their offsets, the particle of every emitted charge
         const int nb = (n + SCAN_TILE - 1) / SCAN_TILE;
         launch_k(tr, FMM_TAG(S_SPLIT_COUNT, 0), k_split_count_reduce,
-                 KSplitCount{g, n, pos, P.count, P.axes, P.scan_tmp, P.hdr}, nb, SCAN_BS, 0, st);
+                 KSplitCount{g, n, io_ref(tr, IO_POS, pos), P.count, P.axes, P.scan_tmp, P.hdr}, nb, SCAN_BS, 0, st);
         launch_k(tr, FMM_TAG(S_SCAN_BLOCKS_E, 0), k_scan_blocks, KScanBlocks{P.scan_tmp, nb}, 1, 1024, 0, st);
         launch_k(tr, FMM_TAG(S_SCAN_APPLY_E, 0), k_scan_apply<true>,
                  KScanApply<true>{P.count, n, P.scan_tmp, P.offset, (int)W.cap, P.e_origin, P.hdr}, nb, SCAN_BS, 0,
@@ -507,7 +508,7 @@ void launch_bin_emit(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, co
     if (nbe < 1) nbe = 1;
     if (nbe > 152 * 64) nbe = 152 * 64;
     launch_k(tr, FMM_TAG(S_EMIT, 0), k_emit<real>,
-             KEmit<real>{g, C, n, pos, q, offset, P.e_key, P.e_pt, g.continuous ? P.e_wd : nullptr, P.e_origin,
+             KEmit<real>{g, C, n, io_ref(tr, IO_POS, pos), io_ref(tr, IO_Q, q), offset, P.e_key, P.e_pt, g.continuous ? P.e_wd : nullptr, P.e_origin,
                          P.e_rank, P.leaf_count, P.hdr},
              nbe, 256, 0, st);
     tr.count();
@@ -895,7 +896,7 @@ struct KSplitDelta {
     Geom g;
     Coef<double> Cd;
     int n;
-    const float *__restrict__ pos;
+    IoRef<const float> pos_;
     const int *__restrict__ count;
     const int *__restrict__ offset;
     const int *__restrict__ leaf_start;
@@ -916,6 +917,7 @@ struct KSplitDelta {
         __shared__ double gsd[SD_WARPS][SD_KMAX];          // plain near-source terms per charge (outer slab)
         __shared__ float msm[SD_WARPS][2][SD_NMOM];        // the moments (high, low) per slab and order
         __shared__ float csum[SD_WARPS][2][CH][32];        // per-lane compensated sums per charge (several axes)
+        const float *__restrict__ pos = pos_.get();
         const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
         const int S = g.S, p = g.p, p3 = g.p3;
         constexpr int PM = CH;  // p <= PM: the launch picks CH = 4, 6 or 8 by p
@@ -1394,15 +1396,14 @@ struct KUnsplit {
     Geom g;
     const WsHeader *hdr;
     int n;
-    const float *__restrict__ q;
+    IoRef<const float> q_;
     const int *__restrict__ offset;
     const int *__restrict__ count;
     const unsigned char *__restrict__ axes;
     const typename Vec4<real>::T *__restrict__ e_wd;
     const typename Vec4<real>::T *__restrict__ out_e;
     const float *__restrict__ delta;
-    real *__restrict__ potential;
-    real *__restrict__ forces;
+    IoRef<real> potential_, forces_;
     real *__restrict__ epart;
     const double *__restrict__ grad_energy;
     real *__restrict__ grad_q;
@@ -1412,6 +1413,8 @@ struct KUnsplit {
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
         // sphi = 1/L and sF = 1/L^2 come from the host: no FP64 arithmetic per thread
         __shared__ real sh[UNSPLIT_BS / 32][2];
+        const float *__restrict__ q = q_.get();
+        real *__restrict__ potential = potential_.get(), *__restrict__ forces = forces_.get();
         double gE = backward ? *grad_energy : 0.0;
         real ehi = 0, elo = 0;
         int i = bid_ * blockDim.x + threadIdx.x;
@@ -1509,7 +1512,7 @@ struct KEnergyFinal {
     static constexpr int BS = 0, MINB = 0;
     const real *__restrict__ epart;
     int nb;
-    double *energy;
+    IoRef<double> energy;
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
         __shared__ real sh[32][2];
         real h = 0, l = 0;
@@ -1527,7 +1530,7 @@ struct KEnergyFinal {
         if (threadIdx.x == 0) {
             real th = sh[0][0], tl = sh[0][1];
             for (int w = 1; w < (int)(blockDim.x >> 5); w++) pair_add(th, tl, sh[w][0], sh[w][1]);
-            *energy = 0.5 * ((double)th + (double)tl);
+            *energy.get() = 0.5 * ((double)th + (double)tl);
         }
     }
 };
@@ -1538,8 +1541,8 @@ __global__ void k_energy_final(const __grid_constant__ KEnergyFinal<real> k) {
 
 struct KZeroEnergy {
     static constexpr int BS = 0, MINB = 0;
-    double *energy;
-    __device__ __forceinline__ void run(const int bid_, const int nblk_) const {     *energy = 0.0;     }
+    IoRef<double> energy;
+    __device__ __forceinline__ void run(const int bid_, const int nblk_) const { *energy.get() = 0.0; }
 };
 __global__ void k_zero_energy(const __grid_constant__ KZeroEnergy k) {
     k.run(blockIdx.x, gridDim.x);
@@ -1552,7 +1555,7 @@ void launch_unsplit(const Geom &g, const Ptrs<real> &P, const WsLayout &W, int n
     tr.begin(FMM_STAGE_UNSPLIT, st);
     if (n == 0) {
         if (energy && !backward) {
-            launch_k(tr, FMM_TAG(S_ZERO_ENERGY, 0), k_zero_energy, KZeroEnergy{energy}, 1, 1, 0, st);
+            launch_k(tr, FMM_TAG(S_ZERO_ENERGY, 0), k_zero_energy, KZeroEnergy{io_ref(tr, IO_ENERGY, energy)}, 1, 1, 0, st);
             tr.count();
         }
         tr.end();
@@ -1563,17 +1566,17 @@ void launch_unsplit(const Geom &g, const Ptrs<real> &P, const WsLayout &W, int n
     // unit box -> box of edge L: potentials of 1/r^k scale by L^-k, forces by L^-(k+1)
     const double iL = 1.0 / g.L, sphi = g.power == 2 ? iL * iL : iL;
     launch_k(tr, FMM_TAG(S_UNSPLIT, 0), k_unsplit<real>,
-             KUnsplit<real>{g, P.hdr, n, q, g.continuous ? P.offset : nullptr, P.count, P.axes,
+             KUnsplit<real>{g, P.hdr, n, io_ref(tr, IO_Q, q), g.continuous ? P.offset : nullptr, P.count, P.axes,
                             g.continuous ? P.e_wd : nullptr, P.out_e,
                             (std::is_same<real, float>::value && g.continuous && g.force_mode == FMM_FORCE_ADJOINT)
                                 ? P.delta
                                 : nullptr,
-                            potential, forces, ep, grad_energy, grad_q, backward ? 1 : 0, (real)sphi,
+                            io_ref(tr, IO_POTENTIAL, potential), io_ref(tr, IO_FORCES, forces), ep, grad_energy, grad_q, backward ? 1 : 0, (real)sphi,
                             (real)(sphi * iL)},
              nb, UNSPLIT_BS, 0, st);
     tr.count();
     if (ep) {
-        launch_k(tr, FMM_TAG(S_ENERGY_FINAL, 0), k_energy_final<real>, KEnergyFinal<real>{ep, nb, energy}, 1, 1024,
+        launch_k(tr, FMM_TAG(S_ENERGY_FINAL, 0), k_energy_final<real>, KEnergyFinal<real>{ep, nb, io_ref(tr, IO_ENERGY, energy)}, 1, 1024,
                  0, st);
         tr.count();
     }
@@ -1596,7 +1599,7 @@ void launch_split_delta(const Geom &g, const Coef<double> &Cd, const Ptrs<float>
     const int ch = g.p <= 4 ? 4 : (g.p <= 6 ? 6 : 8);
 #define SD_LAUNCH(POW, CH)                                                                                  \
     launch_k(tr, FMM_TAG(S_SPLIT_DELTA, 0), k_split_delta<POW, CH>,                                             \
-             KSplitDelta<POW, CH>{g, Cd, n, pos, P.count, P.offset, P.leaf_start, P.s_pt, P.s_origin, leaf, P.delta, \
+             KSplitDelta<POW, CH>{g, Cd, n, io_ref(tr, IO_POS, pos), P.count, P.offset, P.leaf_start, P.s_pt, P.s_origin, leaf, P.delta, \
                                   P.slist},                                                                     \
              nb, 32 * SD_WARPS, 0, st)
     if (g.power == 2) {

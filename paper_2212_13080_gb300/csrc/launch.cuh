@@ -70,6 +70,26 @@ void kb_set_smem(size_t smem) {
         cudaFuncSetAttribute(kb_many_nolb<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
+// The caller's arrays of a batched evaluation, by place in the batch's device
+// table (written before every graph launch): the recorded functors hold the
+// place and an offset, so that a captured graph serves any arrays.
+enum IoPlace { IO_POS, IO_Q, IO_POTENTIAL, IO_FORCES, IO_ENERGY, IO_N };
+
+// An array of the caller: its address, or (recorded launches) an element offset
+// from the address in the table.
+template <typename T>
+struct IoRef {
+    T *p;
+    void *const *place;
+    int64_t off;
+    __device__ __forceinline__ T *get() const { return place ? reinterpret_cast<T *>(*place) + off : p; }
+};
+template <typename T>
+inline IoRef<T> io_ref(const Tracer &tr, int k, T *p) {
+    if (!tr.rec || !tr.io || !p) return IoRef<T>{p, nullptr, 0};
+    return IoRef<T>{nullptr, tr.io + k, p - reinterpret_cast<T *>(const_cast<void *>(tr.io_base[k]))};
+}
+
 // A launch of one system, recorded for merging: call sites (tag: site and
 // level or component) of different systems with equal tags merge.
 struct LaunchRec {
