@@ -207,10 +207,19 @@ __global__ void __launch_bounds__(KP2MWarp<real, P>::BS) k_p2m_warp(const __grid
 // §2.2 step 2, eq. (threethree): Phi_parent = sum_h (G_hx (x) G_hy (x) G_hz) Phi_child_h
 // in the factored order: the x shift summed over the two x siblings (4 arrays),
 // then the y shift summed over y (2 arrays), then z (1): 14 p^4 multiply-adds.
-// One CTA per parent; children of level l, parent of level l-1.  p is a
-// compile-time constant; the shift matrices are staged in shared memory.
+// SH_PAR parents per CTA; children of level l, parents of level l-1.
+//
+// Instructions bound the shifts, not memory: with one output per thread and step
+// every multiply-add took two shared loads and its share of index arithmetic
+// (about 6,000 warp instructions a parent at p = 6, 2.1 ms for a level of 1.8 GB
+// that takes 0.3 ms to move).  A thread takes a whole line instead: it loads
+// the 2p inputs of p outputs once, and the shift matrix is a compile-time index
+// into the kernel's parameters (constant-bank operands of the multiply-adds).
+// All levels, shift up / down: plummer8m 2.10 / 2.25 -> 0.76 / 1.14 ms, water2m
+// 0.42 / 0.29 -> 0.25 / 0.14 ms, plummer1m 0.33 / 0.32 -> 0.16 / 0.16 ms.
 // ---------------------------------------------------------------------------
 #define M2M_BS 128
+#define SH_PAR 4  // parents per CTA
 
 template <typename real, int P>
 struct KM2M {
@@ -226,78 +235,103 @@ struct KM2M {
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
         constexpr int P3 = P * P * P, PP = P * P;
         extern __shared__ unsigned char smraw[];
-        real *A = reinterpret_cast<real *>(smraw);  // [h][k][j][i]          8 p^3
-        real *B = A + 8 * P3;                       // [hz][hy][k][j][I]     4 p^3
-        real *D = B + 4 * P3;                       // [hz][k][J][I]         2 p^3
-        real *Gs = D + 2 * P3;                      // [h][J][i]             2 p^2
+        real *B = reinterpret_cast<real *>(smraw);  // per parent [hz][hy][k][j][I]  4 p^3
+        real *D = B + SH_PAR * 4 * P3;              // per parent [hz][k][J][I]      2 p^3
+        __shared__ int occ[SH_PAR];
+        __shared__ int64_t cell[SH_PAR];            // the parent's cell
         const int Hp = 1 << (l - 1);                // parents per axis
-        const int pid = bid_;
-        const int px = pid % Hp, py = (pid / Hp) % Hp, pz = pid / (Hp * Hp);
-        if (!cell_occupied(leaf_start, depth, l - 1, morton_encode(px, py, pz))) {
-            // no charges below this parent: its children's grid charges are all
-            // zero, and so are its own (what the sums below give)
-            real *out = phi_parent + phi_cell(l - 1, px, py, pz) * P3;
-            for (int o = threadIdx.x; o < P3; o += M2M_BS) out[o] = real(0);
-            if (threadIdx.x == 0) q_parent[phi_cell(l - 1, px, py, pz)] = real(0);
-            return;
-        }
-        for (int e = threadIdx.x; e < 2 * PP; e += M2M_BS) Gs[e] = C.G[e / PP][e % PP];
-        for (int e = threadIdx.x; e < 8 * P3; e += M2M_BS) {
-            const int h = e / P3, o = e % P3;
-            const int cx = 2 * px + (h & 1), cy = 2 * py + ((h >> 1) & 1), cz = 2 * pz + (h >> 2);
-            A[e] = phi_child[phi_cell(l, cx, cy, cz) * P3 + o];
+        const int p0 = bid_ * SH_PAR, np = min(SH_PAR, Hp * Hp * Hp - p0);
+        if ((int)threadIdx.x < np) {
+            const int pid = p0 + threadIdx.x, px = pid % Hp, py = (pid / Hp) % Hp, pz = pid / (Hp * Hp);
+            occ[threadIdx.x] = cell_occupied(leaf_start, depth, l - 1, morton_encode(px, py, pz));
+            cell[threadIdx.x] = phi_cell(l - 1, px, py, pz);
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < 4 * P3; e += M2M_BS) {
-            const int hyz = e / P3, o = e % P3, I = o % P, row = o - I;
-            real s = 0;
+        // x: the line (hz, hy, k, j) of both x siblings
+        for (int e = threadIdx.x; e < np * 4 * PP; e += M2M_BS) {
+            const int q = e / (4 * PP), hyz = (e / PP) % 4, kj = e % PP;
+            if (!occ[q]) continue;
+            const int pid = p0 + q, px = pid % Hp, py = (pid / Hp) % Hp, pz = pid / (Hp * Hp);
+            real in[2][P];
 #pragma unroll
             for (int hx = 0; hx < 2; hx++) {
-                const real *a = A + (hx + 2 * hyz) * P3 + row;
-                const real *g = Gs + hx * PP + I * P;
+                const real *src = phi_child + phi_cell(l, 2 * px + hx, 2 * py + (hyz & 1), 2 * pz + (hyz >> 1)) * P3 + kj * P;
 #pragma unroll
-                for (int i = 0; i < P; i++) s += g[i] * a[i];
+                for (int i = 0; i < P; i++) in[hx][i] = src[i];
             }
-            B[e] = s;
+            real *dst = B + q * 4 * P3 + hyz * P3 + kj * P;
+#pragma unroll
+            for (int I = 0; I < P; I++) {
+                real s = 0;
+#pragma unroll
+                for (int hx = 0; hx < 2; hx++)
+#pragma unroll
+                    for (int i = 0; i < P; i++) s += C.G[hx][I * P + i] * in[hx][i];
+                dst[I] = s;
+            }
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < 2 * P3; e += M2M_BS) {
-            const int hz = e / P3, o = e % P3, I = o % P, J = (o / P) % P, k = o / PP;
-            real s = 0;
+        // y: the line (hz, k, I)
+        for (int e = threadIdx.x; e < np * 2 * PP; e += M2M_BS) {
+            const int q = e / (2 * PP), hz = (e / PP) % 2, k = (e / P) % P, I = e % P;
+            if (!occ[q]) continue;
+            real in[2][P];
 #pragma unroll
             for (int hy = 0; hy < 2; hy++) {
-                const real *b = B + (hy + 2 * hz) * P3 + k * PP + I;
-                const real *g = Gs + hy * PP + J * P;
+                const real *src = B + q * 4 * P3 + (hy + 2 * hz) * P3 + k * PP + I;
 #pragma unroll
-                for (int j = 0; j < P; j++) s += g[j] * b[j * P];
+                for (int j = 0; j < P; j++) in[hy][j] = src[j * P];
             }
-            D[e] = s;
+            real *dst = D + q * 2 * P3 + hz * P3 + k * PP + I;
+#pragma unroll
+            for (int J = 0; J < P; J++) {
+                real s = 0;
+#pragma unroll
+                for (int hy = 0; hy < 2; hy++)
+#pragma unroll
+                    for (int j = 0; j < P; j++) s += C.G[hy][J * P + j] * in[hy][j];
+                dst[J * P] = s;
+            }
         }
         __syncthreads();
-        real *out = phi_parent + phi_cell(l - 1, px, py, pz) * P3;
-        for (int o = threadIdx.x; o < P3; o += M2M_BS) {
-            const int K = o / PP, IJ = o % PP;
-            real s = 0;
+        // z: the line (J, I); a parent without charges: its children's grid charges
+        // are all zero, and so are its own (what the sums would give)
+        for (int e = threadIdx.x; e < np * PP; e += M2M_BS) {
+            const int q = e / PP, JI = e % PP;
+            real *out = phi_parent + cell[q] * P3 + JI;
+            if (!occ[q]) {
 #pragma unroll
-            for (int hz = 0; hz < 2; hz++) {
-                const real *d = D + hz * P3 + IJ;
-                const real *g = Gs + hz * PP + K * P;
-#pragma unroll
-                for (int k = 0; k < P; k++) s += g[k] * d[k * PP];
+                for (int K = 0; K < P; K++) out[K * PP] = real(0);
+                continue;
             }
-            out[o] = s;
+            real in[2][P];
+#pragma unroll
+            for (int hz = 0; hz < 2; hz++)
+#pragma unroll
+                for (int k = 0; k < P; k++) in[hz][k] = D[q * 2 * P3 + hz * P3 + k * PP + JI];
+#pragma unroll
+            for (int K = 0; K < P; K++) {
+                real s = 0;
+#pragma unroll
+                for (int hz = 0; hz < 2; hz++)
+#pragma unroll
+                    for (int k = 0; k < P; k++) s += C.G[hz][K * P + k] * in[hz][k];
+                out[K * PP] = s;
+            }
         }
-        if (threadIdx.x < 32) {  // total charge: the eight children, tree order
+        if (threadIdx.x < 32) {  // total charge: the eight children, tree order; eight lanes a parent
+            const int q = threadIdx.x >> 3, h = threadIdx.x & 7;
             real v = 0;
-            if (threadIdx.x < 8) {
-                const int h = threadIdx.x;
+            if (q < np && occ[q]) {
+                const int pid = p0 + q, px = pid % Hp, py = (pid / Hp) % Hp, pz = pid / (Hp * Hp);
                 v = q_child[phi_cell(l, 2 * px + (h & 1), 2 * py + ((h >> 1) & 1), 2 * pz + (h >> 2))];
             }
             for (int m = 4; m >= 1; m >>= 1) v += __shfl_down_sync(0xffffffffu, v, m);
-            if (threadIdx.x == 0) q_parent[phi_cell(l - 1, px, py, pz)] = v;
+            if (q < np && h == 0) q_parent[cell[q]] = v;
         }
     }
 };
+static_assert(SH_PAR == 4, "eight lanes of a warp per parent");
 template <typename real, int P>
 __global__ void __launch_bounds__(KM2M<real, P>::BS) k_m2m(const __grid_constant__ KM2M<real, P> k) {
     k.run(blockIdx.x, gridDim.x);
@@ -305,7 +339,7 @@ __global__ void __launch_bounds__(KM2M<real, P>::BS) k_m2m(const __grid_constant
 
 template <typename real, int P>
 constexpr size_t m2m_smem() {
-    return sizeof(real) * (14 * P * P * P + 2 * P * P);
+    return sizeof(real) * SH_PAR * 6 * P * P * P;
 }
 
 // Halo of the padded Phi layout of level l >= 1: open form zeros; periodic form
@@ -646,8 +680,9 @@ __global__ void k_lattice(const __grid_constant__ KLattice<real> k) {
 // ---------------------------------------------------------------------------
 // §2.2 step 3: Psi_child(v) = Psi_parent(shift_{child->parent}(v)), i.e.
 // L_child_h += (G_hx (x) G_hy (x) G_hz)^T L_parent, as three passes (z, y, x).
-// One CTA per parent of level l-1; adds to the 8 children of level l (which
-// already hold their own interaction-list contributions).  Only cells that
+// SH_PAR parents of level l-1 per CTA, a line per thread as in the shift up; adds
+// to the 8 children of level l (which already hold their own interaction-list
+// contributions).  Only cells that
 // hold charges are formed: step 4 reads no other functional, and the children
 // of a cell without charges hold none either.
 // ---------------------------------------------------------------------------
@@ -663,55 +698,83 @@ struct KL2L {
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
         constexpr int P3 = P * P * P, PP = P * P;
         extern __shared__ unsigned char smraw[];
-        real *Lp = reinterpret_cast<real *>(smraw);  // [K][J][I]             p^3
-        real *A = Lp + P3;                           // [hz][k][J][I]       2 p^3
-        real *B = A + 2 * P3;                        // [hz][hy][k][j][I]   4 p^3
-        real *Gs = B + 4 * P3;                       // [h][J][i]           2 p^2
-        __shared__ unsigned occ_child;               // bit h: child h holds charges
-        const int Hp = 1 << (l - 1);  // parents per axis (level l-1)
-        const int pid = bid_;
-        const int px = pid % Hp, py = (pid / Hp) % Hp, pz = pid / (Hp * Hp);
-        const int64_t pkey = morton_encode(px, py, pz);
-        if (!cell_occupied(leaf_start, depth, l - 1, pkey)) return;
-        if (threadIdx.x < 32) {
-            const bool o = threadIdx.x < 8 && cell_occupied(leaf_start, depth, l, pkey * 8 + threadIdx.x);
+        real *A = reinterpret_cast<real *>(smraw);  // per parent [hz][k][J][I]      2 p^3
+        real *B = A + SH_PAR * 2 * P3;              // per parent [hz][hy][k][j][I]  4 p^3
+        __shared__ int occ[SH_PAR];                 // bit h: child h holds charges (0: nor does the parent)
+        const int Hp = 1 << (l - 1);                // parents per axis (level l-1)
+        const int p0 = bid_ * SH_PAR, np = min(SH_PAR, Hp * Hp * Hp - p0);
+        if (threadIdx.x < 32) {  // eight lanes a parent
+            const int q = threadIdx.x >> 3, h = threadIdx.x & 7;
+            bool o = false;
+            if (q < np) {
+                const int pid = p0 + q, px = pid % Hp, py = (pid / Hp) % Hp, pz = pid / (Hp * Hp);
+                o = cell_occupied(leaf_start, depth, l, (int64_t)morton_encode(px, py, pz) * 8 + h);
+            }
             const unsigned m = __ballot_sync(0xffffffffu, o);
-            if (threadIdx.x == 0) occ_child = m;
-        }
-        const real *src = loc_parent + loc_cell(l - 1, px, py, pz) * P3;
-        for (int e = threadIdx.x; e < 2 * PP; e += M2M_BS) Gs[e] = C.G[e / PP][e % PP];
-        for (int o = threadIdx.x; o < P3; o += M2M_BS) Lp[o] = src[o];
-        __syncthreads();
-        for (int e = threadIdx.x; e < 2 * P3; e += M2M_BS) {
-            const int hz = e / P3, o = e % P3, IJ = o % PP, k = o / PP;
-            const real *g = Gs + hz * PP + k;
-            real s = 0;
-#pragma unroll
-            for (int K = 0; K < P; K++) s += g[K * P] * Lp[K * PP + IJ];
-            A[e] = s;
+            if (h == 0) occ[q] = (m >> (8 * q)) & 255u;
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < 4 * P3; e += M2M_BS) {
-            const int hh = e / P3, o = e % P3, I = o % P, j = (o / P) % P, k = o / PP;
-            const int hz = hh >> 1, hy = hh & 1;
-            const real *g = Gs + hy * PP + j;
-            const real *a = A + hz * P3 + k * PP + I;
-            real s = 0;
+        if (!(occ[0] | occ[1] | occ[2] | occ[3])) return;
+        // z: the line (J, I) of the parent
+        for (int e = threadIdx.x; e < np * PP; e += M2M_BS) {
+            const int q = e / PP, JI = e % PP;
+            if (!occ[q]) continue;
+            const int pid = p0 + q, px = pid % Hp, py = (pid / Hp) % Hp, pz = pid / (Hp * Hp);
+            const real *src = loc_parent + loc_cell(l - 1, px, py, pz) * P3 + JI;
+            real in[P];
 #pragma unroll
-            for (int J = 0; J < P; J++) s += g[J * P] * a[J * P];
-            B[e] = s;
+            for (int K = 0; K < P; K++) in[K] = src[K * PP];
+#pragma unroll
+            for (int hz = 0; hz < 2; hz++)
+#pragma unroll
+                for (int k = 0; k < P; k++) {
+                    real s = 0;
+#pragma unroll
+                    for (int K = 0; K < P; K++) s += C.G[hz][K * P + k] * in[K];
+                    A[q * 2 * P3 + hz * P3 + k * PP + JI] = s;
+                }
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < 8 * P3; e += M2M_BS) {
-            const int h = e / P3, o = e % P3, i = o % P, row = o - i;
-            const int hx = h & 1, hy = (h >> 1) & 1, hz = h >> 2;
-            const real *g = Gs + hx * PP + i;
-            const real *b = B + ((hz << 1) | hy) * P3 + row;
-            real s = 0;
+        // y: the line (hz, k, I)
+        for (int e = threadIdx.x; e < np * 2 * PP; e += M2M_BS) {
+            const int q = e / (2 * PP), hz = (e / PP) % 2, k = (e / P) % P, I = e % P;
+            if (!occ[q]) continue;
+            const real *src = A + q * 2 * P3 + hz * P3 + k * PP + I;
+            real in[P];
 #pragma unroll
-            for (int I = 0; I < P; I++) s += g[I * P] * b[I];
-            const int cx = 2 * px + hx, cy = 2 * py + hy, cz = 2 * pz + hz;
-            if (occ_child & (1u << h)) loc_child[loc_cell(l, cx, cy, cz) * P3 + o] += s;
+            for (int J = 0; J < P; J++) in[J] = src[J * P];
+#pragma unroll
+            for (int hy = 0; hy < 2; hy++)
+#pragma unroll
+                for (int j = 0; j < P; j++) {
+                    real s = 0;
+#pragma unroll
+                    for (int J = 0; J < P; J++) s += C.G[hy][J * P + j] * in[J];
+                    B[q * 4 * P3 + (2 * hz + hy) * P3 + k * PP + j * P + I] = s;
+                }
+        }
+        __syncthreads();
+        // x: the line (hz, hy, k, j) into both x siblings
+        for (int e = threadIdx.x; e < np * 4 * PP; e += M2M_BS) {
+            const int q = e / (4 * PP), hzy = (e / PP) % 4, kj = e % PP;
+            const int o = occ[q] >> (2 * hzy);  // bit hx: child hx + 2 hy + 4 hz
+            if (!(o & 3)) continue;
+            const int pid = p0 + q, px = pid % Hp, py = (pid / Hp) % Hp, pz = pid / (Hp * Hp);
+            real in[P];
+#pragma unroll
+            for (int I = 0; I < P; I++) in[I] = B[q * 4 * P3 + hzy * P3 + kj * P + I];
+#pragma unroll
+            for (int hx = 0; hx < 2; hx++) {
+                if (!(o & (1 << hx))) continue;
+                real *dst = loc_child + loc_cell(l, 2 * px + hx, 2 * py + (hzy & 1), 2 * pz + (hzy >> 1)) * P3 + kj * P;
+#pragma unroll
+                for (int i = 0; i < P; i++) {
+                    real s = 0;
+#pragma unroll
+                    for (int I = 0; I < P; I++) s += C.G[hx][I * P + i] * in[I];
+                    dst[i] += s;
+                }
+            }
         }
     }
 };
@@ -722,7 +785,7 @@ __global__ void __launch_bounds__(KL2L<real, P>::BS) k_l2l(const __grid_constant
 
 template <typename real, int P>
 constexpr size_t l2l_smem() {
-    return sizeof(real) * (7 * P * P * P + 2 * P * P);
+    return sizeof(real) * SH_PAR * 6 * P * P * P;
 }
 
 // ---------------------------------------------------------------------------
@@ -770,7 +833,7 @@ void launch_upward(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, cons
         launch_k(tr, FMM_TAG(S_M2M, l), k_m2m<real, PP>,                                          \
                  KM2M<real, PP>{C, l, P.phi + W.phi_level[l], P.phi + W.phi_level[l - 1],          \
                                 P.qlev + W.q_level[l], P.qlev + W.q_level[l - 1], depth, P.leaf_start}, \
-                 nparent, M2M_BS, m2m_smem<real, PP>(), st);                                      \
+                 (nparent + SH_PAR - 1) / SH_PAR, M2M_BS, m2m_smem<real, PP>(), st);                                      \
         break;
                 CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
 #undef CASE
@@ -867,7 +930,7 @@ int launch_downward(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, con
     case PP:                                                                                       \
         launch_k(tr, FMM_TAG(S_L2L, 4 * l + c), k_l2l<real, PP>,                                  \
                  KL2L<real, PP>{C, l, depth, P.leaf_start, loc_c + W.loc_level[l - 1], loc_c + W.loc_level[l]}, \
-                 nparent, M2M_BS, l2l_smem<real, PP>(), st);                                      \
+                 (nparent + SH_PAR - 1) / SH_PAR, M2M_BS, l2l_smem<real, PP>(), st);                                      \
         break;
                 CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
 #undef CASE
