@@ -6,9 +6,10 @@ radius 0.1 of the unit box, centred, redrawn outside the box) with +-1
 charges summing to zero, open boundary, plain form, octree depth 7 (2,097,152
 finest cells, 61% of them empty), p = 6 (216 grid charges per cell).
 Default precision "tf32x3": every stage in FP32, the far-field contraction of
-every level on the tcgen05 tensor cores in 3-pass split TF32 (its parity with
-the FP64 oracle meets the FP32 tolerance).  The line also reports the plain
-FP32 form (SIMT contraction), the force-kernel form, the shift-free forms, and
+every level on the tcgen05 tensor cores in three passes over operands split in two
+halves (its parity with the FP64 oracle meets the FP32 tolerance).  The line
+also reports the plain FP32 form (the same operands, the sum over the offsets
+compensated), the force-kernel form, the shift-free forms, and
 shorter lines for BF16x3 and for the uniform (1,048,576 particles, continuous
 form, depth 5, p 4) and water-like (2,097,150 particles, periodic continuous
 form, depth 6, p 5) workloads.
@@ -48,8 +49,8 @@ FP64_NOMINAL_TFLOPS = 1.25  # GB300 FP64 (non-tensor), nominal
 # ran on a smaller case of the same distribution); reported as the
 # rooflines' traffic
 PROFILED_TRAFFIC = {("uniform1m", "tf32x3", "k_p2p"): 48267520 + 187352576,
-                    ("plummer8m", "tf32x3", "k_m2l_tcg"): 339113666816 + 960174080,
-                    ("plummer8m", "tf32x3", "k_p2p"): 353114368 + 1788425728}
+                    ("plummer8m", "tf32x3", "k_m2l_tcg"): 25352380928 + 942289152,
+                    ("plummer8m", "tf32x3", "k_p2p"): 207183616 + 1260335360}
 
 
 def _peaks():
@@ -499,23 +500,20 @@ def m2l_work(start, depth, periodic, p, precision):
                         else:
                             dense += int(np.prod([H - abs(v) for v in d]))
     p3 = p ** 3
-    n_pad = (p3 + 31) // 32 * 32
-    k_pad = (p3 + 63) // 64 * 64 if precision == "bf16x3" else n_pad
+    n_pad = k_pad = (p3 + 31) // 32 * 32
     passes = 1 if precision == "tf32x1" else 3
     return {"dense_pairs": dense, "occupied_pairs": both, "tiles": tiles,
             "algorithmic_flops": 2.0 * p3 * p3 * both, "dense_flops": 2.0 * p3 * p3 * dense,
             "executed_flops": 2.0 * tiles * 128 * 189 * n_pad * k_pad * passes}
 
 
-def tc_peak(precision, long_step):
-    """Dense tensor peak of the contraction's MMA kind (TF/s) and its source."""
+def tc_peak(long_step):
+    """Dense tensor peak of the contraction's MMA kind (kind::f16 in every
+    precision: the measured bf16 rate itself, TF/s) and its source."""
     hbm, bf16_burst, bf16_sust, kind = _peaks()
     ref = bf16_sust if long_step else bf16_burst
     which = "sustained" if long_step else "burst"
-    if precision == "bf16x3":  # kind::f16: the measured bf16 rate itself
-        return ref, "%s bf16 %s %.1f TF/s" % (kind, which, ref)
-    # kind::tf32: 1/2 of it (nominal 1.1 vs 2.25 PF/s)
-    return ref / 2, "%s bf16 %s %.1f TF/s x 1/2 (nominal tf32:bf16 ratio)" % (kind, which, ref)
+    return ref, "%s bf16 %s %.1f TF/s" % (kind, which, ref)
 
 
 class Run:
@@ -603,7 +601,7 @@ def rooflines(run, t_step, stage_ms, stage_iso):
     pairs = p2p_pairs(run.plan, w["depth"], w["periodic"])
     mw = m2l_work(start, w["depth"], w["periodic"], w["p"], run.precision)
     long_step = t_step >= 100.0
-    tc = run.precision in ("tf32x3", "tf32x1", "bf16x3")
+    tc = run.precision in ("tf32x3", "tf32x1", "bf16x3") or (run.precision == "fp32" and 3 <= w["p"] <= 6)
     out = {}
     p2p_flops = float(P2P_FLOPS_PER_PAIR) * pairs
     ach = p2p_flops / (stage_ms["p2p"] * 1e-3) / 1e12
@@ -611,13 +609,14 @@ def rooflines(run, t_step, stage_ms, stage_iso):
     out["p2p"] = {"kernel": "k_p2p", "bound": "alu", "achieved": ach_iso, "peak": FP32_ALU_PEAK_TFLOPS,
                   "unit": "TFLOP/s", "frac": ach_iso / FP32_ALU_PEAK_TFLOPS, "traffic": None,
                   "algorithmic": "%d ordered pairs x %d flop" % (pairs, P2P_FLOPS_PER_PAIR),
-                  "duration": "isolated stage time (every stage on one stream)",
+                  "duration": "isolated stage time (every stage on one stream; with k_near where light "
+                              "cells are taken one-sided)",
                   "peak_source": "derived: 152 SM x 128 FP32 lanes x 2 x 2070 MHz",
                   "achieved_in_step": ach, "frac_in_step": ach / FP32_ALU_PEAK_TFLOPS,
                   "ordered_pairs": pairs}
     m_ms, m_iso = stage_ms["m2l"], stage_iso["m2l"]
     if tc:
-        peak, src = tc_peak(run.precision, long_step)
+        peak, src = tc_peak(long_step)
         a = mw["algorithmic_flops"] / (m_ms * 1e-3) / 1e12
         out["m2l"] = {"kernel": "k_m2l_tcg", "bound": "tensor", "achieved": a, "peak": peak,
                       "unit": "TFLOP/s", "frac": a / peak, "traffic": None,
@@ -762,7 +761,7 @@ def main():
     roof["hbm_peak_source"] = peak_kind
 
     extras = not args.no_extras and world == 1
-    # the plain FP32 form (SIMT contraction), same timing protocol, fewer steps
+    # the plain FP32 form, same timing protocol, fewer steps
     plain = None
     if extras and args.precision != "fp32" and not args.shift_free:
         r32 = Run(args.workload, "fp32", dev, w=w)
