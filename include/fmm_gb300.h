@@ -332,7 +332,8 @@ int fmm_batch_workspace_size(fmm_batch_t batch, const int64_t *n, size_t *bytes)
  * system from the prefix of the systems' block counts), so each system's
  * results equal its single-system evaluation bit for bit.  The merged
  * launches are captured once into a CUDA graph and replayed by later calls
- * with the same pointers and counts (one graph launch per call); the first
+ * with the same workspace, counts and set of wanted outputs, whatever arrays and
+ * whatever first row they are given (one graph launch per call); the first
  * call times the schedules (one stream, or the near field on a second stream)
  * and keeps the faster (fmm_batch_get_stats reports it).  Batches whose
  * systems' launch sequences do not merge (FP64 plans) run as per-system

@@ -1509,12 +1509,19 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
                    size_t workspace_bytes, void *stream) {
     if (!B || !offsets) return FMM_ERR_ARG;
     if (!workspace || ((uintptr_t)workspace & 255)) return FMM_ERR_WORKSPACE;
+    // rows are counted from the first system's, and the arrays start there: equal
+    // counts then mean equal places, wherever in the caller's arrays the systems lie
     std::vector<int64_t> n(B->nsys), pofs(B->nsys);
     for (int i = 0; i < B->nsys; i++) {
-        pofs[i] = offsets[i];
+        pofs[i] = offsets[i] - offsets[0];
         n[i] = offsets[i + 1] - offsets[i];
     }
     if (offsets[B->nsys] > 0 && (!pos || !q)) return FMM_ERR_ARG;
+    const int64_t row0 = offsets[0], rs = B->opts.precision == FMM_PREC_FP64 ? 8 : 4;
+    if (pos) pos += 3 * row0;
+    if (q) q += row0;
+    if (potential) potential = (char *)potential + row0 * rs;
+    if (forces) forces = (char *)forces + 3 * row0 * rs;
     std::vector<size_t> wofs;
     size_t total = 0;
     int rc = batch_layout(B, n.data(), wofs, &total);
@@ -1529,7 +1536,7 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
     cudaStreamWaitEvent(st, B->in_ev, 0);
     char *ws = (char *)workspace;
     // what a captured graph is valid for: the workspace, the counts and which
-    // outputs are wanted; a merged graph reads the arrays' addresses from a table
+    // outputs are wanted; a merged graph reads the first rows' addresses from a table
     // (recording, capturing and instantiating again for every new set of arrays
     // took 4.5 ms a call with 512 systems), the stream lanes hold them
     IoArrays io = {{(void *)pos, (void *)q, potential, forces, energy}};
