@@ -687,7 +687,8 @@ int fmm_plan_create(fmm_plan_t *out, const double box[4], int depth, int p, int 
         }
     }
     fmm::far_set_attributes();
-    int rc = P->fp64 ? upload_tables<double>(P) : upload_tables<float>(P);
+    int rc = P->tc ? tc_set_attributes(g.p3, P->tc_mode) : FMM_OK;
+    if (rc == FMM_OK) rc = P->fp64 ? upload_tables<double>(P) : upload_tables<float>(P);
     if (rc == FMM_OK && o.shift_free) rc = fmm::sf_build(p, depth, P->periodic, P->cd, &P->sf_tab, P->sf_base, &P->sf_H,
                                                    P->sf_hoff);
     // the tables went up by cudaMemcpy from pageable memory, which may return

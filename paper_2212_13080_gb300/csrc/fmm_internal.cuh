@@ -397,6 +397,9 @@ int tc_cross_records(const std::vector<TcXSys> &sys, const std::vector<int> &dep
 int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const void *k_map, const float *kbar,
                   int lmin, int mode, int inject, float *loc, int spow, bool split, int comp, cudaStream_t st,
                   Tracer &tr);
+// the shared-memory limits of the contraction's kernels on the current device
+// (an attribute is the device's: every plan sets its own)
+int tc_set_attributes(int p3, int mode);
 // map of a [343][tc_padded] table of kernel rows
 int tc_encode_kernel_map(void *map, const void *base, int p3, int mode);
 int tc_padded(int p3);     // p^3 rounded up to 32 (MMA N)

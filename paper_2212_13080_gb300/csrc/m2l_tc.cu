@@ -1079,14 +1079,6 @@ template int build_tables<double>(int, double, int, int, int, double *, double *
 template <int N, int MODE>
 static int launch_tcg_kernel(const TcgParams &prm, int blocks, int comp, cudaStream_t st, Tracer &tr) {
     typedef TcgShape<N, MODE> Gh;
-    static bool attr = false;
-    if (!attr) {
-        if (cudaFuncSetAttribute(k_m2l_tcg<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 Gh::SMEM) != cudaSuccess)
-            return FMM_ERR_CUDA;
-        kb_set_smem<KM2LTcg<N, MODE>>(Gh::SMEM);
-        attr = true;
-    }
     launch_k(tr, FMM_TAG(S_M2L_TC, comp), k_m2l_tcg<N, MODE>, KM2LTcg<N, MODE>{prm}, blocks, Gh::THREADS, Gh::SMEM,
              st);
     return FMM_OK;
@@ -1109,6 +1101,32 @@ static int record_tcx_mode(int p3s, const TcgParams &prm, int blocks, int comp, 
     case 224: return record_tcx<224, MODE>(prm, blocks, comp, tr);
     default: return FMM_ERR_UNSUPPORTED;
     }
+}
+
+template <int N, int MODE>
+static int set_attributes() {
+    typedef TcgShape<N, MODE> Gh;
+    if (cudaFuncSetAttribute(k_m2l_tcg<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gh::SMEM) != cudaSuccess)
+        return FMM_ERR_CUDA;
+    kb_set_smem<KM2LTcg<N, MODE>>(Gh::SMEM);
+    return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+}
+template <int MODE>
+static int set_attributes_mode(int p3s) {
+    switch (p3s) {
+    case 32: return set_attributes<32, MODE>();
+    case 64: return set_attributes<64, MODE>();
+    case 128: return set_attributes<128, MODE>();
+    case 224: return set_attributes<224, MODE>();
+    default: return FMM_ERR_UNSUPPORTED;
+    }
+}
+int tc_set_attributes(int p3, int mode) {
+    const int p3s = tc_padded(p3);
+    return mode == FMM_TC_BF16X3  ? set_attributes_mode<TC_BF16X3>(p3s)
+           : mode == FMM_TC_F16X1 ? set_attributes_mode<TC_F16X1>(p3s)
+           : mode == FMM_TC_F16X3C ? set_attributes_mode<TC_F16X3C>(p3s)
+                                  : set_attributes_mode<TC_F16X3>(p3s);
 }
 
 template <int MODE>
