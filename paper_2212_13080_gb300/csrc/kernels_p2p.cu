@@ -1215,8 +1215,9 @@ void launch_p2p(const Geom &g, const Ptrs<real> &P, const WsLayout &W, int64_t n
                  st);
         tr.count();
     }
+    // (a tag each: systems of either kind share a batch)
 #define LAUNCH_LT(F, CK, POW, LT)                                                                  \
-    launch_k(tr, FMM_TAG(S_P2P, 0), k_p2p<real, F, CK, POW, LT>,                                    \
+    launch_k(tr, FMM_TAG(S_P2P, LT), k_p2p<real, F, CK, POW, LT>,                                    \
              KP2P<real, F, CK, POW, LT>{depth, g.periodic, P.leaf_start, P.s_pt, P.s_origin, P.out_pt, P.react, W.cap, \
                                         pord},                                                     \
              ncell, NF_BS, 0, st)
