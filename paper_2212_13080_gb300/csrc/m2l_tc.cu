@@ -69,44 +69,90 @@ __device__ __forceinline__ void tc_wait_failed(int *status, int site, int level,
 }
 
 // The interaction list of every target parity (bx, by, bz): offsets o in
-// [-2 - b, 3 - b]^3 without [-1, 1]^3, ordered by the source's parity, then by
-// its coarse shift (x fastest): a tile's source cells of one parity (a few
-// hundred cells, used by up to 27 offsets) are read in one stretch of the
-// walk, so that the tiles in flight find them in L2 (152 tiles x 0.3 MB at
-// p = 6, against 2.6 MB a tile for all eight parities: measured 54.6 ms with
-// the offsets in x, y, z order).  An entry packs the index of
-// the offset in the 7^3 kernel tables, the source's parity block and its
+// [-2 - b, 3 - b]^3 without [-1, 1]^3, in one of two orders.  An entry packs the
+// index of the offset in the 7^3 kernel tables, the source's parity block and its
 // coarse shift (-1..1 per axis).
+//   0: z, y, x order: neighbouring source cells follow one another, and what they
+//      cancel of each other leaves the sum at once.
+//   1: by the source's parity, then by its coarse shift: a tile's source cells of
+//      one parity (a few hundred cells, used by up to 27 offsets) are read in one
+//      stretch of the walk, so that the tiles in flight find them in L2 (152 tiles x
+//      0.3 MB at p = 6, against 2.6 MB a tile for all eight parities).
+// Order 1 only where a level's operand copy may exceed the L2 (level 6: 282 MB at
+// p = 6, level 5: 42 MB): the contraction of 8M clustered charges takes 38 ms so, 55
+// in order 0.  On coarse levels it would cost digits: the 27 sources of one parity
+// are the 27 images of a single cell at level 1 of the periodic form, and their
+// sum, several times the result, rounds before the other parities cancel it
+// (water, 66,669 charges: potentials up to 1.17 times as far from the 64-bit results
+// as in order 0).
 struct OffTable {
-    uint32_t v[8][TC_NOFF];
+    uint32_t v[2][8][TC_NOFF];
 };
+__host__ __device__ constexpr int off_order(int l) { return l >= 6; }
+constexpr uint32_t off_entry(const int (&b)[3], int ox, int oy, int oz) {
+    const int s[3] = {b[0] + ox, b[1] + oy, b[2] + oz};  // the source in children of the target's parent
+    uint32_t v = (uint32_t)(((oz + 3) * 7 + (oy + 3)) * 7 + (ox + 3));
+    for (int a = 0; a < 3; a++) {
+        const int h = s[a] & 1, d = (s[a] - h) / 2;
+        v |= (uint32_t)h << (9 + a) | (uint32_t)(d + 1) << (12 + 2 * a);
+    }
+    return v;
+}
+constexpr bool off_near(int ox, int oy, int oz) {
+    return ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1;
+}
 constexpr OffTable make_off_table() {
     OffTable t{};
     for (int par = 0; par < 8; par++) {
         const int b[3] = {par & 1, (par >> 1) & 1, par >> 2};
         int n = 0;
+        for (int oz = -2 - b[2]; oz <= 3 - b[2]; oz++)
+            for (int oy = -2 - b[1]; oy <= 3 - b[1]; oy++)
+                for (int ox = -2 - b[0]; ox <= 3 - b[0]; ox++)
+                    if (!off_near(ox, oy, oz)) t.v[0][par][n++] = off_entry(b, ox, oy, oz);
+        n = 0;
         for (int sp = 0; sp < 8; sp++)
-            for (int dz = -1; dz <= 1; dz++)
-                for (int dy = -1; dy <= 1; dy++)
-                    for (int dx = -1; dx <= 1; dx++) {
-                        const int ox = 2 * dx + (sp & 1) - b[0], oy = 2 * dy + ((sp >> 1) & 1) - b[1],
-                                  oz = 2 * dz + (sp >> 2) - b[2];
-                        if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1) continue;
-                        t.v[par][n++] = (uint32_t)(((oz + 3) * 7 + (oy + 3)) * 7 + (ox + 3)) | (uint32_t)sp << 9 |
-                                        (uint32_t)(dx + 1) << 12 | (uint32_t)(dy + 1) << 14 | (uint32_t)(dz + 1) << 16;
-                    }
+            for (int d = 0; d < 27; d++) {
+                const int ox = 2 * (d % 3 - 1) + (sp & 1) - b[0], oy = 2 * (d / 3 % 3 - 1) + ((sp >> 1) & 1) - b[1],
+                          oz = 2 * (d / 9 - 1) + (sp >> 2) - b[2];
+                if (!off_near(ox, oy, oz)) t.v[1][par][n++] = off_entry(b, ox, oy, oz);
+            }
     }
     return t;
 }
-__constant__ const OffTable c_off = make_off_table();
 struct Off {
     int oi, spar, dX, dY, dZ;
 };
-__device__ __forceinline__ Off list_offset(int par, int i) {
-    const uint32_t v = c_off.v[par][i];
+__host__ __device__ constexpr Off unpack_off(uint32_t v) {
     return Off{(int)(v & 511u), (int)((v >> 9) & 7u), (int)((v >> 12) & 3u) - 1, (int)((v >> 14) & 3u) - 1,
                (int)(v >> 16) - 1};
 }
+// both orders hold every offset of every target parity's list once, each with the
+// source cell it leads to; order 1 goes by source parity
+constexpr bool off_table_ok(const OffTable &t) {
+    for (int ord = 0; ord < 2; ord++)
+        for (int par = 0; par < 8; par++) {
+            const int b[3] = {par & 1, (par >> 1) & 1, par >> 2};
+            bool seen[343] = {};
+            int last = 0;
+            for (int i = 0; i < TC_NOFF; i++) {
+                const Off f = unpack_off(t.v[ord][par][i]);
+                const int o[3] = {f.oi % 7 - 3, f.oi / 7 % 7 - 3, f.oi / 49 - 3}, d[3] = {f.dX, f.dY, f.dZ};
+                if (f.oi >= 343 || seen[f.oi] || off_near(o[0], o[1], o[2])) return false;
+                seen[f.oi] = true;
+                for (int a = 0; a < 3; a++) {
+                    if (o[a] < -2 - b[a] || o[a] > 3 - b[a] || d[a] < -1 || d[a] > 1) return false;
+                    if (2 * d[a] + ((f.spar >> a) & 1) != b[a] + o[a]) return false;
+                }
+                if (ord == 1 && f.spar < last) return false;
+                last = f.spar;
+            }
+        }
+    return true;
+}
+static_assert(off_table_ok(make_off_table()), "the interaction lists of the eight target parities");
+__constant__ const OffTable c_off = make_off_table();
+__device__ __forceinline__ Off list_offset(int ord, int par, int i) { return unpack_off(c_off.v[ord][par][i]); }
 
 #define TC_F16X3 FMM_TC_F16X3
 #define TC_F16X1 FMM_TC_F16X1
@@ -390,7 +436,7 @@ struct KM2LTcg {
         while (k + 1 < prm.nseg && (int)bid_ >= seg_first[k + 1]) k++;
         const int sg = cross ? k : prm.nseg - 1 - k;  // a system's own blocks: the deepest level first
         const int l = prm.lmin + sg / 8, par = sg & 7;
-        const int H = 1 << (l - 1), P = H + 2;
+        const int H = 1 << (l - 1), P = H + 2, ord = off_order(l);
         const int count = seg_cnt[sg];
         const int parts = cross ? 1 : tc_parts(l, prm.depth);
         const int tile = ((int)bid_ - seg_first[k]) / parts, part = ((int)bid_ - seg_first[k]) % parts;
@@ -508,17 +554,17 @@ struct KM2LTcg {
             // fetched one offset ahead: the charge into registers, the means by the
             // epilogue's threads into a shared row
             auto source = [&](int i) {
-                const Off f = list_offset(par, i);
+                const Off f = list_offset(ord, par, i);
                 return valid ? q[((f.spar * P + f.dZ) * P + f.dY) * P + f.dX] : make_float2(0.0f, 0.0f);
             };
             const int et = threadIdx.x;  // epilogue thread (the epilogue warps come first)
             float2 qs = source(i0);
-            if (et < N) kbs[et] = prm.kbar[list_offset(par, i0).oi * N + et];
+            if (et < N) kbs[et] = prm.kbar[list_offset(ord, par, i0).oi * N + et];
             asm volatile("bar.sync 1, %0;" ::"n"(32 * Sh::EPI) : "memory");
             for (int i = i0; i < i1; i++) {
                 const int j = i - i0, in = i + 1 < i1 ? i + 1 : i;
                 const float2 qn = source(in);
-                const float kn = et < N ? prm.kbar[list_offset(par, in).oi * N + et] : 0.0f;
+                const float kn = et < N ? prm.kbar[list_offset(ord, par, in).oi * N + et] : 0.0f;
                 const float2 Q2 = make_float2(qs.x, qs.x), inv2 = make_float2(qs.y, qs.y);
                 const float *kb = kbs + (j & 1) * N + c0;
 #pragma unroll 1
@@ -546,8 +592,9 @@ struct KM2LTcg {
                             d0 = __fmul2_rn(d0, inv2);
                             d1 = __fmul2_rn(d1, inv2);
                         } else if (Sh::SCALED) {
-                            d0 = __ffma2_rn(d0, inv2, __fmul2_rn(m0, Q2));
-                            d1 = __ffma2_rn(d1, inv2, __fmul2_rn(m1, Q2));
+                            // (the factor is a power of two: one rounding, of the sum)
+                            d0 = __ffma2_rn(m0, Q2, __fmul2_rn(d0, inv2));
+                            d1 = __ffma2_rn(m1, Q2, __fmul2_rn(d1, inv2));
                         } else {
                             d0 = __ffma2_rn(m0, Q2, d0);
                             d1 = __ffma2_rn(m1, Q2, d1);
@@ -667,7 +714,7 @@ struct KM2LTcg {
                 int last_phase[4] = {-1, -1, -1, -1};
                 int it = 0, sig = 0;  // sig: next gathered stage to signal
                 for (int i = i0; i < i1 && !failed; i++) {
-                    const Off f = list_offset(par, i);
+                    const Off f = list_offset(ord, par, i);
                     const int delta = (((f.spar * P + f.dZ) * P + f.dY) * P + f.dX) * Sh::RC;
                     for (int kc = 0; kc < Sh::KC; kc++, it++) {
                         const int s = it % Gh::SA;
@@ -732,7 +779,7 @@ struct KM2LTcg {
                     int last_phase[4] = {-1, -1, -1, -1};
                     int it = 0;
                     for (int i = i0; i < i1 && !failed; i++) {
-                        const int oi = list_offset(par, i).oi;
+                        const int oi = list_offset(ord, par, i).oi;
                         for (int kc = 0; kc < Sh::KC; kc++, it++) {
                             const int s = it % Gh::SB;
                             const uint32_t ph = (uint32_t)(it / Gh::SB) & 1u;
