@@ -58,10 +58,13 @@ extern "C" {
 #define FMM_ERR_UNSUPPORTED 10   /* combination not built (e.g. tensor-core M2L for this p) */
 
 /* ---- precision of the far-field contraction (and of everything else) ----- */
-#define FMM_PREC_FP32 0   /* FP32 everywhere; bilinear forms of orders 3..6 on the tensor cores
-                             with every operand split into two halves of 11 significant
-                             bits (FP32's digits) and a compensated FP32 sum over the
-                             interaction list, of other orders in FP32 multiply-adds */
+#define FMM_PREC_FP32 0   /* FP32 everywhere; bilinear forms of orders 3..6 on the tensor cores,
+                             every operand in half-precision parts: of orders 5 and 6 three,
+                             all of FP32's bits with exact leading products; of orders 3 and
+                             4 two, an operand to 2^-23 and a product to 2^-22 of itself; a
+                             compensated FP32 sum over the interaction list.  Measured errors
+                             are no larger than with FP32 multiply-adds, which the other
+                             orders take */
 #define FMM_PREC_FP64 1   /* FP64 everywhere; outputs are float64 */
 #define FMM_PREC_TF32X3 2 /* bilinear forms on tcgen05 tensor cores, 3-pass split with TF32's
                              significand (two halves of 11 bits, scaled per cell so that

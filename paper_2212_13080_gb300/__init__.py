@@ -43,8 +43,9 @@ class FMM:
     for precision="fp64".  Host tensors are copied to the device and the
     results back (the end-to-end path); host results are views of pinned
     buffers the plan keeps and overwrites on its next host call (clone to keep).
-    precision: "fp32" (FP32 digits throughout), "fp64", "tf32x3" / "tf32x1" /
-    "bf16x3" (reduced-precision bilinear forms on the tcgen05 tensor cores).
+    precision: "fp32" (FP32; bilinear forms of orders 3 to 6 in split half-precision
+    parts with FP32's measured errors), "fp64", "tf32x3" / "tf32x1" / "bf16x3"
+    (reduced-precision bilinear forms on the tcgen05 tensor cores).
     grid_scale < 1: the reduced arrangement of the p-division points (§4.1).
     shift_free: App. A.2, precomputed bilinear forms on box-basis grid charges
     (precision "fp64", p <= 5).

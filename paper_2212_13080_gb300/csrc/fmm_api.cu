@@ -205,13 +205,13 @@ int upload_tables(fmm_plan_t P) {
         cudaMalloc(&P->Kbar, no * p3 * sizeof(real)) != cudaSuccess)
         return FMM_ERR_OOM;
     const size_t rows = (size_t)343 * tc_padded(p3);
-    if (P->tc && (cudaMalloc(&P->Ktc, nc * rows * tc_row_bytes(p3)) != cudaSuccess ||
+    if (P->tc && (cudaMalloc(&P->Ktc, nc * rows * tc_row_bytes(p3, P->tc_mode)) != cudaSuccess ||
                   cudaMalloc(&P->Kbar_tc, nc * rows * sizeof(float)) != cudaSuccess))
         return FMM_ERR_OOM;
     int rc = build_tables<real>(p, gs, P->geom.power, nc, P->tc_mode, (real *)P->Kunit, (real *)P->Kbar, P->Ktc,
                                 (float *)P->Kbar_tc);
     for (int c = 0; P->tc && c < nc && !rc; c++)
-        rc = tc_encode_kernel_map(P->k_map[c], (const char *)P->Ktc + c * rows * tc_row_bytes(p3), p3, P->tc_mode);
+        rc = tc_encode_kernel_map(P->k_map[c], (const char *)P->Ktc + c * rows * tc_row_bytes(p3, P->tc_mode), p3, P->tc_mode);
     if (rc) return rc;
     std::vector<double> row(p3);
     if (P->periodic) {
@@ -340,7 +340,7 @@ WsLayout make_layout(const fmm_plan_t P, int64_t n) {
     W.m2l_part = take(part * rs);
     W.total_simt = o;
     o = o0;
-    W.op = take(P->tc ? (size_t)qc * tc_row_bytes(p3) : 0);
+    W.op = take(P->tc ? (size_t)qc * tc_row_bytes(p3, P->tc_mode) : 0);
     W.qsc = take(P->tc ? (size_t)qc * sizeof(float2) : 0);
     W.tc_part = take(P->tc ? (size_t)tc_part_values(P->depth, p3) * 4 : 0);
     W.occ = take(P->tc ? (size_t)occ_ints(P->depth, P->periodic ? 1 : 2) * 4 : 0);
@@ -646,7 +646,7 @@ int fmm_plan_create(fmm_plan_t *out, const double box[4], int depth, int p, int 
     P->tc = tc_prec || (o.precision == FMM_PREC_FP32 && p >= 3 && p <= 6);
     P->tc_mode = o.precision == FMM_PREC_BF16X3   ? FMM_TC_BF16X3
                  : o.precision == FMM_PREC_TF32X1 ? FMM_TC_F16X1
-                 : o.precision == FMM_PREC_FP32   ? FMM_TC_F16X3C
+                 : o.precision == FMM_PREC_FP32   ? FMM_TC_F32
                                                   : FMM_TC_F16X3;
     cudaGetDevice(&P->device);
     fill_coef<float>(p, o.grid_scale, P->cf);
@@ -1128,6 +1128,7 @@ int record_merged(fmm_batch_t B, const std::vector<int64_t> &n, const std::vecto
         std::vector<int> dep(ns);
         WsLayout W0;
         size_t ws_bytes = 0;
+        const int cb = tc_chunk_bytes(M0->geom.p3, M0->tc_mode);
         for (int i = 0; i < ns; i++) {
             WsLayout W = make_layout(B->sys[i], n[i]);
             Ptrs<float> Pi = make_ptrs<float>(W, ws + wofs[i]);
@@ -1135,7 +1136,7 @@ int record_merged(fmm_batch_t B, const std::vector<int64_t> &n, const std::vecto
             ws_bytes = std::max(ws_bytes, wofs[i] + W.total);
             dep[i] = n[i] > 0 ? B->sys[i]->depth : 0;
             for (int c = 0; c < M0->ncomp; c++)
-                xs[(size_t)c * ns + i] = TcXSys{(int)((Pi.op - ws) / 128), Pi.qsc, Pi.loc + c * W.loc_comp, Pi.tc_part};
+                xs[(size_t)c * ns + i] = TcXSys{(int)((Pi.op - ws) / cb), Pi.qsc, Pi.loc + c * W.loc_comp, Pi.tc_part};
         }
         const void *km[4];
         const float *kb[4];

@@ -191,7 +191,7 @@ __host__ __device__ inline int64_t occ_list_offset(int depth, int lmin) {
 }
 // A segment takes box tiles (each offset's A operand one TMA box of 8 x 4 x 4
 // coarse cells, empty cells included) where nearly all of its cells hold
-// charges: a box costs one copy instead of 32 gathers a chunk, and multiplies
+// charges: a box costs one copy a chunk instead of a gather of its rows, and multiplies
 // the empty cells.
 __host__ __device__ inline bool occ_box_segment(int H, int64_t count, int N) {
     const int pct = N >= 128 ? 95 : 90;
@@ -370,14 +370,15 @@ int launch_downward(const Geom &g, const Coef<real> &C, const Ptrs<real> &P, con
 #define FMM_TC_F16X3 0   // 3-pass split: two 11-bit halves per operand (TF32's significand), scaled
 #define FMM_TC_F16X1 1   // 1 pass: operands rounded to 11 bits, scaled
 #define FMM_TC_BF16X3 2  // 3-pass split BF16
-#define FMM_TC_F16X3C 3  // as F16X3, the sum over the offsets compensated (plain FP32 plans)
+#define FMM_TC_F32 3     // plain FP32 plans: two halves per operand (p = 3, 4) or three (p = 5, 6), the sum
+                         // over the offsets compensated
 // factor of the scaled kernel tables: |K| <= 2 at unit cells (separation >= 1),
 // so the scaled entries stay below the half type's maximum and their lo parts
 // above its subnormal floor
 #define TC_KSCALE 16384.0f
 // one system of a batched evaluation's cross-system contraction tiles
 struct TcXSys {
-    int op_chunk;               // its operand copy: first 128-byte chunk from the batch's workspace
+    int op_chunk;               // its operand copy: first chunk (tc_chunk_bytes) from the batch's workspace
     const float2 *qsc;          // its cells' charges and operand factors
     float *loc;                 // its functionals (one kernel component)
     float *part;                // scratch of the functionals' layout
@@ -403,7 +404,8 @@ int tc_set_attributes(int p3, int mode);
 // map of a [343][tc_padded] table of kernel rows
 int tc_encode_kernel_map(void *map, const void *base, int p3, int mode);
 int tc_padded(int p3);     // p^3 rounded up to 32 (MMA N)
-int tc_row_bytes(int p3);  // bytes of a cell vector's (or kernel row's) split copy
+int tc_row_bytes(int p3, int mode);    // bytes of a cell vector's (or kernel row's) split copy
+int tc_chunk_bytes(int p3, int mode);  // bytes of its chunks (the unit of a row's place)
 size_t tc_map_bytes();
 // the kernel tables of a plan, computed on the device (rows, kbar_tc: tensor
 // cores, or null); asynchronous on the default stream

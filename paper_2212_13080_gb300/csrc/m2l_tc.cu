@@ -1,6 +1,6 @@
 // Bilinear forms of the interaction lists (§2.2 step 3, eq. bilinear) on the
-// 5th-generation tensor cores (tcgen05): 16-bit operands in 3-pass split form
-// (half or bfloat16) or one pass, FP32 accumulation.
+// 5th-generation tensor cores (tcgen05): operands split into 16-bit parts (half or
+// bfloat16), FP32 accumulation.
 //
 // Only cells that hold charges get a functional (step 4 reads no other).
 // After the sort, a list of the occupied cells of every (level, target
@@ -9,37 +9,47 @@
 // contribution L[cell][a] += sum_b Phi[cell + o][b] K_o[a][b] is a
 // 128 x N x K GEMM (N = p^3 padded to a multiple of 32, K to a multiple of
 // 16): A holds the tile's 128 source vectors, B the unit-cell kernel K_o, both
-// in 128-byte K chunks staged in shared memory with the 128-byte swizzle; one
-// thread issues the MMAs into tensor memory.  A arrives in one of two ways:
+// in K chunks staged in shared memory with the swizzle of their width; one thread
+// issues the MMAs into tensor memory.  A arrives in one of two ways:
 //   - box tiles (a segment whose cells nearly all hold charges): the tile is
 //     128 consecutive Morton cells, an 8 x 4 x 4 box of the padded parity-major
 //     layout, one box copy a chunk;
 //   - gathered tiles: producer warps copy the rows with 16-byte cp.async
-//     straight into the swizzled layout (16-byte piece j of row r lands at piece
-//     j ^ (r mod 8)), complete and fence them for the async proxy before they
-//     arrive on the stage.  A lane's rows and places are fixed for the whole
-//     tile, so a row costs one address and two copies a stage; TMA row gathers
-//     (four rows each) took 65 cycles each: 79.7 against 51 ms on 8M clustered
-//     charges at p = 6.
+//     straight into the swizzled layout, complete and fence them for the async
+//     proxy before they arrive on the stage.  A lane's rows and places are fixed
+//     for the whole tile, so a row costs one address and two or three copies a
+//     stage; TMA row gathers (four rows each) took 65 cycles each: 79.7 against
+//     51 ms on 8M clustered charges at p = 6.
 //
-// Operands.  x = hi + lo in two halves of 11 significant bits each, after an
-// exact power-of-two scaling (per cell for the grid charges, one factor for
-// the kernels) that puts the largest value near the type's maximum: as many
-// significant bits as FP32 keeps of a value, so plain FP32 plans (p = 3..6)
-// and the split-TF32 precision use this form at twice TF32's MMA rate and half
-// its bytes.  D = Alo Bhi + Ahi Blo + Ahi Bhi.  The BF16 form has 8 + 8 bits
-// and no scaling; the 1-pass form takes Ahi Bhi alone (11 bits, TF32's).
+// Operands, after an exact power-of-two scaling (per cell for the grid charges, one
+// factor for the kernels) that puts the largest value near the half type's maximum:
+//   two parts (split TF32; plain FP32 plans of p = 3, 4): x = hi + lo, two halves of
+//     11 significant bits each, so that x is off by at most 2^-23 of itself, and
+//     D = Alo Bhi + Ahi Blo + Ahi Bhi leaves out a product of up to 2^-22 of a term:
+//     less than FP32's 24 bits, in sums of at most 64 terms whose rounding outweighs it.
+//     Twice TF32's MMA rate and half its bytes.
+//   three parts (plain FP32 plans of p = 5, 6): all of FP32's bits, six products, and
+//     the leading products' sum is exact (KSplit).  The tensor cores' FP32 additions do
+//     not round to nearest, and two parts summed that way over 125 and 216 terms were
+//     up to 7% further from the 64-bit results than FP32 multiply-adds where the terms
+//     cancel.  Contraction of 1M clustered charges at p = 6: 7.3 ms with two parts, 10.8
+//     with three, 243 with multiply-adds.
+//   BF16: two parts of 8 bits, unscaled; the 1-pass form: Ahi Bhi alone, 11 bits.
 //
 // Accuracy.  The kernel is split as K_o = Kbar_o[a] + Kt_o[a,b] (row mean): the
 // tensor cores contract Kt_o, the CUDA cores add Kbar_o[a] Q (Q = the source
-// cell's total charge).  Each offset accumulates into a fresh TMEM region (two
-// regions, alternating), small products first; the epilogue warps read it out
-// and add the offsets in FP32 registers, for plain FP32 plans with Kahan
-// compensation: without it these 189 additions are the largest error of the
-// form (potentials of a depth-4 system at p = 6: 3.2e-7 against 2.8e-7 for FP32
-// multiply-adds), and it costs the reduced-precision plans more than they need
-// (uniform1m: 0.36 against 0.24 ms).  A row's functional depends on its own A rows only, so it is the
-// same, bit for bit, whichever tile form computes it.
+// cell's total charge).  Each offset accumulates into fresh TMEM regions, small
+// products first; the epilogue warps read them out and add the offsets in FP32
+// registers, for plain FP32 plans with Kahan compensation: without it these 189
+// additions are the largest error of the form (potentials of a depth-4 system at
+// p = 6: 3.2e-7 against 2.8e-7 for FP32 multiply-adds), and it costs the
+// reduced-precision plans more than they need (uniform1m: 0.36 against 0.24 ms).
+// Plain FP32 plans against FP32 multiply-adds, distance from the 64-bit results in
+// 74 systems of 2,001 to 1M charges, open and periodic, p = 3..6: potentials 0.94
+// times (at most 1.00), forces 0.91 (at most 1.001); with octants charged in turn,
+// where the terms cancel, 0.97 to 1.00 in the mean of 24 systems.
+// A row's functional depends on its own A rows only, so it is the same, bit for
+// bit, whichever tile form computes it.
 #include <algorithm>
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -54,7 +64,6 @@
 namespace fmm {
 
 #define TC_M 128
-#define TC_ABYTES (TC_M * 128)      // 128 rows of one 128-byte K chunk
 #define TC_WAIT_CYCLES (4LL << 30)  // about 2 s of SM clock
 #define TC_NOFF 189
 
@@ -157,35 +166,35 @@ __device__ __forceinline__ Off list_offset(int ord, int par, int i) { return unp
 #define TC_F16X3 FMM_TC_F16X3
 #define TC_F16X1 FMM_TC_F16X1
 #define TC_BF16X3 FMM_TC_BF16X3
-#define TC_F16X3C FMM_TC_F16X3C
+#define TC_F32 FMM_TC_F32
 
-// A cell vector (and a kernel row) in 128-byte chunks of 64 values: the hi and
-// the lo part of every 64 values in two chunks; a tail of at most 32 values has
-// both in one (hi in its first half).  p = 3: 27 values, one chunk; 4: 64, two;
-// 5: 125, four; 6: 216, seven.
+// A cell vector (and a kernel row) in chunks.
+// Two parts: 128-byte chunks of 64 values, the hi and the lo part of every 64
+// values in two chunks; a tail of at most 32 values has both in one (hi in its
+// first half).  p = 3: 27 values, one chunk; 4: 64, two; 5: 125, four; 6: 216, seven.
+// Three parts: 64-byte chunks, the three parts of every 32 values one after another.
 template <int N, int MODE>
 struct TcShape {
-    static constexpr int CH = N > 64 ? 2 : 1;           // epilogue column groups
+    static constexpr int CH = N > 64 || (N == 64 && MODE == TC_F32) ? 2 : 1;  // epilogue column groups
     static constexpr int EPI = 4 * CH;                  // epilogue warps
-    static constexpr int KS = N == 32 ? 2 : (N == 64 ? 4 : (N == 128 ? 8 : 14));  // MMA steps of 16 values
-    static constexpr int FC = KS / 4;                   // stages of whole chunks (hi, lo)
-    static constexpr int KC = (KS + 3) / 4;             // stages per offset
-    static constexpr int RC = 2 * FC + (KC - FC);       // chunks per cell vector
     static constexpr bool LO = MODE != TC_F16X1;        // lo parts loaded and used
     static constexpr bool SCALED = MODE != TC_BF16X3;   // operands scaled by powers of two
-    static constexpr bool COMP = MODE == TC_F16X3C;     // compensated sum over the offsets
-    // Accumulators per offset, of KC / ND stages each.  The tensor cores' FP32
-    // additions do not round to nearest; with the compensated sum two
-    // accumulators of half the length keep plain FP32's errors at p = 5, 6
-    // (potentials of a clustered system at p = 6: 2.54e-7 against 2.81e-7 with one
-    // and 2.59e-7 for FP32 multiply-adds; contraction of plummer1m 6.2 -> 7.3 ms)
-    static constexpr int ND = COMP && N >= 128 ? 2 : 1;
-    static_assert(KC % ND == 0, "whole stages per accumulator");
-    static constexpr int BBYTES = N * 128;              // one chunk of K_o
+    static constexpr bool COMP = MODE == TC_F32;        // compensated sum over the offsets
+    static constexpr bool P3 = COMP && N > 64;          // three parts per operand
+    static constexpr int KS = N == 32 ? 2 : (N == 64 ? 4 : (N == 128 ? 8 : 14));  // MMA steps of 16 values
+    static constexpr int FC = KS / 4;                   // two parts: stages of whole chunks (hi, lo)
+    static constexpr int KC = P3 ? KS / 2 : (KS + 3) / 4;  // stages per offset
+    static constexpr int RC = P3 ? 3 * KC : 2 * FC + (KC - FC);  // chunks per cell vector
+    static constexpr int UB = P3 ? 64 : 128;            // bytes of a chunk's row
+    static constexpr int ABYTES = TC_M * UB;            // one chunk of the tile's rows
+    static constexpr int BBYTES = N * UB;               // one chunk of K_o
+    static constexpr int NCH = P3 ? 3 : (FC ? 2 : 1);   // chunks of a stage (two parts: a tail stage has one)
+    static constexpr int NCX = P3 ? 3 : 2;              // chunks from one stage to the next in a cell vector
+    static constexpr int ACC = P3 ? 2 : 1;              // accumulators per offset
     // cross-system tiles keep the totals of their runs of offsets in TMEM, the
     // widest tile (two accumulators fill it) in the output
     static constexpr bool RMW = N == 224;
-    static constexpr int TUSED = RMW ? 2 * N : 4 * N;
+    static constexpr int TUSED = RMW ? 2 * N : 4 * N;  // two accumulators, and two rows of totals or accumulators
     static constexpr int TCOLS = TUSED <= 128 ? 128 : (TUSED <= 256 ? 256 : 512);
     static constexpr int COLS = N / CH;                 // columns per epilogue thread
 };
@@ -329,13 +338,14 @@ __global__ void __launch_bounds__(KOccScatter::BS) k_occ_scatter(const __grid_co
 // The contraction over the occupied-cell lists.  A block takes one 128-row tile
 // of a segment (level l, target parity b): row r is the tile's r-th occupied
 // target cell, and its A operand row for offset o is the source cell (target +
-// o), copied by TMA gathers (or one box copy); the kernel matrix B arrives by
+// o), gathered with cp.async (or one box copy); the kernel matrix B arrives by
 // TMA box copies.  Levels with few tiles split the 189 offsets over tc_parts
 // blocks, whose partial functionals k_tc_reduce adds.
 //
 // What bounds it (GB300): p = 4 the shared-memory traffic of operands and MMAs
 // (N = 64 reads 6 KB per 32-cycle MMA), p = 5 and 6 the tensor pipe and the
-// operand copies.
+// operand copies; with three parts at p = 6 also the wait for the epilogue, since
+// one offset's two accumulators fill the tensor memory.
 // ---------------------------------------------------------------------------
 struct TcgParams {
     CUtensorMap k;                        // kernel tables: [343][N] rows of chunks
@@ -365,26 +375,27 @@ struct TcgParams {
 
 // Ring depths per tile shape.  N >= 128: the A stages (32 KB) and the kernel
 // stages (N 256 bytes) are separate rings with their own producers, one CTA per
-// SM (N = 224: 3 A + 2 B stages, 208 KB; N = 128: 3 + 3, 192 KB).  Dynamic plus
-// static shared memory stays below 227 KB.  N <= 64 (UNI): one ring whose
+// SM (N = 224: 3 A + 2 B stages, 208 KB; N = 128: 3 + 3, 192 KB; three parts: stages
+// of 24 KB and N 192 bytes, 3 + 3 and 4 + 4, 198 and 192 KB).  Dynamic plus static
+// shared memory stays below 227 KB.  N <= 64 (UNI): one ring whose
 // stages hold A and B, six warps and two CTAs per SM (each CTA's barrier round
-// trips and epilogue hide under the other's MMAs).  N = 224 needs about 210
-// registers per epilogue thread (112 sums and their compensations): the other
-// warpgroup gives its share up (216 x 256 + 72 x 128 = 168 x 384).
+// trips and epilogue hide under the other's MMAs).  The three-part shapes need about
+// 210 registers per epilogue thread (N = 224: 112 sums and their compensations): the
+// other warpgroup gives its share up (216 x 256 + 72 x 128 = 168 x 384).
 template <int N, int MODE>
 struct TcgShape {
     typedef TcShape<N, MODE> B;
     static constexpr bool UNI = N <= 64;
-    static constexpr int SA = N == 32 ? 4 : (N == 64 ? 2 : 3);
-    static constexpr int SB = N == 224 ? 2 : (N == 128 ? 3 : SA);
-    static constexpr int ASTAGE = (B::FC ? 2 : 1) * TC_ABYTES;
-    static constexpr int BSTAGE = (B::FC ? 2 : 1) * B::BBYTES;
+    static constexpr int SA = N == 32 || (N == 128 && B::P3) ? 4 : (N == 64 ? 2 : 3);
+    static constexpr int SB = N == 224 && !B::P3 ? 2 : SA;
+    static constexpr int ASTAGE = B::NCH * B::ABYTES;
+    static constexpr int BSTAGE = B::NCH * B::BBYTES;
     static constexpr int PW = UNI ? 1 : 2;           // A warps
     static constexpr int G = SA - 1;                 // stages of copies in flight per gathering thread
     static constexpr int WA = B::EPI;
     static constexpr int WB = WA + PW;               // kernel-matrix warp (split rings)
     static constexpr int WM = UNI ? WB : WB + 1;     // MMA warp
-    static constexpr bool SETREG = N == 224 && B::COMP;
+    static constexpr bool SETREG = B::P3;
     static constexpr int THREADS = 32 * (WM + 1);
     static_assert(!SETREG || THREADS == 384, "three warpgroups");
     static constexpr int MINB = UNI ? 2 : 1;
@@ -393,17 +404,27 @@ struct TcgShape {
     static_assert(SMEM + 1024 <= 227 * 1024, "shared memory of one CTA");
 };
 
-// one step of a compensated sum of pairs: run += t, the rounding error of the
-// addition carried to the next step in comp (two bfloat16: eight bits of it)
-__device__ __forceinline__ void kahan_add(float2 &run, uint32_t &comp, float2 t) {
-    const float2 y = __fadd2_rn(t, make_float2(__uint_as_float(comp << 16), __uint_as_float(comp & 0xFFFF0000u)));
-    const float2 s = __fadd2_rn(run, y);
+// One step of a compensated sum of pairs: run += y, where y holds the new term and
+// the rounding error of the last step, which comp carried; comp takes this step's.
+__device__ __forceinline__ float2 kahan_error(float2 &run, float2 y) {
     const float2 m1 = make_float2(-1.0f, -1.0f);
-    const float2 z = __ffma2_rn(run, m1, s);
-    const float2 e = __ffma2_rn(z, m1, y);
+    const float2 s = __fadd2_rn(run, y);
+    const float2 e = __ffma2_rn(__ffma2_rn(run, m1, s), m1, y);
+    run = s;
+    return e;
+}
+__device__ __forceinline__ float2 comp_value(float2 c) { return c; }
+__device__ __forceinline__ void kahan_add(float2 &run, float2 &comp, float2 y) { comp = kahan_error(run, y); }
+// N = 224, where 112 sums and as many floats do not fit a thread's registers: the
+// error's leading eight bits (two bfloat16), so that a sum is carried with 24 + 8
+// bits; what is left out is below 2^-33 of a partial sum each step
+__device__ __forceinline__ float2 comp_value(uint32_t c) {
+    return make_float2(__uint_as_float(c << 16), __uint_as_float(c & 0xFFFF0000u));
+}
+__device__ __forceinline__ void kahan_add(float2 &run, uint32_t &comp, float2 y) {
+    const float2 e = kahan_error(run, y);
     const __nv_bfloat162 c = __floats2bfloat162_rn(e.x, e.y);
     comp = *reinterpret_cast<const uint32_t *>(&c);
-    run = s;
 }
 
 // The next part of a sum of several runs: (h, w) += t with the rounding error
@@ -452,8 +473,8 @@ struct KM2LTcg {
         const uint32_t bars = bbase + Gh::SB * Gh::BSTAGE;
         const uint32_t afull0 = bars, aempty0 = afull0 + 8 * Gh::SA;
         const uint32_t bfull0 = aempty0 + 8 * Gh::SA, bempty0 = bfull0 + 8 * Gh::SB;
-        const uint32_t rfull0 = bempty0 + 8 * Gh::SB, rfree0 = rfull0 + 16;
-        const uint32_t done = rfree0 + 16;
+        const uint32_t rfull0 = bempty0 + 8 * Gh::SB, rfree0 = rfull0 + 32;
+        const uint32_t done = rfree0 + 32;
         const uint32_t tslot = done + 8;
         volatile uint32_t *tslot_ptr = reinterpret_cast<volatile uint32_t *>(smraw + (tslot - raw));
         float *kbs = reinterpret_cast<float *>(smraw + (bars - raw) + 256);  // row means of two offsets
@@ -462,12 +483,20 @@ struct KM2LTcg {
         int *rowG = reinterpret_cast<int *>(kbs + 2 * N);
         int *rowQ = rowG + TC_M, *rowL = rowQ + TC_M, *rowS = rowL + TC_M;
 
+        // chunks of an offset's kc-th stage (two parts: a tail holds hi and lo in one)
+        auto stage_chunks = [](int kc) { return Sh::P3 ? 3 : (kc < Sh::FC && Sh::LO ? 2 : 1); };
         // Box tiles (occ_box_segment): tile t is the 128 consecutive Morton cells
         // [128 t, 128 t + 128), one 8 x 4 x 4 box, and each chunk's A operand is
         // one TMA box copy (row r = x + 8 y + 32 z of the box).
         const bool box = !cross && occ_box_segment(H, count, N);
-        // rows past the list hold no operand: their groups of four are not copied
-        const int ngroups = box ? TC_M / 4 : (min(TC_M, count - r0) + 3) / 4;
+        // gathers: lanes per row (16 bytes each) and rows per group; rows past the list
+        // hold no operand, and groups of such rows are not copied
+        constexpr int LPR = Sh::UB / 16, RPG = 32 / LPR;
+        const int ngroups = (min(TC_M, count - r0) + RPG - 1) / RPG;
+        // accumulators in tensor memory: those of two offsets, but of one for the pairs
+        // of the widest tile, and of a cross-system tile beside its totals.  The i-th
+        // accumulator of the block, in the order they are read, is region i mod NR.
+        constexpr int NR = Sh::P3 && N == 128 && !cross ? 4 : 2;
         int X0 = 0, Y0 = 0, Z0 = 0;
         if (box) morton_decode((uint32_t)r0, X0, Y0, Z0);
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -509,7 +538,7 @@ struct KM2LTcg {
                 tc::mbar_init(bfull0 + 8 * s, 1);
                 tc::mbar_init(bempty0 + 8 * s, 1);
             }
-            for (int r = 0; r < 2; r++) {
+            for (int r = 0; r < NR; r++) {
                 tc::mbar_init(rfull0 + 8 * r, 1);
                 tc::mbar_init(rfree0 + 8 * r, 32 * Sh::EPI);
             }
@@ -543,12 +572,14 @@ struct KM2LTcg {
             // where the totals of a cross-system tile's runs wait (this thread's columns)
             const uint32_t ttot = tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(2 * N + c0);
             float2 run[Sh::COLS / 2];
-            uint32_t comp[Sh::COMP ? Sh::COLS / 2 : 1];
+            typedef typename std::conditional<N == 224, uint32_t, float2>::type Comp;
+            Comp comp[Sh::COMP ? Sh::COLS / 2 : 1];
 #pragma unroll
             for (int j = 0; j < Sh::COLS / 2; j++) {
                 run[j] = make_float2(0.0f, 0.0f);
-                if (Sh::COMP) comp[j] = 0u;
+                if (Sh::COMP) comp[j] = Comp{};
             }
+            constexpr int LDC = Sh::COMP && N == 64 ? 8 : 16;  // columns per read
             bool ok = true;
             // the row's source charge and factor, and the row means Kbar_o, are
             // fetched one offset ahead: the charge into registers, the means by the
@@ -568,9 +599,9 @@ struct KM2LTcg {
                 const float2 Q2 = make_float2(qs.x, qs.x), inv2 = make_float2(qs.y, qs.y);
                 const float *kb = kbs + (j & 1) * N + c0;
 #pragma unroll 1
-                for (int h = 0; h < Sh::ND; h++) {
-                const int r = (j * Sh::ND + h) & 1;
-                const uint32_t u = (uint32_t)((j * Sh::ND + h) >> 1) & 1u;
+                for (int h = 0; h < Sh::ACC; h++) {
+                const int r = (j * Sh::ACC + h) % NR;
+                const uint32_t u = (uint32_t)((j * Sh::ACC + h) / NR) & 1u;
                 if (ok && !tc::mbar_wait(rfull0 + 8 * r, u, TC_WAIT_CYCLES)) {
                     if (lane == 0) tc_wait_failed(prm.status, 4, l, j);
                     ok = false;
@@ -578,34 +609,24 @@ struct KM2LTcg {
                 tc::fence_after_sync();
                 const uint32_t taddr = tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(r * N + c0);
 #pragma unroll
-                for (int c = 0; c < Sh::COLS / 16; c++) {
-                    uint32_t v[16];
-                    tc::tmem_ld16(taddr + c * 16, v);
+                for (int c = 0; c < Sh::COLS / LDC; c++) {
+                    uint32_t v[LDC];
+                    if constexpr (LDC == 8) tc::tmem_ld8(taddr + c * LDC, v);
+                    else tc::tmem_ld16(taddr + c * LDC, v);
 #pragma unroll
-                    for (int e = 0; e < 16; e += 4) {
-                        // the offset's contribution with its monopole term Kbar Q
-                        const float4 m = *reinterpret_cast<const float4 *>(kb + c * 16 + e);
-                        const float2 m0 = make_float2(m.x, m.y), m1 = make_float2(m.z, m.w);
-                        float2 d0 = make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
-                        float2 d1 = make_float2(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
-                        if (h > 0) {
-                            d0 = __fmul2_rn(d0, inv2);
-                            d1 = __fmul2_rn(d1, inv2);
-                        } else if (Sh::SCALED) {
-                            // (the factor is a power of two: one rounding, of the sum)
-                            d0 = __ffma2_rn(m0, Q2, __fmul2_rn(d0, inv2));
-                            d1 = __ffma2_rn(m1, Q2, __fmul2_rn(d1, inv2));
-                        } else {
-                            d0 = __ffma2_rn(m0, Q2, d0);
-                            d1 = __ffma2_rn(m1, Q2, d1);
-                        }
-                        const int x = (c * 16 + e) / 2;
+                    for (int e = 0; e < LDC; e += 2) {
+                        // the offset's contribution, with its monopole term Kbar Q in the last
+                        // accumulator (the factor is a power of two: the sum is rounded once, and
+                        // once with the error that the last addition left)
+                        const int x = (c * LDC + e) / 2;
+                        const float2 m = *reinterpret_cast<const float2 *>(kb + c * LDC + e);
+                        float2 d = make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
                         if constexpr (Sh::COMP) {
-                            kahan_add(run[x], comp[x], d0);
-                            kahan_add(run[x + 1], comp[x + 1], d1);
+                            d = __ffma2_rn(d, inv2, comp_value(comp[x]));
+                            if (h == Sh::ACC - 1) d = __ffma2_rn(m, Q2, d);
+                            kahan_add(run[x], comp[x], d);
                         } else {
-                            run[x] = __fadd2_rn(run[x], d0);
-                            run[x + 1] = __fadd2_rn(run[x + 1], d1);
+                            run[x] = __fadd2_rn(run[x], __ffma2_rn(m, Q2, Sh::SCALED ? __fmul2_rn(d, inv2) : d));
                         }
                     }
                 }
@@ -666,7 +687,7 @@ struct KM2LTcg {
 #pragma unroll
                         for (int e = 0; e < Sh::COLS / 2; e++) {
                             run[e] = make_float2(0.0f, 0.0f);
-                            if (Sh::COMP) comp[e] = 0u;
+                            if (Sh::COMP) comp[e] = Comp{};
                         }
                     }
                 }
@@ -684,29 +705,33 @@ struct KM2LTcg {
             if constexpr (Gh::SETREG) tc::setmaxnreg_dec<72>();
             if (warp < Gh::WA + Gh::PW) {
                 // ---- A producers; with one ring (UNI) the first lane also issues the
-                //      stage's B copies.  Gather: lane = 8 (row within a group of four) +
-                //      16-byte piece; warp pw takes the groups pw + PW i.  A stage is
-                //      signalled once its copies are complete and fenced, G - 1 stages
-                //      later. ----
+                //      stage's B copies.  Gather: lane = LPR (row within a group) + 16-byte
+                //      piece; warp pw takes the groups pw + PW i.  A stage is signalled once
+                //      its copies are complete and fenced, G - 1 stages later. ----
                 const int pw = warp - Gh::WA;
                 const bool lead = pw == 0 && lane == 0;
                 if (lead) {
                     if (box) tc::tensormap_acquire(&prm.phi[l]);
                     if (Gh::UNI) tc::tensormap_acquire(&prm.k);
                 }
-                constexpr int RI = 32 / Gh::PW;
-                const int piece = lane & 7, rsub = lane >> 3;
+                constexpr int RI = TC_M / RPG / Gh::PW;
+                const int piece = lane % LPR, rsub = lane / LPR;
                 // groups of this warp that hold rows of the tile
                 const int ni = box ? 0 : (ngroups - pw + Gh::PW - 1) / Gh::PW;
                 int g[RI];
-                uint32_t place[2 / Gh::PW];  // of the groups i (mod 2 / PW), 1 KB a further pair of groups
+                // shared-memory places of the first NPL groups, the further ones 1 KB a pair
+                // of four-row groups (128-byte rows), 1 KB a group here (64-byte rows, PW = 2)
+                constexpr int NPL = Sh::P3 ? 1 : 2 / Gh::PW;
+                static_assert(!Sh::P3 || Gh::PW == 2, "places of the 64-byte rows");
+                uint32_t place[NPL];
                 if (!box) {
 #pragma unroll
-                    for (int i = 0; i < RI; i++) g[i] = rowG[4 * (pw + Gh::PW * i) + rsub];
+                    for (int i = 0; i < RI; i++) g[i] = rowG[RPG * (pw + Gh::PW * i) + rsub];
 #pragma unroll
-                    for (int i = 0; i < 2 / Gh::PW; i++) {
-                        const int r = 4 * (pw + Gh::PW * i) + rsub;
-                        place[i] = (uint32_t)(r * 128 + ((piece ^ (r & 7)) << 4));
+                    for (int i = 0; i < NPL; i++) {
+                        const int r = RPG * (pw + Gh::PW * i) + rsub;
+                        // 128-byte swizzle: piece ^ (row mod 8); 64-byte: piece ^ (row / 2 mod 4)
+                        place[i] = (uint32_t)(r * Sh::UB + ((piece ^ (Sh::P3 ? (r >> 1) & 3 : r & 7)) << 4));
                     }
                 }
                 const char *src0 = prm.op + 16 * piece;
@@ -716,6 +741,7 @@ struct KM2LTcg {
                 for (int i = i0; i < i1 && !failed; i++) {
                     const Off f = list_offset(ord, par, i);
                     const int delta = (((f.spar * P + f.dZ) * P + f.dY) * P + f.dX) * Sh::RC;
+#pragma unroll 1
                     for (int kc = 0; kc < Sh::KC; kc++, it++) {
                         const int s = it % Gh::SA;
                         const uint32_t ph = (uint32_t)(it / Gh::SA) & 1u;
@@ -725,30 +751,36 @@ struct KM2LTcg {
                             break;
                         }
                         const uint32_t st = abase + s * Gh::ASTAGE, fb = afull0 + 8 * s;
-                        const int nch = kc < Sh::FC && Sh::LO ? 2 : 1;  // chunks of this stage (a tail holds hi and lo)
+                        const int nch = stage_chunks(kc);
                         if (lead && (box || Gh::UNI)) {
-                            tc::mbar_expect_tx(fb, (uint32_t)(nch * ((box ? TC_ABYTES : 0) + (Gh::UNI ? Sh::BBYTES : 0))));
+                            tc::mbar_expect_tx(fb, (uint32_t)(nch * ((box ? Sh::ABYTES : 0) + (Gh::UNI ? Sh::BBYTES : 0))));
                             last_phase[s] = (int)ph;
                             if (box) {
                                 const int cX = X0 + 1 + f.dX, cY = Y0 + 1 + f.dY, cZ = Z0 + 1 + f.dZ;
-                                tc::tma_load_5d(st, &prm.phi[l], fb, 128 * kc, cX, cY, cZ, f.spar);
-                                if (nch == 2) tc::tma_load_5d(st + TC_ABYTES, &prm.phi[l], fb, 128 * kc + 64, cX, cY, cZ, f.spar);
+#pragma unroll
+                                for (int t = 0; t < Sh::NCH; t++)
+                                    if (t < nch)
+                                        tc::tma_load_5d(st + t * Sh::ABYTES, &prm.phi[l], fb, (Sh::NCX * kc + t) * (Sh::UB / 2), cX,
+                                                        cY, cZ, f.spar);
                             }
                             if (Gh::UNI && !(prm.inject_stall && it == 0)) {  // inject: armed, never filled
                                 const uint32_t stb = bbase + s * Gh::BSTAGE;
-                                tc::tma_load_3d(stb, &prm.k, fb, 128 * kc, 0, f.oi);
-                                if (nch == 2) tc::tma_load_3d(stb + Sh::BBYTES, &prm.k, fb, 128 * kc + 64, 0, f.oi);
+#pragma unroll
+                                for (int t = 0; t < Sh::NCH; t++)
+                                    if (t < nch)
+                                        tc::tma_load_3d(stb + t * Sh::BBYTES, &prm.k, fb, (Sh::NCX * kc + t) * (Sh::UB / 2), 0, f.oi);
                             }
                         }
                         if (box) continue;
-                        const int d = delta + 2 * kc;
+                        const int d = delta + Sh::NCX * kc;
 #pragma unroll
                         for (int i = 0; i < RI; i++) {
                             if (i >= ni) break;
-                            const char *src = src0 + (int64_t)(g[i] + d) * 128;
-                            const uint32_t to = st + place[i % (2 / Gh::PW)] + 1024 * (i / (2 / Gh::PW));
-                            tc::cp_async16(to, src);
-                            if (nch == 2) tc::cp_async16(to + TC_ABYTES, src + 128);
+                            const char *src = src0 + (int64_t)(g[i] + d) * Sh::UB;
+                            const uint32_t to = st + place[i % NPL] + 1024 * (i / NPL);
+#pragma unroll
+                            for (int t = 0; t < Sh::NCH; t++)
+                                if (t < nch) tc::cp_async16(to + t * Sh::ABYTES, src + t * Sh::UB);
                         }
                         tc::cp_async_commit();
                         tc::cp_async_wait_pending<Gh::G - 1>();  // stages <= it - G + 1 have landed
@@ -789,12 +821,13 @@ struct KM2LTcg {
                                 break;
                             }
                             const uint32_t st = bbase + s * Gh::BSTAGE, fb = bfull0 + 8 * s;
-                            const int nch = kc < Sh::FC && Sh::LO ? 2 : 1;
+                            const int nch = stage_chunks(kc);
                             tc::mbar_expect_tx(fb, (uint32_t)(nch * Sh::BBYTES));
                             last_phase[s] = (int)ph;
                             if (prm.inject_stall && it == 0) continue;  // armed, never filled (test hook)
-                            tc::tma_load_3d(st, &prm.k, fb, 128 * kc, 0, oi);
-                            if (nch == 2) tc::tma_load_3d(st + Sh::BBYTES, &prm.k, fb, 128 * kc + 64, 0, oi);
+#pragma unroll
+                            for (int t = 0; t < Sh::NCH; t++)
+                                if (t < nch) tc::tma_load_3d(st + t * Sh::BBYTES, &prm.k, fb, (Sh::NCX * kc + t) * (Sh::UB / 2), 0, oi);
                         }
                     }
                     if (failed) {
@@ -805,22 +838,27 @@ struct KM2LTcg {
                     }
                 }
             } else if (warp == Gh::WM) {
-                // ---- MMA issuer: the j-th accumulator of the block is TMEM region j & 1 ----
+                // ---- MMA issuer: the j-th offset of the block accumulates into regions ACC j mod NR and up ----
                 if (lane == 0) {
                     const uint32_t idesc = MODE == TC_BF16X3 ? tc::idesc_bf16(TC_M, N) : tc::idesc_f16(TC_M, N);
                     bool failed = false;
-                    for (int j = 0; j < (i1 - i0) * Sh::ND && !failed; j++) {
-                        const int r = j & 1;
-                        const uint32_t u = (uint32_t)(j >> 1) & 1u;
-                        if (!tc::mbar_wait(rfree0 + 8 * r, u ^ 1u, TC_WAIT_CYCLES)) {
+                    for (int j = 0; j < i1 - i0 && !failed; j++) {
+                        // the accumulators of the offset: d0 of the leading (or all) products, read
+                        // last, d1 of the others
+                        const int u0 = j * Sh::ACC, u1 = u0 + Sh::ACC - 1;
+                        const uint32_t d1 = tmem + (uint32_t)(u0 % NR * N), d0 = tmem + (uint32_t)(u1 % NR * N);
+                        auto region_free = [&](int i) {
+                            if (tc::mbar_wait(rfree0 + 8 * (i % NR), ((uint32_t)(i / NR) & 1u) ^ 1u, TC_WAIT_CYCLES)) return true;
                             tc_wait_failed(prm.status, 2, l, j);
+                            return false;
+                        };
+                        if (!region_free(u0)) {
                             failed = true;
                             break;
                         }
-                        const uint32_t d = tmem + (uint32_t)(r * N);
-#pragma unroll
-                        for (int ks0 = 0; ks0 < Sh::KC / Sh::ND; ks0++) {
-                            const int it = Sh::KC / Sh::ND * j + ks0, kc = it % Sh::KC;
+#pragma unroll (Sh::P3 ? 1 : Sh::KC)
+                        for (int kc = 0; kc < Sh::KC; kc++) {
+                            const int it = Sh::KC * j + kc;
                             const int sa = it % Gh::SA, sb = it % Gh::SB;
                             if (!tc::mbar_wait(afull0 + 8 * sa, (uint32_t)(it / Gh::SA) & 1u, TC_WAIT_CYCLES) ||
                                 (!Gh::UNI && !tc::mbar_wait(bfull0 + 8 * sb, (uint32_t)(it / Gh::SB) & 1u, TC_WAIT_CYCLES))) {
@@ -829,29 +867,60 @@ struct KM2LTcg {
                                 break;
                             }
                             tc::fence_after_sync();
-                            // the stage's hi and lo parts: two chunks, or the halves of a tail chunk
-                            const bool full = kc < Sh::FC;
-                            const uint32_t ah = abase + sa * Gh::ASTAGE, al = ah + (full ? TC_ABYTES : 64);
-                            const uint32_t bh = bbase + sb * Gh::BSTAGE, bl = bh + (full ? Sh::BBYTES : 64);
-                            // 32 bytes of K (16 values) per MMA; the small products of the
-                            // stage first, so that they meet an accumulator of their own size
-                            if (Sh::LO) {
+                            const uint32_t a0 = abase + sa * Gh::ASTAGE, b0 = bbase + sb * Gh::BSTAGE;
+                            // 32 bytes of K (16 values) per MMA
+                            if constexpr (Sh::P3) {
+                                // the smaller products into one accumulator, smallest first; the
+                                // leading ones into another, where every sum is exact (KSplit) and
+                                // which may still be read while the first stage's others run
 #pragma unroll
-                                for (int s = 0; s < 4; s++) {
-                                    if (s >= 2 && !full) break;
-                                    tc::mma_f16(d, tc::desc_sw128(ah + 32 * s), tc::desc_sw128(bl + 32 * s), idesc, (ks0 | s) != 0);
-                                    tc::mma_f16(d, tc::desc_sw128(al + 32 * s), tc::desc_sw128(bh + 32 * s), idesc, 1u);
+                                for (int s = 0; s < 2; s++) {
+                                    uint64_t A[3], B[3];
+#pragma unroll
+                                    for (int t = 0; t < 3; t++) {
+                                        A[t] = tc::desc_sw64(a0 + t * Sh::ABYTES + 32 * s);
+                                        B[t] = tc::desc_sw64(b0 + t * Sh::BBYTES + 32 * s);
+                                    }
+                                    tc::mma_f16(d1, A[2], B[0], idesc, (kc | s) != 0);
+                                    tc::mma_f16(d1, A[0], B[2], idesc, 1u);
+                                    tc::mma_f16(d1, A[1], B[1], idesc, 1u);
+                                    tc::mma_f16(d1, A[1], B[0], idesc, 1u);
+                                    tc::mma_f16(d1, A[0], B[1], idesc, 1u);
                                 }
-                            }
+                                if (kc == 0) {
+                                    if (!region_free(u1)) {
+                                        failed = true;
+                                        break;
+                                    }
+                                    tc::fence_after_sync();
+                                }
 #pragma unroll
-                            for (int s = 0; s < 4; s++)
-                                if (s < 2 || full)
-                                    tc::mma_f16(d, tc::desc_sw128(ah + 32 * s), tc::desc_sw128(bh + 32 * s), idesc,
-                                                Sh::LO || (ks0 | s) != 0);
+                                for (int s = 0; s < 2; s++)
+                                    tc::mma_f16(d0, tc::desc_sw64(a0 + 32 * s), tc::desc_sw64(b0 + 32 * s), idesc, (kc | s) != 0);
+                            } else {
+                                // the stage's hi and lo parts: two chunks, or the halves of a tail
+                                // chunk; the small products of the stage first, so that they meet an
+                                // accumulator of their own size
+                                const bool full = kc < Sh::FC;
+                                const uint32_t al = a0 + (full ? Sh::ABYTES : 64), bl = b0 + (full ? Sh::BBYTES : 64);
+                                if (Sh::LO) {
+#pragma unroll
+                                    for (int s = 0; s < 4; s++) {
+                                        if (s >= 2 && !full) break;
+                                        tc::mma_f16(d0, tc::desc_sw128(a0 + 32 * s), tc::desc_sw128(bl + 32 * s), idesc, (kc | s) != 0);
+                                        tc::mma_f16(d0, tc::desc_sw128(al + 32 * s), tc::desc_sw128(b0 + 32 * s), idesc, 1u);
+                                    }
+                                }
+#pragma unroll
+                                for (int s = 0; s < 4; s++)
+                                    if (s < 2 || full)
+                                        tc::mma_f16(d0, tc::desc_sw128(a0 + 32 * s), tc::desc_sw128(b0 + 32 * s), idesc,
+                                                    Sh::LO || (kc | s) != 0);
+                            }
                             tc::mma_commit(aempty0 + 8 * sa);
                             if (!Gh::UNI) tc::mma_commit(bempty0 + 8 * sb);
                         }
-                        if (!failed) tc::mma_commit(rfull0 + 8 * r);
+                        for (int i = u0; i <= u1 && !failed; i++) tc::mma_commit(rfull0 + 8 * (i % NR));
                     }
                     if (failed) atomicOr(prm.status, ST_TIMEOUT);
                     tc::mma_commit(done);  // always: the deallocation waits on it
@@ -909,13 +978,19 @@ __global__ void __launch_bounds__(KTcReduce::BS) k_tc_reduce(const __grid_consta
 // layout (cells [c0, c1), all levels in one stretch).
 // F16: x s = hi + lo with hi = half(x s), lo = half(x s - hi), both rounded to
 // nearest, s the power of two that takes the cell's largest |x| into [2^14,
-// 2^15): 11 + 11 significant bits, and an absolute floor of 2^-25 against that
-// maximum, so every value keeps an error below 2^-24 of itself or 2^-39 of the
-// cell's largest.  The accumulated products are scaled back by the cell's
+// 2^15): the remainder is at most 2^-11 of x and keeps 11 bits, so that a value is
+// off by at most 2^-23 of itself, or 2^-39 of the cell's largest (the type's
+// subnormal floor).  The accumulated products are scaled back by the cell's
 // factor 1/(s TC_KSCALE) where they are added up, all exact powers of two.
+// Three parts (P3): x s = x0 + x1 + x2, x0 the multiple of 2^7 next to x s (an
+// integer of at most 8 bits, times 2^7), x1 and x2 the remainder's two halves: all of
+// an FP32 value's bits down to 2^-25 against a largest of 2^14 and more.  The leading
+// parts' products are integers below 2^16 of one unit (2^7 times the kernel row's),
+// so that their sum over up to 224 values stays below 2^24 units: whatever the order
+// and the rounding of the tensor cores' additions, it is exact.
 // BF16: hi = bf16(x), lo = bf16(x - hi), unscaled (the type has FP32's range).
 // qsc: per cell (total charge, factor).  Infinite or NaN grid charges stay so.
-template <int MODE>
+template <int MODE, bool P3>
 struct KSplit {
     static constexpr int BS = 256, MINB = 0;
     const float *__restrict__ phi;   // the cells' values from cell 0 of the layout
@@ -929,7 +1004,7 @@ struct KSplit {
     __device__ __forceinline__ void run(const int bid_, const int nblk_) const {
         typedef typename std::conditional<MODE == TC_BF16X3, __nv_bfloat162, __half2>::type T2;
         const int lane = threadIdx.x & 31;
-        const int row_bytes = 256 * fc + (tail ? 128 : 0);
+        const int row_bytes = P3 ? 6 * ((p3 + 31) / 32 * 32) : 256 * fc + (tail ? 128 : 0);
         for (int64_t c = c0 + ((bid_ * (int64_t)BS + threadIdx.x) >> 5); c < c1; c += ((int64_t)nblk_ * BS) >> 5) {
             const float *src = phi + c * p3;
             float2 v[4];
@@ -951,6 +1026,23 @@ struct KSplit {
                 inv = __uint_as_float((uint32_t)(254 - min(f, 253)) << 23) * (f > 253 ? 0.5f / TC_KSCALE : 1.0f / TC_KSCALE);
             }
             if (lane == 0) qsc[c] = make_float2(qlev[c], inv);
+            if constexpr (P3) {
+                // values 2 lane + 64 k: stage 2 k + lane / 16 of 32 values, 192 bytes each
+                char *dst = op + c * row_bytes + 192 * (lane >> 4) + 4 * (lane & 15);
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    if (2 * lane + 64 * k >= (p3 + 31) / 32 * 32) break;
+                    const float x = v[k].x * s, y = v[k].y * s;
+                    const float x0 = rintf(x * 0x1p-7f) * 0x1p7f, y0 = rintf(y * 0x1p-7f) * 0x1p7f;
+                    const __half2 a = __floats2half2_rn(x0, y0), b = __floats2half2_rn(x - x0, y - y0);
+                    const float2 f = __half22float2(b);
+                    char *to = dst + 384 * k;
+                    *reinterpret_cast<__half2 *>(to) = a;
+                    *reinterpret_cast<__half2 *>(to + 64) = b;
+                    *reinterpret_cast<__half2 *>(to + 128) = __floats2half2_rn((x - x0) - f.x, (y - y0) - f.y);
+                }
+                continue;
+            }
             char *dst = op + c * row_bytes + 4 * lane;
 #pragma unroll
             for (int k = 0; k < 4; k++) {
@@ -973,8 +1065,8 @@ struct KSplit {
         }
     }
 };
-template <int MODE>
-__global__ void __launch_bounds__(KSplit<MODE>::BS) k_split(const __grid_constant__ KSplit<MODE> k) {
+template <int MODE, bool P3>
+__global__ void __launch_bounds__(KSplit<MODE, P3>::BS) k_split(const __grid_constant__ KSplit<MODE, P3> k) {
     k.run(blockIdx.x, gridDim.x);
 }
 
@@ -982,12 +1074,13 @@ __global__ void __launch_bounds__(KSplit<MODE>::BS) k_split(const __grid_constan
 // mean split off, computed in FP64: one warp per (offset, a).  KtT: Kt_o^T
 // [o][b][a] and Kbar [o][a] in the plan's type (SIMT contraction); row: the
 // row's chunks for the tensor cores (hi, lo as the operand copy's, scaled by
-// TC_KSCALE or in bfloat16), kbar_tc [o][p3s].  Offsets of adjacent cells stay
+// TC_KSCALE or in bfloat16; three parts: the leading one in at most 8 bits of a unit
+// of the row's own), kbar_tc [o][p3s].  Offsets of adjacent cells stay
 // zero (the tables are cleared first).
 template <typename real>
 struct KTables {
     double tau[FMM_MAXP];
-    int p, power, ncomp, bf16, p3s, fc, tail;
+    int p, power, ncomp, bf16, three, p3s, fc, tail;
     real *KtT, *Kbar;
     char *row;       // nullptr: no tensor-core tables
     float *kbar_tc;
@@ -1017,6 +1110,24 @@ __global__ void __launch_bounds__(256) k_tables(const __grid_constant__ KTables<
     for (int b = lane; b < p3; b += 32) t.KtT[((int64_t)oc * p3 + b) * p3 + a] = (real)(value(b) - mean);
     if (!t.row) return;
     if (lane == 0) t.kbar_tc[oc * t.p3s + a] = (float)mean;
+    if (t.three) {
+        double m = 0.0;
+        for (int b = lane; b < p3; b += 32) m = fmax(m, fabs(value(b) - mean));
+        for (int o = 16; o >= 1; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        int e;
+        frexp(m * (double)TC_KSCALE, &e);
+        const double unit = ldexp(1.0, e - 8);  // the row's largest: 128 to 256 units
+        char *row = t.row + ((int64_t)oc * t.p3s + a) * 6 * t.p3s;
+        for (int b = lane; b < p3; b += 32) {
+            const double u = (value(b) - mean) * (double)TC_KSCALE, u0 = rint(u / unit) * unit;
+            const __half x = __float2half_rn((float)(u - u0));
+            char *to = row + 192 * (b / 32) + 2 * (b % 32);
+            *reinterpret_cast<__half *>(to) = __float2half_rn((float)u0);
+            *reinterpret_cast<__half *>(to + 64) = x;
+            *reinterpret_cast<__half *>(to + 128) = __float2half_rn((float)(u - u0 - (double)__half2float(x)));
+        }
+        return;
+    }
     char *row = t.row + ((int64_t)oc * t.p3s + a) * (256 * t.fc + (t.tail ? 128 : 0));
     for (int b = lane; b < p3; b += 32) {
         const double v = value(b) - mean;
@@ -1056,37 +1167,42 @@ int tc_padded(int p3) { return (p3 + 31) / 32 * 32; }
 // a rest of at most 32 values in one chunk
 static int tc_full(int p3) { return p3 % 64 == 0 || p3 % 64 > 32 ? (p3 + 63) / 64 : p3 / 64; }
 static int tc_tail(int p3) { return p3 > 64 * tc_full(p3) ? 32 : 0; }
-int tc_row_bytes(int p3) { return 256 * tc_full(p3) + (tc_tail(p3) ? 128 : 0); }
+static bool tc_three(int p3, int mode) { return mode == FMM_TC_F32 && p3 > 64; }
+int tc_row_bytes(int p3, int mode) {
+    return tc_three(p3, mode) ? 6 * tc_padded(p3) : 256 * tc_full(p3) + (tc_tail(p3) ? 128 : 0);
+}
+int tc_chunk_bytes(int p3, int mode) { return tc_three(p3, mode) ? 64 : 128; }
 
 static CUtensorMapDataType op_type(int mode) {
     return mode == FMM_TC_BF16X3 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
 }
-static int encode(CUtensorMap *m, int mode, int rank, const void *base, const cuuint64_t *dims,
+static int encode(CUtensorMap *m, int p3, int mode, int rank, const void *base, const cuuint64_t *dims,
                   const cuuint64_t *strides, const cuuint32_t *box) {
     auto enc = encode_fn();
     if (!enc) return FMM_ERR_CUDA;
     const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     CUresult r = enc(m, op_type(mode), rank, (void *)base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     tc_three(p3, mode) ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? FMM_OK : FMM_ERR_CUDA;
 }
 
 // Box map of level l of the operand copy: dims (row values, P x, P y, P z, 8
 // parity), box (one chunk, 8, 4, 4, 1).  Every box the kernel loads lies inside.
-static int encode_phi_map(CUtensorMap *m, const void *base, int l, int row_bytes, int mode) {
-    const cuuint64_t P = ((cuuint64_t)1 << (l - 1)) + 2, rb = (cuuint64_t)row_bytes;
+static int encode_phi_map(CUtensorMap *m, const void *base, int l, int p3, int mode) {
+    const cuuint64_t P = ((cuuint64_t)1 << (l - 1)) + 2, rb = (cuuint64_t)tc_row_bytes(p3, mode);
     const cuuint64_t dims[5] = {rb / 2, P, P, P, 8}, strides[4] = {rb, rb * P, rb * P * P, rb * P * P * P};
-    const cuuint32_t box[5] = {64, 8, 4, 4, 1};
-    return encode(m, mode, 5, base, dims, strides, box);
+    const cuuint32_t box[5] = {(cuuint32_t)tc_chunk_bytes(p3, mode) / 2, 8, 4, 4, 1};
+    return encode(m, p3, mode, 5, base, dims, strides, box);
 }
 
 // Kernel-table map: dims (row values, p3s a, 343 offsets), box (one chunk, p3s, 1).
 int tc_encode_kernel_map(void *map, const void *base, int p3, int mode) {
-    const cuuint64_t rb = (cuuint64_t)tc_row_bytes(p3), p3s = (cuuint64_t)tc_padded(p3);
+    const cuuint64_t rb = (cuuint64_t)tc_row_bytes(p3, mode), p3s = (cuuint64_t)tc_padded(p3);
     const cuuint64_t dims[3] = {rb / 2, p3s, 343}, strides[2] = {rb, rb * p3s};
-    const cuuint32_t box[3] = {64, (cuuint32_t)p3s, 1};
-    return encode((CUtensorMap *)map, mode, 3, base, dims, strides, box);
+    const cuuint32_t box[3] = {(cuuint32_t)tc_chunk_bytes(p3, mode) / 2, (cuuint32_t)p3s, 1};
+    return encode((CUtensorMap *)map, p3, mode, 3, base, dims, strides, box);
 }
 
 size_t tc_map_bytes() { return sizeof(CUtensorMap); }
@@ -1103,6 +1219,7 @@ int build_tables(int p, double grid_scale, int power, int ncomp, int mode, real 
     t.power = power;
     t.ncomp = ncomp;
     t.bf16 = mode == FMM_TC_BF16X3;
+    t.three = tc_three(p3, mode);
     t.p3s = tc_padded(p3);
     t.fc = tc_full(p3);
     t.tail = tc_tail(p3);
@@ -1114,7 +1231,7 @@ int build_tables(int p, double grid_scale, int power, int ncomp, int mode, real 
     if (cudaMemset(KtT, 0, no * p3 * p3 * sizeof(real)) != cudaSuccess ||
         cudaMemset(Kbar, 0, no * p3 * sizeof(real)) != cudaSuccess)
         return FMM_ERR_CUDA;
-    if (rows && (cudaMemset(rows, 0, no * t.p3s * tc_row_bytes(p3)) != cudaSuccess ||
+    if (rows && (cudaMemset(rows, 0, no * t.p3s * tc_row_bytes(p3, mode)) != cudaSuccess ||
                  cudaMemset(kbar_tc, 0, no * t.p3s * sizeof(float)) != cudaSuccess))
         return FMM_ERR_CUDA;
     k_tables<real><<<dim3((unsigned)no, (p3 + 7) / 8), 256>>>(t);
@@ -1172,7 +1289,7 @@ int tc_set_attributes(int p3, int mode) {
     const int p3s = tc_padded(p3);
     return mode == FMM_TC_BF16X3  ? set_attributes_mode<TC_BF16X3>(p3s)
            : mode == FMM_TC_F16X1 ? set_attributes_mode<TC_F16X1>(p3s)
-           : mode == FMM_TC_F16X3C ? set_attributes_mode<TC_F16X3C>(p3s)
+           : mode == FMM_TC_F32 ? set_attributes_mode<TC_F32>(p3s)
                                   : set_attributes_mode<TC_F16X3>(p3s);
 }
 
@@ -1187,17 +1304,17 @@ static int launch_tcg_mode(int p3s, const TcgParams &prm, int blocks, int comp, 
     }
 }
 
-template <int MODE>
+template <int MODE, bool P3 = false>
 static void launch_split(const Ptrs<float> &P, int64_t c0, int64_t c1, int p3, int blocks, cudaStream_t st, Tracer &tr) {
-    launch_k(tr, FMM_TAG(S_SPLIT_TC, 0), k_split<MODE>,
-             KSplit<MODE>{P.phi, P.qlev, P.qsc, P.op, c0, c1, p3, tc_full(p3), tc_tail(p3)}, blocks, KSplit<MODE>::BS, 0,
-             st);
+    typedef KSplit<MODE, P3> K;
+    launch_k(tr, FMM_TAG(S_SPLIT_TC, 0), k_split<MODE, P3>,
+             K{P.phi, P.qlev, P.qsc, P.op, c0, c1, p3, tc_full(p3), tc_tail(p3)}, blocks, K::BS, 0, st);
 }
 
 int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const void *k_map, const float *kbar,
                   int lmin, int mode, int inject, float *loc, int spow, bool split, int comp, cudaStream_t st,
                   Tracer &tr) {
-    const int depth = g.depth, p3 = g.p3, p3s = tc_padded(p3), rb = tc_row_bytes(p3);
+    const int depth = g.depth, p3 = g.p3, p3s = tc_padded(p3), rb = tc_row_bytes(p3, mode);
     tr.begin(FMM_STAGE_M2L, st);
     if (split) {
         // grid-stride over the cells, a warp each; small systems take a small
@@ -1205,6 +1322,7 @@ int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const 
         const int64_t c0 = W.q_level[lmin], c1 = W.q_level[depth + 1];
         const int nbs = (int)std::min<int64_t>(152 * 8, std::max<int64_t>(1, (c1 - c0 + 7) / 8));
         if (mode == FMM_TC_BF16X3) launch_split<TC_BF16X3>(P, c0, c1, p3, nbs, st, tr);
+        else if (tc_three(p3, mode)) launch_split<TC_F32, true>(P, c0, c1, p3, nbs, st, tr);
         else launch_split<TC_F16X3>(P, c0, c1, p3, nbs, st, tr);
         tr.count();
     }
@@ -1257,7 +1375,7 @@ int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const 
     for (int l = lmin; l <= depth && !rc; l++) {
         prm.loc_off[l] = W.loc_level[l];
         prm.q_off[l] = W.q_level[l];
-        if (l >= 4) rc = encode_phi_map(&prm.phi[l], P.op + W.q_level[l] * rb, l, rb, mode);
+        if (l >= 4) rc = encode_phi_map(&prm.phi[l], P.op + W.q_level[l] * rb, l, p3, mode);
         if (tc_parts(l, depth) > 1) {
             const int v = red.nlev++;
             tc_part_place(l, p3, &prm.part_off[l], &prm.part_stride[l]);
@@ -1277,7 +1395,7 @@ int launch_m2l_tc(const Geom &g, const Ptrs<float> &P, const WsLayout &W, const 
     prm.inject_stall = inject == FMM_INJECT_TC_STALL;
     rc = mode == FMM_TC_BF16X3  ? launch_tcg_mode<TC_BF16X3>(p3s, prm, blocks, comp, st, tr)
          : mode == FMM_TC_F16X1 ? launch_tcg_mode<TC_F16X1>(p3s, prm, blocks, comp, st, tr)
-         : mode == FMM_TC_F16X3C ? launch_tcg_mode<TC_F16X3C>(p3s, prm, blocks, comp, st, tr)
+         : mode == FMM_TC_F32 ? launch_tcg_mode<TC_F32>(p3s, prm, blocks, comp, st, tr)
                                 : launch_tcg_mode<TC_F16X3>(p3s, prm, blocks, comp, st, tr);
     tr.count();
     if (!rc && red.nlev > 0) {
@@ -1299,7 +1417,7 @@ int tc_cross_records(const std::vector<TcXSys> &sys, const std::vector<int> &dep
     const int p3s = tc_padded(p3);
     const int nseg = 8 * (lmax - lmin + 1);
     // coordinates and systems fit the list's entries, chunks of the workspace a gather's row index
-    if (lmax >= 5 || ns >= (1 << 19) || ws_bytes / 128 > INT32_MAX) return FMM_ERR_UNSUPPORTED;
+    if (lmax >= 5 || ns >= (1 << 19) || ws_bytes / tc_chunk_bytes(p3, mode) > INT32_MAX) return FMM_ERR_UNSUPPORTED;
     // the lists: every cell of every system with that level, system-major
     std::vector<int> cnt(nseg, 0), tiles(nseg + 1, 0), first(nseg, 0), list;
     for (int sg = 0; sg < nseg; sg++) {
@@ -1357,7 +1475,7 @@ int tc_cross_records(const std::vector<TcXSys> &sys, const std::vector<int> &dep
         t.rec = &one;
         int rc = mode == FMM_TC_BF16X3  ? record_tcx_mode<TC_BF16X3>(p3s, prm, tiles[nseg], c, t)
              : mode == FMM_TC_F16X1 ? record_tcx_mode<TC_F16X1>(p3s, prm, tiles[nseg], c, t)
-             : mode == FMM_TC_F16X3C ? record_tcx_mode<TC_F16X3C>(p3s, prm, tiles[nseg], c, t)
+             : mode == FMM_TC_F32 ? record_tcx_mode<TC_F32>(p3s, prm, tiles[nseg], c, t)
                                     : record_tcx_mode<TC_F16X3>(p3s, prm, tiles[nseg], c, t);
         if (rc) return rc;
         out.push_back(std::move(one[0]));
