@@ -137,11 +137,11 @@ void fmm_opts_default(fmm_opts_t *opts);
  *   periodic 0: open boundary; 1: periodic box (§4.2).
  *   opts    host, nullable (defaults).
  *   max_n   largest particle count fmm_eval will be given with this plan.
- * Builds in FP64 on the host: the p-division points and Lagrange coefficients,
- * the two child->parent shift matrices (eq. trans), the 316 unit-cell
- * bilinear-form kernels 1/|a - (o + b)| for |o|_inf <= 3 (eq. bilinear), and
- * (periodic) the Ewald lattice kernel of the box's far images; uploads them to
- * the current device.  The plan owns those tables (device memory freed by
+ * Builds in FP64: on the host the p-division points and Lagrange coefficients,
+ * the two child->parent shift matrices (eq. trans) and (periodic) the Ewald
+ * lattice kernel of the box's far images, uploaded to the current device; on the
+ * device the 316 unit-cell bilinear-form kernels 1/|a - (o + b)| for |o|_inf <= 3
+ * (eq. bilinear).  The call waits until they are there.  The plan owns those tables (device memory freed by
  * fmm_plan_destroy).  With opts.shift_free it also builds the per-axis
  * shift_{S->C} matrices and computes the App. A.2 forms on the device (FP64,
  * synchronous).  Errors: FMM_ERR_ARG, FMM_ERR_OOM, FMM_ERR_CUDA,
@@ -163,6 +163,18 @@ void fmm_plan_destroy(fmm_plan_t plan);
 int fmm_workspace_size(fmm_plan_t plan, int64_t n, size_t *bytes);
 
 /*
+ * fmm_workspace_minimum — the smallest workspace fmm_eval accepts for n
+ * particles.  Less than fmm_workspace_size for FP32 plans of orders 3..6 only:
+ * with fewer bytes than fmm_workspace_size the workspace holds no split copy of the
+ * grid charges, and the evaluation takes FP32 multiply-adds in place of the
+ * tensor cores (slower; same errors, other last digits).  So the size of the
+ * workspace, and nothing else, selects the form; give every call at least
+ * fmm_workspace_size bytes for results that are the same bit for bit.
+ * Errors: FMM_ERR_ARG.
+ */
+int fmm_workspace_minimum(fmm_plan_t plan, int64_t n, size_t *bytes);
+
+/*
  * fmm_eval — one evaluation of §2.2 (+ §2.3 split, §4.2 periodic).
  *   n          number of particles, 0 <= n <= max_n (n = 0: energy 0).
  *   pos        device, float32 (n,3).  Open form: every position must lie in
@@ -171,7 +183,10 @@ int fmm_workspace_size(fmm_plan_t plan, int64_t n, size_t *bytes);
  *   potential  device, (n) float32 (float64 for FP64 plans), nullable.
  *   energy     device, 1 double, nullable.
  *   forces     device, (n,3) float32 (float64 for FP64 plans), nullable.
- *   workspace  device, >= fmm_workspace_size(plan, n) bytes, 256-byte aligned.
+ *   workspace  device, 256-byte aligned, of workspace_bytes bytes: >=
+ *              fmm_workspace_size(plan, n), or, where device memory is short, >=
+ *              fmm_workspace_minimum(plan, n) (a slower form, see there; fewer:
+ *              FMM_ERR_WORKSPACE).
  *   stream     cudaStream_t as void*.
  * With opts.sync = 1 the call waits for the device and returns the device
  * status (FMM_ERR_OUT_OF_BOX, FMM_ERR_NONFINITE, FMM_ERR_SPLIT_OVERFLOW);
@@ -322,8 +337,11 @@ int fmm_batch_create(fmm_batch_t *batch, int nsys, const double *boxes, const in
                      int periodic, const fmm_opts_t *opts, const int64_t *max_n);
 void fmm_batch_destroy(fmm_batch_t batch);
 
-/* Bytes of device workspace for particle counts n (host, nsys). */
+/* Bytes of device workspace for particle counts n (host, nsys); the smallest
+ * workspace accepted for them, in which FP32 systems take the form that
+ * fmm_workspace_minimum describes. */
 int fmm_batch_workspace_size(fmm_batch_t batch, const int64_t *n, size_t *bytes);
+int fmm_batch_workspace_minimum(fmm_batch_t batch, const int64_t *n, size_t *bytes);
 
 /*
  * fmm_batch_eval — evaluates every system.  Particles of system i are rows
@@ -382,8 +400,9 @@ int fmm_batch_set_schedule(fmm_batch_t batch, int schedule);
  * memory at start-up).
  *   Scratch: a static device array of FMM_STATIC_WORKSPACE_BYTES (32 MiB),
  *   which every GPU that loads the library holds until the process exits.
- *   Limit: (plan, n) whose fmm_workspace_size exceeds it are rejected with
- *   FMM_ERR_WORKSPACE before any device work.
+ *   Limit: (plan, n) whose fmm_workspace_minimum exceeds it are rejected with
+ *   FMM_ERR_WORKSPACE before any device work; those whose fmm_workspace_size
+ *   exceeds it take the form that fmm_workspace_minimum describes.
  *   Allocation: none (no cudaMalloc/cudaFree, no allocating library call);
  *   the plan, created beforehand, owns its tables.
  *   Device: the current device must be the one the plan was created on, else

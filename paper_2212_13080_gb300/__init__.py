@@ -35,6 +35,24 @@ def _stream(stream):
     return ctypes.c_void_p(s.cuda_stream)
 
 
+def _keep_workspace(plan, need, least):
+    """plan._ws: a kept device allocation of at least `need` bytes (and 256 to
+    align it), or, where memory does not hold that, of at least `least`, with which
+    plans of the default precision take a slower form.  A size that did not fit is
+    not tried again for calls that need no more."""
+    have = plan._ws.numel() - 256 if plan._ws is not None else -1
+    if have >= need or (have >= least and plan._ws_for >= need):
+        return
+    try:
+        plan._ws = torch.empty(need + 256, dtype=torch.uint8, device=plan.device)
+    except torch.cuda.OutOfMemoryError:
+        if least >= need:
+            raise
+        if have < least:
+            plan._ws = torch.empty(least + 256, dtype=torch.uint8, device=plan.device)
+    plan._ws_for = need
+
+
 class FMM:
     """One plan of the method: box (x0, y0, z0, L), octree depth, order p.
 
@@ -83,7 +101,7 @@ class FMM:
         with torch.cuda.device(self.device):
             self._h = B.fmm_plan_create(self.box, self.depth, self.p, self.periodic, o, self.max_n)
         self.out_dtype = torch.float64 if precision == "fp64" else torch.float32
-        self._ws = None
+        self._ws, self._ws_for = None, 0
         self._last = None
 
     def close(self):
@@ -102,9 +120,8 @@ class FMM:
 
     def workspace(self, n):
         """A device workspace for n particles (kept by the plan and reused)."""
-        need = self.workspace_size(n)
-        if self._ws is None or self._ws.numel() < need:
-            self._ws = torch.empty(need + 256, dtype=torch.uint8, device=self.device)
+        need, least = self.workspace_size(n), B.fmm_workspace_minimum(self._h, n)
+        _keep_workspace(self, need, least)
         return self._ws
 
     @staticmethod
@@ -273,7 +290,7 @@ class FMMBatch:
             self._h = B.fmm_batch_create(np.asarray(boxes, np.float64).reshape(-1, 4),
                                          np.asarray(depths), p, periodic, o,
                                          np.asarray(max_n, np.int64))
-        self._ws = None
+        self._ws, self._ws_for = None, 0
 
     def close(self):
         if getattr(self, "_h", None):
@@ -292,8 +309,7 @@ class FMMBatch:
         offs = np.asarray(offsets, np.int64)
         counts = np.diff(offs)
         need = B.fmm_batch_workspace_size(self._h, counts)
-        if self._ws is None or self._ws.numel() < need + 256:
-            self._ws = torch.empty(need + 256, dtype=torch.uint8, device=self.device)
+        _keep_workspace(self, need, B.fmm_batch_workspace_minimum(self._h, counts))
         ws = FMM._aligned(self._ws)
         n = int(offs[-1])
         o = out if out is not None else {}

@@ -49,10 +49,10 @@ FMM_INJECT_TC_STALL = 1
 
 # every symbol include/fmm_gb300.h declares
 EXPORTED = ["fmm_opts_default", "fmm_plan_create", "fmm_plan_destroy", "fmm_workspace_size",
-            "fmm_eval", "fmm_backward", "fmm_status", "fmm_debug_dump", "fmm_debug_size",
+            "fmm_workspace_minimum", "fmm_eval", "fmm_backward", "fmm_status", "fmm_debug_dump", "fmm_debug_size",
             "fmm_set_timing", "fmm_get_stats", "fmm_strerror", "fmm_version",
             "fmm_eval_static", "fmm_batch_create", "fmm_batch_destroy",
-            "fmm_batch_workspace_size", "fmm_batch_eval", "fmm_batch_get_stats",
+            "fmm_batch_workspace_size", "fmm_batch_workspace_minimum", "fmm_batch_eval", "fmm_batch_get_stats",
             "fmm_batch_set_schedule", "fmm_debug_inject"]
 
 FMM_STATIC_WORKSPACE_BYTES = 32 << 20
@@ -102,6 +102,7 @@ def lib():
         L.fmm_plan_destroy.argtypes = [P]
         L.fmm_plan_destroy.restype = None
         L.fmm_workspace_size.argtypes = [P, i64, ctypes.POINTER(sz)]
+        L.fmm_workspace_minimum.argtypes = [P, i64, ctypes.POINTER(sz)]
         L.fmm_eval.argtypes = [P, i64, P, P, P, P, P, P, sz, P]
         L.fmm_backward.argtypes = [P, i64, P, P, P, P, P, P, sz, P]
         L.fmm_status.argtypes = [P, P, P]
@@ -119,6 +120,7 @@ def lib():
         L.fmm_batch_destroy.argtypes = [P]
         L.fmm_batch_destroy.restype = None
         L.fmm_batch_workspace_size.argtypes = [P, P, ctypes.POINTER(sz)]
+        L.fmm_batch_workspace_minimum.argtypes = [P, P, ctypes.POINTER(sz)]
         L.fmm_batch_eval.argtypes = [P, P, P, P, P, P, P, P, sz, P]
         L.fmm_batch_get_stats.argtypes = [P, ctypes.POINTER(fmm_batch_stats_t)]
         L.fmm_batch_set_schedule.argtypes = [P, i32]
@@ -162,6 +164,12 @@ def fmm_plan_destroy(h):
 def fmm_workspace_size(h, n):
     s = ctypes.c_size_t()
     _check(lib().fmm_workspace_size(h, int(n), ctypes.byref(s)), "fmm_workspace_size")
+    return s.value
+
+
+def fmm_workspace_minimum(h, n):
+    s = ctypes.c_size_t()
+    _check(lib().fmm_workspace_minimum(h, int(n), ctypes.byref(s)), "fmm_workspace_minimum")
     return s.value
 
 
@@ -229,6 +237,15 @@ def fmm_batch_workspace_size(h, n):
     s = ctypes.c_size_t()
     _check(lib().fmm_batch_workspace_size(h, a.ctypes.data_as(ctypes.c_void_p), ctypes.byref(s)),
            "fmm_batch_workspace_size")
+    return s.value
+
+
+def fmm_batch_workspace_minimum(h, n):
+    import numpy as np
+    a = np.ascontiguousarray(n, dtype=np.int64)
+    s = ctypes.c_size_t()
+    _check(lib().fmm_batch_workspace_minimum(h, a.ctypes.data_as(ctypes.c_void_p), ctypes.byref(s)),
+           "fmm_batch_workspace_minimum")
     return s.value
 
 

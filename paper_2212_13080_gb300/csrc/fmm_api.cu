@@ -736,6 +736,11 @@ int fmm_workspace_size(fmm_plan_t P, int64_t n, size_t *bytes) {
     return FMM_OK;
 }
 
+int fmm_workspace_minimum(fmm_plan_t P, int64_t n, size_t *bytes) {
+    if (!P || !bytes) return FMM_ERR_ARG;
+    return plan_min_workspace(P, n, bytes);
+}
+
 int fmm_eval(fmm_plan_t P, int64_t n, const float *pos, const float *q, void *potential,
              double *energy, void *forces, void *workspace, size_t workspace_bytes, void *stream) {
     if (!P || n < 0 || n > P->max_n) return FMM_ERR_ARG;
@@ -1089,7 +1094,7 @@ struct MergedLaunch {
 // different kernels or launch shapes.  The table (functors, prefixes) is
 // uploaded to the device before the call returns.
 int record_merged(fmm_batch_t B, const std::vector<int64_t> &n, const std::vector<int64_t> &pofs,
-                  const std::vector<size_t> &wofs, const float *pos, const float *q, void *potential,
+                  const std::vector<size_t> &wofs, bool least, const float *pos, const float *q, void *potential,
                   double *energy, void *forces, char *ws, std::vector<MergedLaunch> &out) {
     const int ns = B->nsys;
     if (B->opts.precision == FMM_PREC_FP64) return FMM_ERR_UNSUPPORTED;
@@ -1099,7 +1104,7 @@ int record_merged(fmm_batch_t B, const std::vector<int64_t> &n, const std::vecto
     // tensor-core plans: the levels with fewer than 8 coarse cells per axis
     // (l <= 3) of every system run as cross-system tiles, full rows; each
     // system's own contraction takes levels 4 and up
-    const int tc_lmin = M0->tc ? (B->periodic ? 1 : 2) : 0;
+    const int tc_lmin = M0->tc && !least ? (B->periodic ? 1 : 2) : 0;
     const int x_lmax = 3;
     std::vector<std::vector<LaunchRec>> recs(ns);
     const Lane &L = B->lane[0];
@@ -1117,7 +1122,7 @@ int record_merged(fmm_batch_t B, const std::vector<int64_t> &n, const std::vecto
         char *frc = forces ? (char *)forces + 3 * o * 4 : nullptr;
         double *en = energy ? energy + i : nullptr;
         int rc = eval_impl<float>(P, n[i], pos + 3 * o, q + o, (float *)pot, en, (float *)frc, ws + wofs[i],
-                                  SIZE_MAX, S, tr);
+                                  least ? 0 : SIZE_MAX, S, tr);
         if (rc) return rc;
     }
     if (tc_lmin) {
@@ -1315,7 +1320,7 @@ int capture_merged(fmm_batch_t B, const std::vector<MergedLaunch> &ml, int sched
 }
 
 int capture_batch(fmm_batch_t B, int lanes, const std::vector<int64_t> &n,
-                  const std::vector<int64_t> &pofs, const std::vector<size_t> &wofs, const float *pos,
+                  const std::vector<int64_t> &pofs, const std::vector<size_t> &wofs, bool least, const float *pos,
                   const float *q, void *potential, double *energy, void *forces, char *ws,
                   cudaStream_t st, cudaGraphExec_t *out, int *launches) {
     const size_t rs = B->opts.precision == FMM_PREC_FP64 ? 8 : 4;
@@ -1337,10 +1342,10 @@ int capture_batch(fmm_batch_t B, int lanes, const std::vector<int64_t> &n,
         double *en = energy ? energy + i : nullptr;
         if (P->fp64)
             rc = eval_impl<double>(P, n[i], pos + 3 * o, q + o, (double *)pot, en, (double *)frc,
-                                   ws + wofs[i], SIZE_MAX, S, tr);
+                                   ws + wofs[i], least ? 0 : SIZE_MAX, S, tr);
         else
             rc = eval_impl<float>(P, n[i], pos + 3 * o, q + o, (float *)pot, en, (float *)frc,
-                                  ws + wofs[i], SIZE_MAX, S, tr);
+                                  ws + wofs[i], least ? 0 : SIZE_MAX, S, tr);
         total += tr.launches;
     }
     for (int k = 0; k < lanes; k++) {
@@ -1488,13 +1493,16 @@ void fmm_batch_destroy(fmm_batch_t B) {
     delete B;
 }
 
-static int batch_layout(fmm_batch_t B, const int64_t *n, std::vector<size_t> &wofs, size_t *total) {
+// least: the smallest workspaces that the systems accept (FP32 plans without the
+// contraction's operand copy)
+static int batch_layout(fmm_batch_t B, const int64_t *n, bool least, std::vector<size_t> &wofs, size_t *total) {
     wofs.resize(B->nsys);
     size_t o = 0;
     for (int i = 0; i < B->nsys; i++) {
         if (n[i] < 0 || n[i] > B->max_n[i]) return FMM_ERR_ARG;
         wofs[i] = o;
-        o += align256(make_layout(B->sys[i], n[i]).total);
+        const WsLayout W = make_layout(B->sys[i], n[i]);
+        o += align256(least ? W.total_simt : W.total);
     }
     *total = o;
     return FMM_OK;
@@ -1503,7 +1511,13 @@ static int batch_layout(fmm_batch_t B, const int64_t *n, std::vector<size_t> &wo
 int fmm_batch_workspace_size(fmm_batch_t B, const int64_t *n, size_t *bytes) {
     if (!B || !n || !bytes) return FMM_ERR_ARG;
     std::vector<size_t> w;
-    return batch_layout(B, n, w, bytes);
+    return batch_layout(B, n, false, w, bytes);
+}
+
+int fmm_batch_workspace_minimum(fmm_batch_t B, const int64_t *n, size_t *bytes) {
+    if (!B || !n || !bytes) return FMM_ERR_ARG;
+    std::vector<size_t> w;
+    return batch_layout(B, n, true, w, bytes);
 }
 
 int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, const float *q,
@@ -1526,9 +1540,12 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
     if (forces) forces = (char *)forces + 3 * row0 * rs;
     std::vector<size_t> wofs;
     size_t total = 0;
-    int rc = batch_layout(B, n.data(), wofs, &total);
+    int rc = batch_layout(B, n.data(), false, wofs, &total);
     if (rc) return rc;
-    if (workspace_bytes < total) return FMM_ERR_WORKSPACE;
+    const bool least = workspace_bytes < total;
+    if (least && !(rc = batch_layout(B, n.data(), true, wofs, &total)) && workspace_bytes < total)
+        rc = FMM_ERR_WORKSPACE;
+    if (rc) return rc;
     cudaStream_t caller = (cudaStream_t)stream;
     // capture and launch on the batch's own stream (the caller's may be the
     // legacy default stream, which cannot be captured), ordered after the
@@ -1537,13 +1554,13 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
     cudaEventRecord(B->in_ev, caller);
     cudaStreamWaitEvent(st, B->in_ev, 0);
     char *ws = (char *)workspace;
-    // what a captured graph is valid for: the workspace, the counts and which
+    // what a captured graph is valid for: the workspace and its layout, the counts and which
     // outputs are wanted; a merged graph reads the first rows' addresses from a table
     // (recording, capturing and instantiating again for every new set of arrays
     // took 4.5 ms a call with 512 systems), the stream lanes hold them
     IoArrays io = {{(void *)pos, (void *)q, potential, forces, energy}};
     const bool by_table = B->merged && B->opts.precision != FMM_PREC_FP64;
-    std::vector<int64_t> key = {(int64_t)by_table, (int64_t)(uintptr_t)workspace};
+    std::vector<int64_t> key = {(int64_t)by_table, (int64_t)least, (int64_t)(uintptr_t)workspace};
     for (int k = 0; k < IO_N; k++) key.push_back(by_table ? io.p[k] != nullptr : (int64_t)(uintptr_t)io.p[k]);
     key.insert(key.end(), n.begin(), n.end());
     cudaGetLastError();
@@ -1563,7 +1580,7 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
             B->gexec = nullptr;
         }
         // the merged form where the systems' sequences merge, else stream lanes
-        rc = B->merged ? record_merged(B, n, pofs, wofs, pos, q, potential, energy, forces, ws, ml)
+        rc = B->merged ? record_merged(B, n, pofs, wofs, least, pos, q, potential, energy, forces, ws, ml)
                        : FMM_ERR_UNSUPPORTED;
         if (rc != FMM_OK && rc != FMM_ERR_UNSUPPORTED) return rc;
         B->merged = rc == FMM_OK;
@@ -1620,7 +1637,7 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
                 const int l = kLaneChoices[c] < B->nsys ? kLaneChoices[c] : B->nsys;
                 cudaGraphExec_t ex = nullptr;
                 int launches = 0;
-                rc = capture_batch(B, l, n, pofs, wofs, pos, q, potential, energy, forces, ws, st, &ex,
+                rc = capture_batch(B, l, n, pofs, wofs, least, pos, q, potential, energy, forces, ws, st, &ex,
                                    &launches);
                 if (rc) break;
                 cudaGraphLaunch(ex, st);  // warm-up
@@ -1643,7 +1660,7 @@ int fmm_batch_eval(fmm_batch_t B, const int64_t *offsets, const float *pos, cons
             if (rc) return rc;
             B->lanes = best_l;
         }
-        rc = capture_batch(B, B->lanes, n, pofs, wofs, pos, q, potential, energy, forces, ws, st,
+        rc = capture_batch(B, B->lanes, n, pofs, wofs, least, pos, q, potential, energy, forces, ws, st,
                            &B->gexec, &B->launches);
         if (rc) return rc;
         B->glanes = B->lanes;
