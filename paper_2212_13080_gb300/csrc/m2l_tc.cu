@@ -28,8 +28,9 @@
 //     D = Alo Bhi + Ahi Blo + Ahi Bhi leaves out a product of up to 2^-22 of a term:
 //     less than FP32's 24 bits, in sums of at most 64 terms whose rounding outweighs it.
 //     Twice TF32's MMA rate and half its bytes.
-//   three parts (plain FP32 plans of p = 5, 6): all of FP32's bits, six products, and
-//     the leading products' sum is exact (KSplit).  The tensor cores' FP32 additions do
+//   three parts (plain FP32 plans of p = 5, 6): all of FP32's bits of values down to
+//     2^-9 of their cell's largest (smaller ones to 2^-32 of it), six products, and the
+//     leading products' sum is exact (KSplit).  The tensor cores' FP32 additions do
 //     not round to nearest, and two parts summed that way over 125 and 216 terms were
 //     up to 7% further from the 64-bit results than FP32 multiply-adds where the terms
 //     cancel.  Contraction of 1M clustered charges at p = 6: 7.3 ms with two parts, 10.8
@@ -415,6 +416,8 @@ __device__ __forceinline__ float2 kahan_error(float2 &run, float2 y) {
 }
 __device__ __forceinline__ float2 comp_value(float2 c) { return c; }
 __device__ __forceinline__ void kahan_add(float2 &run, float2 &comp, float2 y) { comp = kahan_error(run, y); }
+__device__ __forceinline__ void comp_keep(float2 &comp, float2 y) { comp = y; }
+__device__ __forceinline__ void comp_keep(uint32_t &, float2) {}
 // N = 224, where 112 sums and as many floats do not fit a thread's registers: the
 // error's leading eight bits (two bfloat16), so that a sum is carried with 24 + 8
 // bits; what is left out is below 2^-33 of a partial sum each step
@@ -624,7 +627,8 @@ struct KM2LTcg {
                         if constexpr (Sh::COMP) {
                             d = __ffma2_rn(d, inv2, comp_value(comp[x]));
                             if (h == Sh::ACC - 1) d = __ffma2_rn(m, Q2, d);
-                            kahan_add(run[x], comp[x], d);
+                            if (h < Sh::ACC - 1 && N != 224) comp_keep(comp[x], d);  // joins the sum with the next term
+                            else kahan_add(run[x], comp[x], d);
                         } else {
                             run[x] = __fadd2_rn(run[x], __ffma2_rn(m, Q2, Sh::SCALED ? __fmul2_rn(d, inv2) : d));
                         }
@@ -659,17 +663,17 @@ struct KM2LTcg {
                         }
                     } else {
 #pragma unroll
-                        for (int c = 0; c < Sh::COLS / 16; c++) {
-                            uint32_t h[16], w[16];
+                        for (int c = 0; c < Sh::COLS / 8; c++) {
+                            uint32_t h[8], w[8];
 #pragma unroll
-                            for (int e = 0; e < 16; e++) h[e] = w[e] = 0u;
+                            for (int e = 0; e < 8; e++) h[e] = w[e] = 0u;
                             if (!first) {
-                                tc::tmem_ld16(ttot + c * 16, h);
-                                tc::tmem_ld16(ttot + N + c * 16, w);
+                                tc::tmem_ld8(ttot + c * 8, h);
+                                tc::tmem_ld8(ttot + N + c * 8, w);
                             }
 #pragma unroll
-                            for (int e = 0; e < 16; e++) {
-                                float &t = e & 1 ? run[c * 8 + e / 2].y : run[c * 8 + e / 2].x;
+                            for (int e = 0; e < 8; e++) {
+                                float &t = e & 1 ? run[c * 4 + e / 2].y : run[c * 4 + e / 2].x;
                                 float hf = __uint_as_float(h[e]), wf = __uint_as_float(w[e]);
                                 part_add(hf, wf, t, last);
                                 if (last) t = hf;
@@ -677,8 +681,8 @@ struct KM2LTcg {
                                 w[e] = __float_as_uint(wf);
                             }
                             if (!last) {
-                                tc::tmem_st16(ttot + c * 16, h);
-                                tc::tmem_st16(ttot + N + c * 16, w);
+                                tc::tmem_st8(ttot + c * 8, h);
+                                tc::tmem_st8(ttot + N + c * 8, w);
                             }
                         }
                         tc::tmem_wait_st();
@@ -984,7 +988,8 @@ __global__ void __launch_bounds__(KTcReduce::BS) k_tc_reduce(const __grid_consta
 // factor 1/(s TC_KSCALE) where they are added up, all exact powers of two.
 // Three parts (P3): x s = x0 + x1 + x2, x0 the multiple of 2^7 next to x s (an
 // integer of at most 8 bits, times 2^7), x1 and x2 the remainder's two halves: all of
-// an FP32 value's bits down to 2^-25 against a largest of 2^14 and more.  The leading
+// an FP32 value's bits where it is at least 2^6, 2^-9 of the cell's largest; a smaller
+// one is off by at most 2^-23 of itself, 2^-32 of the largest.  The leading
 // parts' products are integers below 2^16 of one unit (2^7 times the kernel row's),
 // so that their sum over up to 224 values stays below 2^24 units: whatever the order
 // and the rounding of the tensor cores' additions, it is exact.
