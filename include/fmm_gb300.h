@@ -59,10 +59,11 @@ extern "C" {
 
 /* ---- precision of the far-field contraction (and of everything else) ----- */
 #define FMM_PREC_FP32 0   /* FP32 everywhere; bilinear forms of orders 3..6 on the tensor cores,
-                             every operand in half-precision parts: of orders 5 and 6 three,
-                             all of FP32's bits with exact leading products; of orders 3 and
-                             4 two, an operand to 2^-23 and a product to 2^-22 of itself; a
-                             compensated FP32 sum over the interaction list.  Measured errors
+                             every operand in half-precision parts: of orders 5 and 6 three
+                             (FP32's bits, or 2^-32 of the cell's largest value, and exact
+                             sums of the leading products); of orders 3 and 4 two (an operand
+                             to 2^-23 of itself, a product to 2^-22); a compensated FP32 sum
+                             over the interaction list.  Measured errors
                              are no larger than with FP32 multiply-adds, which the other
                              orders take */
 #define FMM_PREC_FP64 1   /* FP64 everywhere; outputs are float64 */
@@ -281,7 +282,8 @@ int fmm_debug_size(fmm_plan_t plan, int what, const void *workspace, size_t *byt
  * MMAs, frees its tensor memory and returns, and the call returns
  * FMM_ERR_TIMEOUT.  No fault, trap or unbounded wait: the context stays usable.
  * The hook disarms itself after one evaluation; FMM_INJECT_NONE disarms it.
- * Plans without tensor-core contraction (FP32, FP64) return FMM_ERR_UNSUPPORTED.
+ * Plans of the reduced precisions only: FP32 and FP64 plans return
+ * FMM_ERR_UNSUPPORTED.
  * The wait site: fmm_debug_dump(FMM_DUMP_WAIT) = int[4] (site: 1 producer slot,
  * 2 MMA region, 3 MMA operands, 4 epilogue region, 0 none; block; level;
  * iteration).
