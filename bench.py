@@ -8,8 +8,8 @@ finest cells, 61% of them empty), p = 6 (216 grid charges per cell).
 Default precision "tf32x3": every stage in FP32, the far-field contraction of
 every level on the tcgen05 tensor cores in three passes over operands split in two
 halves (its parity with the FP64 oracle meets the FP32 tolerance).  The line
-also reports the plain FP32 form (the same operands, the sum over the offsets
-compensated), the force-kernel form, the shift-free forms, and
+also reports the plain FP32 form (operands in three halves at this order, the sum
+over the offsets compensated), the force-kernel form, the shift-free forms, and
 shorter lines for BF16x3 and for the uniform (1,048,576 particles, continuous
 form, depth 5, p 4) and water-like (2,097,150 particles, periodic continuous
 form, depth 6, p 5) workloads.
@@ -472,8 +472,9 @@ def m2l_work(start, depth, periodic, p, precision):
     whose target and source both hold charges (the method's own work: a functional
     is read only where there are charges, an empty source adds nothing), and the
     tensor-core work the contraction executes (128-row tiles of the occupied
-    targets, 189 offsets each, p^3 padded to the MMA shape, 3 passes for the
-    split forms)."""
+    targets, 189 offsets each, p^3 padded to the MMA shape; one product for the
+    1-pass form, three for two-part operands, six for the three parts of plain FP32
+    at p = 5 and 6)."""
     import numpy as np
     occ = cell_occupancy(start, depth)
     dense = both = tiles = 0
@@ -501,10 +502,10 @@ def m2l_work(start, depth, periodic, p, precision):
                             dense += int(np.prod([H - abs(v) for v in d]))
     p3 = p ** 3
     n_pad = k_pad = (p3 + 31) // 32 * 32
-    passes = 1 if precision == "tf32x1" else 3
+    passes = 1 if precision == "tf32x1" else 6 if precision == "fp32" and p >= 5 else 3
     return {"dense_pairs": dense, "occupied_pairs": both, "tiles": tiles,
             "algorithmic_flops": 2.0 * p3 * p3 * both, "dense_flops": 2.0 * p3 * p3 * dense,
-            "executed_flops": 2.0 * tiles * 128 * 189 * n_pad * k_pad * passes}
+            "executed_flops": 2.0 * tiles * 128 * 189 * n_pad * k_pad * passes, "passes": passes}
 
 
 def tc_peak(long_step):
@@ -630,7 +631,7 @@ def rooflines(run, t_step, stage_ms, stage_iso):
                       "executed_tflops": mw["executed_flops"] / (m_ms * 1e-3) / 1e12,
                       "executed_frac": mw["executed_flops"] / (m_ms * 1e-3) / 1e12 / peak,
                       "executed": "%d tiles x 128 rows x 189 offsets, p^3 padded, %d passes"
-                                  % (mw["tiles"], 1 if run.precision == "tf32x1" else 3),
+                                  % (mw["tiles"], mw["passes"]),
                       "achieved_isolated": mw["algorithmic_flops"] / (m_iso * 1e-3) / 1e12}
     else:
         a = mw["algorithmic_flops"] / (m_ms * 1e-3) / 1e12

@@ -1159,7 +1159,15 @@ __global__ void __launch_bounds__(KNear<FORCES, CK, POW>::BS, KNear<FORCES, CK, 
 // 16 particles a cell (water2m, 8 a cell: near field 2.04 -> 1.13 ms; plummer8m,
 // 4 a cell: 20.3 -> 18.0 ms).  Elsewhere the mutual form takes every pair: with
 // 32 a cell (uniform1m) the split took 0.76 against 0.62 ms, with 8 a cell in
-// 16^3 cells 0.088 against 0.054 ms.
+// 16^3 cells 0.088 against 0.054 ms.  Near field of uniform charges, mutual / split:
+//   64^3 cells, 1, 4, 8, 12 a cell  0.96 / 0.46, 1.66 / 0.64, 1.93 / 0.89, 2.25 / 1.33
+//   64^3 cells, 16, 20, 24 a cell   2.48 / 2.00, 3.15 / 2.98, 3.56 / 3.89
+//   32^3 cells, 1, 4, 8, 16 a cell  0.13 / 0.07, 0.21 / 0.10, 0.23 / 0.13, 0.31 / 0.27
+// so the bars are on the safe side: the split form would still win up to 20 a cell
+// and in 32^3 cells, by 0.1 ms there (clustered charges there: equal, 5.06 / 5.05).
+// NF_LIGHT itself: with 16 in place of 24 the split took 1.58 against 1.33 ms at 12 a
+// cell and 1.29 against 1.14 on water2m, with 32 the same as with 24 (plummer1m 2.95
+// against 2.83).
 template <typename real>
 static int nf_light(const WsLayout &W, int64_t n) {
     return sizeof(real) == 4 && W.ncell >= 262144 && n < 16 * W.ncell ? NF_LIGHT : 1;
