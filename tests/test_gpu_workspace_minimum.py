@@ -27,7 +27,7 @@ def test_sizes_by_precision():
         plan.close()
 
 
-@pytest.mark.parametrize("p", [4, 6])
+@pytest.mark.parametrize("p", [3, 4, 5, 6])
 def test_batch_in_the_smallest_workspace(p):
     pos, q, offs, boxes, counts = inputs.batch_systems(4, 45, lo=1024, hi=9000)
     depths = np.array([3, 4, 5, 2])
